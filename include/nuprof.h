@@ -197,7 +197,7 @@ typedef struct nu_opts {
 } nu_opts;
 
 #define NU_MAX_STEPS 3000  /* the per-step coefficient table (80 B per step in FP32,
-                              160 B in FP64 and in the packed path) is staged in
+                              160 B in FP64) is staged in
                               shared memory when it fits in 227 KB and read
                               through the L1 cache otherwise                     */
 

@@ -414,7 +414,7 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
     h->n_radii = n_radii;
     h->tiles_per_seg = tps;
     h->n_tiles = info.n_tiles;
-    h->smem = coef_smem_bytes(o.precision, o.n_steps, o.tpt);
+    h->smem = coef_smem_bytes(o.precision, o.n_steps);
 
     // ---- host tables (FP64) ----
     const int nq = p_grid->n_q, nmu = p_grid->n_mu, N = o.n_steps;
@@ -453,7 +453,6 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
     const size_t o_prob = carve(sizeof(DevProblem));
     const size_t o_pref = carve(2 * sizeof(int));
     const size_t o_coef = carve((size_t)N * C_COUNT * sz);
-    const size_t o_coef2 = fp64 ? 0 : carve((size_t)N * C_COUNT * 2 * sizeof(float));
     const size_t o_x0 = carve((size_t)n_radii * sz);
     const size_t o_v0 = carve((size_t)nq * sz);
     const size_t o_mu = carve((size_t)nmu * sz);
@@ -482,7 +481,6 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
     DevProblem& P = h->hdp;
     std::memset(&P, 0, sizeof(P));
     P.coef = base + o_coef;
-    P.coef2 = fp64 ? nullptr : base + o_coef2;
     P.x0 = base + o_x0;
     P.v0 = base + o_v0;
     P.mu = base + o_mu;
@@ -535,8 +533,7 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
             put<double>(stage, o_mu, mu.data(), nmu);
             put<double>(stage, o_smu, smu.data(), nmu);
         } else {
-            fp32_table(coef.data(), N, d, reinterpret_cast<float*>(stage + o_coef),
-                       reinterpret_cast<float*>(stage + o_coef2));
+            fp32_table(coef.data(), N, d, reinterpret_cast<float*>(stage + o_coef));
             put<float>(stage, o_x0, x0.data(), n_radii);
             put<float>(stage, o_v0, v0.data(), nq);
             put<float>(stage, o_mu, mu.data(), nmu);
@@ -725,7 +722,7 @@ int nu_batch_create(nu_profile* const* hs, int n, const nu_opts* opts, nu_batch*
     }
     if (b->tpt == kTptPacked && b->precision != NU_MIXED) return NU_EINVAL;
     for (int i = 0; i < n; ++i) {
-        b->smem = std::max(b->smem, coef_smem_bytes(b->precision, hs[i]->opts.n_steps, b->tpt));
+        b->smem = std::max(b->smem, coef_smem_bytes(b->precision, hs[i]->opts.n_steps));
     }
     const int tile = b->block * traj_per_thread(b->tpt);
     std::vector<DevProblem> descs(n);

@@ -149,15 +149,14 @@ double relic_f(const nu_relic& relic, double q)
     return 1.0 / (1.0 + std::exp(q - relic.f_p[0]));
 }
 
-// FP32 copy of the coefficient table, and with dup != nullptr the packed copy
-// with every value stored twice.  The FP32 force tests the NFW edge on y, so
+// FP32 copy of the coefficient table.  The FP32 force tests the NFW edge on y, so
 // the C_Q slots, which hold the squared edge for the FP64 force, carry in the
 // FP32 tables the bound in y below which a lane takes the rational branch of
 // I(y): min(c, kRationalYMax, (1 - 1e-3) R S) with S the stage's
 // 1/((1+z) r_s).  The last term matters only while the NFW edge lies beyond R
 // (before the collapse onset); its factor keeps every lane below the bound
 // inside R whatever the rounding of y.
-void fp32_table(const double* tab, int n_steps, const Derived& d, float* out, float* dup)
+void fp32_table(const double* tab, int n_steps, const Derived& d, float* out)
 {
     const double c = d.r_s > 0.0 ? d.r200 / d.r_s : 0.0;
     const double ymax = std::min(c, kRationalYMax);
@@ -167,10 +166,7 @@ void fp32_table(const double* tab, int n_steps, const Derived& d, float* out, fl
             double v = t[k];
             if (k >= C_Q0 && k <= C_Q2)
                 v = std::min(ymax, (1.0 - 1e-3) * d.R * t[C_S0 + (k - C_Q0)]);
-            const float f = (float)v;
-            const size_t j = (size_t)n * C_COUNT + k;
-            if (out) out[j] = f;
-            if (dup) dup[2 * j] = dup[2 * j + 1] = f;
+            out[(size_t)n * C_COUNT + k] = (float)v;
         }
     }
 }
@@ -405,7 +401,6 @@ long long device_bytes(int precision, int n_steps, int n_radii, int n_q, int n_m
     b += align256(sizeof(DevProblem));
     b += align256(2 * sizeof(int));                             // tile prefix
     b += align256((size_t)n_steps * C_COUNT * sz);               // coefficient table
-    if (precision == NU_MIXED) b += align256((size_t)n_steps * C_COUNT * 2 * sizeof(float));
     b += align256((size_t)n_radii * sz);                         // x0
     b += align256((size_t)n_q * sz);                             // v0
     b += 2 * align256((size_t)n_mu * sz);                        // mu, sin psi

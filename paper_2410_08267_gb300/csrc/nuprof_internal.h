@@ -71,8 +71,8 @@ void coef_table_into(const nu_cosmo& cosmo, const nu_halo& halo, const Derived& 
                      double* table);   // [n_steps][C_COUNT]
 // Largest y of the FP32 force's rational approximation of I(y)/y^2.
 constexpr double kRationalYMax = 16.0;
-// FP32 (and packed FP32) copies of a coefficient table; see host_model.cpp.
-void fp32_table(const double* tab, int n_steps, const Derived& d, float* out, float* dup);
+// FP32 copy of a coefficient table; see host_model.cpp.
+void fp32_table(const double* tab, int n_steps, const Derived& d, float* out);
 void coef_table(const nu_cosmo& cosmo, const nu_halo& halo, const Derived& d, int n_steps,
                 std::vector<double>& table);
 void log_nodes_into(int n, double q_min, double q_max, double* q, double* wl, double* wl_coarse);
@@ -89,7 +89,6 @@ inline int relic_n_mass(const nu_relic& r) { return r.n_masses > 0 ? r.n_masses 
 // Device-visible description of one request (POD, lives in device memory).
 struct DevProblem {
     const void* coef;       // [n_steps][C_COUNT] float (mixed) or double (fp64)
-    const void* coef2;      // [n_steps][C_COUNT][2] float, every value twice (mixed; packed path)
     const void* x0;         // [n_radii] start radius, kpc
     const void* v0;         // [n_q] start speed, km/s
     const void* mu;         // [n_mu] cos psi
@@ -180,7 +179,7 @@ int max_ctas_per_sm(int precision, int tpt, int block, size_t smem_bytes, int* o
 // Smallest tile (block 64 x 1 trajectory): request buffers of tile sums are
 // sized for it, so a batch may run any tile shape over existing requests.
 constexpr int kMinTile = 64;
-size_t coef_smem_bytes(int precision, int n_steps, int tpt);
+size_t coef_smem_bytes(int precision, int n_steps);
 // Trajectories per thread of a tile shape: tpt 3 is two trajectories per
 // thread in packed FP32x2 arithmetic (mixed precision only).
 inline int traj_per_thread(int tpt) { return tpt == 3 ? 2 : tpt; }

@@ -91,7 +91,7 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
     nu_opts o;
     resolve_opts(opts, o);
     if (o.flags != 0 || o.timeout_ms < 0.0) return NU_EINVAL;
-    if (o.tpt == kTptPacked) return NU_ENOTSUP;   // the packed table is not staged here
+    if (o.tpt == kTptPacked) return NU_ENOTSUP;   // scalar shapes only
     if (relic && relic->n_masses > 0) return NU_ENOTSUP;   // one mass per call
     if (relic && relic->f_kind == NU_F_TABLE) return NU_ENOTSUP;   // closed-form f only
     int rc = validate(cosmo, halo, relic, radii, n_radii, p_grid, &o);
@@ -236,7 +236,7 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
         put_into<double>(st, o_mu, mu, nmu);
         put_into<double>(st, o_smu, smu, nmu);
     } else {
-        fp32_table(coef, N, d, reinterpret_cast<float*>(st + o_coef), nullptr);
+        fp32_table(coef, N, d, reinterpret_cast<float*>(st + o_coef));
         put_into<float>(st, o_x0, x0, n_radii);
         put_into<float>(st, o_v0, q, nq);
         put_into<float>(st, o_mu, mu, nmu);
@@ -249,7 +249,7 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
     put_into<double>(st, o_mass, mass, 3);
 
     int per_sm = 0, sms = 0;
-    const size_t smem = coef_smem_bytes(o.precision, N, o.tpt);
+    const size_t smem = coef_smem_bytes(o.precision, N);
     rc = max_ctas_per_sm(o.precision, o.tpt, o.block, smem, &per_sm);
     if (rc != NU_OK) return rc;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_id) != cudaSuccess ||

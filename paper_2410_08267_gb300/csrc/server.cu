@@ -406,7 +406,7 @@ void nu_server::run()
         size_t smem = 0;                          // the largest table staged this launch
         for (size_t i = 0; i < active.size(); ++i) {
             const Active& a = active[i];
-            smem = std::max(smem, coef_smem_bytes(o.precision, a.n_steps, tpt));
+            smem = std::max(smem, coef_smem_bytes(o.precision, a.n_steps));
             DevProblem d = profile_desc(a.h);
             const long long seg = (long long)d.n_q * d.n_mu;
             d.tile = tile;
@@ -439,7 +439,7 @@ void nu_server::run()
         // a resident launch stages tables up to the largest a request may have
         // (requests join it later), so that its shared memory fits any of them
         const bool res = o.resident != 0;
-        if (res) smem = std::max(smem, coef_smem_bytes(o.precision, NU_MAX_STEPS, tpt));
+        if (res) smem = std::max(smem, coef_smem_bytes(o.precision, NU_MAX_STEPS));
         if (rc == NU_OK) rc = max_ctas_per_sm(o.precision, tpt, o.block, smem, &per_sm, gtab);
         if (rc == NU_OK && (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
                             per_sm < 1))

@@ -387,8 +387,10 @@ __device__ __forceinline__ void rk4_step(T& x, T& y, T& vx, T& vy, const T* c,
 // Each component sees exactly the operations of the scalar path above, in the
 // same order, so the results are bitwise those of the two-trajectory scalar
 // kernel; only selects, comparisons and the special functions stay scalar.
-// The coefficients come from a table with every value stored twice ({c, c}),
-// so a 16-byte shared load yields two ready operand pairs.
+// The coefficients come from the same table as the scalar path's, each widened
+// to a pair in registers: a table with every value stored twice costs twice the
+// loads and more spills (precision sweep, four masses: 6.79 ms with the doubled
+// table and 38 B of spill stores, 6.41-6.50 ms with the plain one and 14 B).
 // ---------------------------------------------------------------------------
 struct f2 {
     unsigned long long v;
@@ -588,34 +590,34 @@ __device__ __forceinline__ void accel_m_pair_x2(f2 xa, f2 ya, f2 Sa, f2 Ya, f2 T
     mb = m_mixed_x2<NARROW>(gb, Tb, hc, need_log);
 }
 
-// One 16-byte entry of the duplicated table (two slots, each a {c, c} pair).
+// Four consecutive slots of a step's coefficients.
 template <bool GTAB>
-__device__ __forceinline__ ulonglong2 coef_pair(const uint4* src4, int q)
+__device__ __forceinline__ float4 coef4(const float4* c4, int q)
 {
-    const uint4 w = GTAB ? __ldg(&src4[q]) : src4[q];
-    return make_ulonglong2(((unsigned long long)w.y << 32) | w.x,
-                           ((unsigned long long)w.w << 32) | w.z);
+    return GTAB ? __ldg(&c4[q]) : c4[q];
 }
 
-// rk4_step for two trajectories at once.  src4 points at the step's 10 x 16
-// bytes of the duplicated table (slot j -> floats 2j, 2j+1); each entry is
-// loaded where it is first needed, which keeps the table out of registers.
+// rk4_step for two trajectories at once.  c4 points at the step's C_COUNT
+// coefficients; each group of four is loaded where it is first needed, which
+// keeps the table out of registers.
 // The four force evaluations run as two independent pairs (stages 1 and 2,
 // then 3 and 4); every value is formed by the same operations as in rk4_step.
 template <bool GTAB, bool NARROW>
-__device__ __forceinline__ void rk4_step_x2(f2& x, f2& y, f2& vx, f2& vy, const uint4* src4,
+__device__ __forceinline__ void rk4_step_x2(f2& x, f2& y, f2& vx, f2& vy, const float4* c4,
                                             const HaloX2& hc)
 {
-    const ulonglong2 q0 = coef_pair<GTAB>(src4, 0);
-    const f2 MA1{q0.x}, MA2{q0.y};
+    const float4 q0 = coef4<GTAB>(c4, 0);          // MA1 MA2 MA3 B1
+    const f2 MA1 = dup(q0.x), MA2 = dup(q0.y), MA3 = dup(q0.z), B1 = dup(q0.w);
     const f2 X2 = fma2(MA1, vx, x), Y2 = fma2(MA1, vy, y);
-    const ulonglong2 q5 = coef_pair<GTAB>(src4, 5), q6 = coef_pair<GTAB>(src4, 6);
-    const ulonglong2 q7 = coef_pair<GTAB>(src4, 7), q8 = coef_pair<GTAB>(src4, 8);
-    const f2 S0{q5.x}, S1{q5.y}, Yq0{q6.y}, Yq1{q7.x}, T0{q8.x}, T1{q8.y};
+    const float4 q2 = coef4<GTAB>(c4, 2);          // W1 W2 S0 S1
+    const float4 q3 = coef4<GTAB>(c4, 3);          // S2 Q0 Q1 Q2
+    const float4 q4 = coef4<GTAB>(c4, 4);          // T0 T1 T2 IREM
+    const f2 S0 = dup(q2.z), S1 = dup(q2.w), T0 = dup(q4.x), T1 = dup(q4.y);
+    const f2 Yq0 = dup(q3.y), Yq1 = dup(q3.z);
     f2 m1, m2;
     accel_m_pair_x2<NARROW>(x, y, S0, Yq0, T0, X2, Y2, S1, Yq1, T1, hc, m1, m2);
-    const ulonglong2 q1 = coef_pair<GTAB>(src4, 1), q2 = coef_pair<GTAB>(src4, 2);
-    const f2 MA3{q1.x}, B1{q1.y}, B2{q2.x};
+    const float4 q1 = coef4<GTAB>(c4, 1);          // B2 B3 B4 W0
+    const f2 B2 = dup(q1.x);
     const f2 p1 = mul2(B1, m1);
     const f2 VX2 = fma2(p1, x, vx), VY2 = fma2(p1, y, vy);
     const f2 p2 = mul2(B2, m2);
@@ -623,12 +625,10 @@ __device__ __forceinline__ void rk4_step_x2(f2& x, f2& y, f2& vx, f2& vy, const 
     const f2 X3 = fma2(MA2, VX2, x), Y3 = fma2(MA2, VY2, y);
     const f2 X4 = fma2(MA3, VX3, x), Y4 = fma2(MA3, VY3, y);
 
-    const ulonglong2 q9 = coef_pair<GTAB>(src4, 9);
-    const f2 S2{q6.x}, Yq2{q7.y}, T2{q9.x};
+    const f2 S2 = dup(q3.x), Yq2 = dup(q3.w), T2 = dup(q4.z);
     f2 m3, m4;
     accel_m_pair_x2<NARROW>(X3, Y3, S1, Yq1, T1, X4, Y4, S2, Yq2, T2, hc, m3, m4);
-    const ulonglong2 q3 = coef_pair<GTAB>(src4, 3), q4 = coef_pair<GTAB>(src4, 4);
-    const f2 B3{q2.y}, B4{q3.x}, W0{q3.y}, W1{q4.x}, W2{q4.y};
+    const f2 B3 = dup(q1.y), B4 = dup(q1.z), W0 = dup(q1.w), W1 = dup(q2.x), W2 = dup(q2.y);
     const f2 p3 = mul2(B3, m3);
     const f2 VX4 = fma2(p3, X3, vx), VY4 = fma2(p3, Y3, vy);
     const f2 p4 = mul2(B4, m4);
@@ -658,14 +658,14 @@ __device__ __forceinline__ void packed_steps(f2& X, f2& Y, f2& VX, f2& VY, const
             const f2 r2 = fma2(X, X, mul2(Y, Y));
             const f2 dot = fma2(X, VX, mul2(Y, VY));
             const f2 v2 = fma2(VX, VX, mul2(VY, VY));
-            const float irem = tab[(size_t)n * 2 * C_COUNT + 2 * C_IREM];
+            const float irem = tab[(size_t)n * C_COUNT + C_IREM];
             const bool fin0 = !act0 || escapes(f2lo(r2), f2lo(dot), f2lo(v2), h2.R2, R, irem);
             const bool fin1 = !act1 || escapes(f2hi(r2), f2hi(dot), f2hi(v2), h2.R2, R, irem);
             done |= fin0 && fin1;
             if (__all_sync(0xffffffffu, done)) break;
         }
         rk4_step_x2<GTAB, NARROW>(X, Y, VX, VY,
-                                  reinterpret_cast<const uint4*>(tab + (size_t)n * 2 * C_COUNT), h2);
+                                  reinterpret_cast<const float4*>(tab + (size_t)n * C_COUNT), h2);
     }
 }
 
@@ -781,11 +781,11 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
 
         // coefficient table: staged once per request into shared memory, or
         // (GTAB) read in place through the L1 cache with warp-uniform loads
-        const T* tab = GTAB ? reinterpret_cast<const T*>(PACKED ? P.coef2 : P.coef) : s_coef;
+        const T* tab = GTAB ? reinterpret_cast<const T*>(P.coef) : s_coef;
         if (!GTAB && lo != cur) {   // stage this request's table (uniform branch)
-            const float4* src = reinterpret_cast<const float4*>(PACKED ? P.coef2 : P.coef);
+            const float4* src = reinterpret_cast<const float4*>(P.coef);
             float4* dst = reinterpret_cast<float4*>(s_coef);
-            const int n16 = (int)((size_t)n_steps * C_COUNT * sizeof(T) * (PACKED ? 2 : 1) / 16);
+            const int n16 = (int)((size_t)n_steps * C_COUNT * sizeof(T) / 16);
             for (int i = threadIdx.x; i < n16; i += blockDim.x) dst[i] = __ldg(&src[i]);
             __syncthreads();
             cur = lo;
@@ -1041,11 +1041,9 @@ int launch_force_probe(int precision, const DevProblem* d_prob, int stage, const
     return NU_OK;
 }
 
-size_t coef_smem_bytes(int precision, int n_steps, int tpt)
+size_t coef_smem_bytes(int precision, int n_steps)
 {
-    // the packed path stages the duplicated table (two floats per coefficient)
-    const size_t per = precision == NU_FP64 ? sizeof(double) : sizeof(float) * (tpt == 3 ? 2 : 1);
-    return (size_t)n_steps * C_COUNT * per;
+    return (size_t)n_steps * C_COUNT * (precision == NU_FP64 ? sizeof(double) : sizeof(float));
 }
 
 template <typename T, int TPT, bool COUNT, bool PACKED = false, bool GTAB = false>
