@@ -433,6 +433,13 @@ __device__ __forceinline__ f2 add2(f2 a, f2 b)
     return r;
 }
 __device__ __forceinline__ f2 dup(float a) { return pk(a, a); }
+// largest of three, NaN if one of them is NaN
+__device__ __forceinline__ float max3_nan(float a, float b, float c)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
 
 struct HaloX2 {
     f2 invIc, neg_invR3;
@@ -491,22 +498,18 @@ __device__ __forceinline__ f2 nfw_I_log_x2(f2 y, f2 u)
 }
 
 // Geometry of one force evaluation for both lanes of a register pair:
-// guarded r^2, 1/r, rs = S/r and y = r^2 rs, and per lane whether it is on
-// the rational branch of the NFW part (y < Yq, which implies r < R).
+// guarded r^2, 1/r, rs = S/r and y = r^2 rs.
 struct Geo2 {
     f2 r2, rinv, rs, ys;
-    bool q0, q1;
 };
 
-__device__ __forceinline__ Geo2 geometry_x2(f2 x, f2 y, f2 S, f2 Yq)
+__device__ __forceinline__ Geo2 geometry_x2(f2 x, f2 y, f2 S)
 {
     Geo2 g;
     g.r2 = fma2(x, x, fma2(y, y, dup(kR2Guard)));
     g.rinv = pk(rsqrt_approx(f2lo(g.r2)), rsqrt_approx(f2hi(g.r2)));
     g.rs = mul2(g.rinv, S);
     g.ys = mul2(g.r2, g.rs);
-    g.q0 = f2lo(g.ys) < f2lo(Yq);
-    g.q1 = f2hi(g.ys) < f2hi(Yq);
     return g;
 }
 
@@ -534,9 +537,10 @@ __device__ __forceinline__ f2 m_out_x2(const Geo2& g, const HaloX2& hc)
     return pk(f2lo(g.r2) < hc.R2 ? f2lo(ms) : 0.0f, f2hi(g.r2) < hc.R2 ? f2hi(ms) : 0.0f);
 }
 // any mix of branches: each formula that some lane of the warp needs,
-// evaluated for both lanes and selected per lane
+// evaluated for both lanes and selected per lane (q0, q1: on the rational branch)
 template <bool NARROW>
-__device__ __forceinline__ f2 m_mixed_x2(const Geo2& g, f2 T, const HaloX2& hc, bool need_log)
+__device__ __forceinline__ f2 m_mixed_x2(const Geo2& g, f2 T, const HaloX2& hc, bool need_log,
+                                         bool q0, bool q1)
 {
     const f2 rinv2 = mul2(g.rinv, g.rinv);
     const f2 mq = m_rational_x2<NARROW>(g, T, hc);
@@ -544,8 +548,8 @@ __device__ __forceinline__ f2 m_mixed_x2(const Geo2& g, f2 T, const HaloX2& hc, 
     const f2 ms = m_shell_x2(g, rinv2, hc);
     const bool n0 = f2lo(g.ys) < hc.c, n1 = f2hi(g.ys) < hc.c;
     const bool in0 = f2lo(g.r2) < hc.R2, in1 = f2hi(g.r2) < hc.R2;
-    return pk(!in0 ? 0.0f : g.q0 ? f2lo(mq) : n0 ? f2lo(ml) : f2lo(ms),
-              !in1 ? 0.0f : g.q1 ? f2hi(mq) : n1 ? f2hi(ml) : f2hi(ms));
+    return pk(!in0 ? 0.0f : q0 ? f2lo(mq) : n0 ? f2lo(ml) : f2lo(ms),
+              !in1 ? 0.0f : q1 ? f2hi(mq) : n1 ? f2hi(ml) : f2hi(ms));
 }
 
 // m = Mhat/r^3 at two independent points (a, b) of both lanes: lane by lane
@@ -554,23 +558,25 @@ __device__ __forceinline__ f2 m_mixed_x2(const Geo2& g, f2 T, const HaloX2& hc, 
 // given the first two, so their force evaluations are independent and run
 // interleaved.  One warp vote covers all four lane-evaluations (the two
 // points of a pair almost always share their branch): every one on the
-// rational branch of the NFW part (the common case: it covers the whole NFW
-// part of halos with c <= 16), every one outside the NFW edge (shell or
-// beyond R), or any mix (each formula that a lane needs evaluated for all and
-// selected per lane).  All lanes of the warp execute this function together
-// (the integration loop is warp-uniform).
+// rational branch of the NFW part (y < Yq, which implies r < R), every one
+// outside the NFW edge (shell or beyond R), or any mix (each formula that a
+// lane needs evaluated for all and selected per lane).  Returns whether every
+// one was on the rational branch.  All lanes of the warp execute this function
+// together (the integration loop is warp-uniform).
 template <bool NARROW>
-__device__ __forceinline__ void accel_m_pair_x2(f2 xa, f2 ya, f2 Sa, f2 Ya, f2 Ta,
-                                                f2 xb, f2 yb, f2 Sb, f2 Yb, f2 Tb,
+__device__ __forceinline__ bool accel_m_pair_x2(f2 xa, f2 ya, f2 Sa, float Ya, f2 Ta,
+                                                f2 xb, f2 yb, f2 Sb, float Yb, f2 Tb,
                                                 const HaloX2& hc, f2& ma, f2& mb)
 {
-    const Geo2 ga = geometry_x2(xa, ya, Sa, Ya);
-    const Geo2 gb = geometry_x2(xb, yb, Sb, Yb);
+    const Geo2 ga = geometry_x2(xa, ya, Sa);
+    const Geo2 gb = geometry_x2(xb, yb, Sb);
+    const bool qa0 = f2lo(ga.ys) < Ya, qa1 = f2hi(ga.ys) < Ya;
+    const bool qb0 = f2lo(gb.ys) < Yb, qb1 = f2hi(gb.ys) < Yb;
     const unsigned full = 0xffffffffu;
-    if (__all_sync(full, ga.q0 && ga.q1 && gb.q0 && gb.q1)) {
+    if (__all_sync(full, qa0 && qa1 && qb0 && qb1)) {
         ma = m_rational_x2<NARROW>(ga, Ta, hc);
         mb = m_rational_x2<NARROW>(gb, Tb, hc);
-        return;
+        return true;
     }
     // lanes inside R and inside the NFW edge
     const bool na0 = f2lo(ga.r2) < hc.R2 && f2lo(ga.ys) < hc.c;
@@ -580,14 +586,15 @@ __device__ __forceinline__ void accel_m_pair_x2(f2 xa, f2 ya, f2 Sa, f2 Ya, f2 T
     if (__all_sync(full, !(na0 || na1 || nb0 || nb1))) {
         ma = m_out_x2(ga, hc);
         mb = m_out_x2(gb, hc);
-        return;
+        return false;
     }
     // a lane of the NFW part above the rational branch (only halos with c > 16)
-    const bool la = (na0 && !ga.q0) || (na1 && !ga.q1);
-    const bool lb = (nb0 && !gb.q0) || (nb1 && !gb.q1);
+    const bool la = (na0 && !qa0) || (na1 && !qa1);
+    const bool lb = (nb0 && !qb0) || (nb1 && !qb1);
     const bool need_log = __any_sync(full, la || lb);
-    ma = m_mixed_x2<NARROW>(ga, Ta, hc, need_log);
-    mb = m_mixed_x2<NARROW>(gb, Tb, hc, need_log);
+    ma = m_mixed_x2<NARROW>(ga, Ta, hc, need_log, qa0, qa1);
+    mb = m_mixed_x2<NARROW>(gb, Tb, hc, need_log, qb0, qb1);
+    return false;
 }
 
 // Four consecutive slots of a step's coefficients.
@@ -597,13 +604,22 @@ __device__ __forceinline__ float4 coef4(const float4* c4, int q)
     return GTAB ? __ldg(&c4[q]) : c4[q];
 }
 
-// rk4_step for two trajectories at once.  c4 points at the step's C_COUNT
-// coefficients; each group of four is loaded where it is first needed, which
-// keeps the table out of registers.
-// The four force evaluations run as two independent pairs (stages 1 and 2,
-// then 3 and 4); every value is formed by the same operations as in rk4_step.
-template <bool GTAB, bool NARROW>
-__device__ __forceinline__ void rk4_step_x2(f2& x, f2& y, f2& vx, f2& vy, const float4* c4,
+// One RK4 step of both trajectories: every value is formed by the operations of
+// rk4_step.  c4 points at the step's C_COUNT coefficients; each group of four is
+// loaded where it is first needed, which keeps the table out of registers.  The
+// four force evaluations run as two independent pairs (stages 1 and 2, then 3
+// and 4).
+//
+// RATIONAL takes every evaluation of the warp to be on the rational branch of
+// the NFW part, as it mostly is, and finds out with one vote near
+// the step's end; where that was not so it returns false and leaves the state
+// as it was.  The bounds of the four evaluations do not rise from stage to stage
+// (S falls with z), so the largest of the eight y against the last stage's
+// bound decides, and a NaN (r^2 out of range far beyond R) decides against it.
+// Otherwise each pair votes, and the return value says whether every evaluation
+// was on the rational branch.
+template <bool GTAB, bool NARROW, bool RATIONAL>
+__device__ __forceinline__ bool rk4_step_x2(f2& x, f2& y, f2& vx, f2& vy, const float4* c4,
                                             const HaloX2& hc)
 {
     const float4 q0 = coef4<GTAB>(c4, 0);          // MA1 MA2 MA3 B1
@@ -613,21 +629,38 @@ __device__ __forceinline__ void rk4_step_x2(f2& x, f2& y, f2& vx, f2& vy, const 
     const float4 q3 = coef4<GTAB>(c4, 3);          // S2 Q0 Q1 Q2
     const float4 q4 = coef4<GTAB>(c4, 4);          // T0 T1 T2 IREM
     const f2 S0 = dup(q2.z), S1 = dup(q2.w), T0 = dup(q4.x), T1 = dup(q4.y);
-    const f2 Yq0 = dup(q3.y), Yq1 = dup(q3.z);
     f2 m1, m2;
-    accel_m_pair_x2<NARROW>(x, y, S0, Yq0, T0, X2, Y2, S1, Yq1, T1, hc, m1, m2);
+    float y_max = 0.0f;
+    bool rational = true;
+    if constexpr (RATIONAL) {
+        const Geo2 g1 = geometry_x2(x, y, S0), g2 = geometry_x2(X2, Y2, S1);
+        m1 = m_rational_x2<NARROW>(g1, T0, hc);
+        m2 = m_rational_x2<NARROW>(g2, T1, hc);
+        y_max = max3_nan(f2lo(g1.ys), f2hi(g1.ys), f2lo(g2.ys));
+        y_max = max3_nan(y_max, f2hi(g2.ys), y_max);
+    } else {
+        rational = accel_m_pair_x2<NARROW>(x, y, S0, q3.y, T0, X2, Y2, S1, q3.z, T1, hc, m1, m2);
+    }
     const float4 q1 = coef4<GTAB>(c4, 1);          // B2 B3 B4 W0
-    const f2 B2 = dup(q1.x);
     const f2 p1 = mul2(B1, m1);
     const f2 VX2 = fma2(p1, x, vx), VY2 = fma2(p1, y, vy);
-    const f2 p2 = mul2(B2, m2);
+    const f2 p2 = mul2(dup(q1.x), m2);
     const f2 VX3 = fma2(p2, X2, vx), VY3 = fma2(p2, Y2, vy);
     const f2 X3 = fma2(MA2, VX2, x), Y3 = fma2(MA2, VY2, y);
     const f2 X4 = fma2(MA3, VX3, x), Y4 = fma2(MA3, VY3, y);
 
-    const f2 S2 = dup(q3.x), Yq2 = dup(q3.w), T2 = dup(q4.z);
+    const f2 S2 = dup(q3.x), T2 = dup(q4.z);
     f2 m3, m4;
-    accel_m_pair_x2<NARROW>(X3, Y3, S1, Yq1, T1, X4, Y4, S2, Yq2, T2, hc, m3, m4);
+    if constexpr (RATIONAL) {
+        const Geo2 g3 = geometry_x2(X3, Y3, S1), g4 = geometry_x2(X4, Y4, S2);
+        m3 = m_rational_x2<NARROW>(g3, T1, hc);
+        m4 = m_rational_x2<NARROW>(g4, T2, hc);
+        y_max = max3_nan(y_max, f2lo(g3.ys), f2hi(g3.ys));
+        y_max = max3_nan(y_max, f2lo(g4.ys), f2hi(g4.ys));
+        if (!__all_sync(0xffffffffu, y_max < q3.w)) return false;
+    } else {
+        rational &= accel_m_pair_x2<NARROW>(X3, Y3, S1, q3.z, T1, X4, Y4, S2, q3.w, T2, hc, m3, m4);
+    }
     const f2 B3 = dup(q1.y), B4 = dup(q1.z), W0 = dup(q1.w), W1 = dup(q2.x), W2 = dup(q2.y);
     const f2 p3 = mul2(B3, m3);
     const f2 VX4 = fma2(p3, X3, vx), VY4 = fma2(p3, Y3, vy);
@@ -643,29 +676,52 @@ __device__ __forceinline__ void rk4_step_x2(f2& x, f2& y, f2& vx, f2& vy, const 
     vy = fma2(p4, Y4, fma2(ty, third, vy));
     x = nx;
     y = ny;
+    return rational;
 }
 
-// The packed step loop of one tile for steps [s_begin, s_end): early-exit test
-// every kExitEvery steps, then an RK4 step of both lanes.  NARROW is fixed per
-// request (the rational fit its force uses), so the tile chooses the loop once.
+// The packed step loop of one tile for steps [s_begin, s_end).  NARROW is fixed
+// per request (the rational fit its force uses), so the tile chooses the loop
+// once.
+//
+// Bound by register operands and issue: a packed fused multiply-add with three
+// different register pairs takes 3 cycles of a scheduler, one with a constant
+// operand 2, and each other instruction one more (measured with independent
+// chains).  So the loop's instructions count: a warp whose lanes all stay on the
+// rational branch runs steps with one vote instead of two, four 3-input maxima
+// instead of eight compares, and no exit test (no lane of it is beyond R).
+// Where a step's vote fails, the step is done again with a vote per pair, and so
+// are the following ones until one is on the rational branch throughout: lanes
+// stay outside the NFW edge for many steps, so few steps are done twice.
+// Precision sweep of four masses, 128-thread CTAs: 6.41-6.50 -> 5.85-5.92 ms.
 template <bool GTAB, bool NARROW>
 __device__ __forceinline__ void packed_steps(f2& X, f2& Y, f2& VX, f2& VY, const float* tab,
                                              int s_begin, int s_end, bool act0, bool act1,
                                              bool done, const HaloX2& h2, float R)
 {
-    for (int n = s_begin; n < s_end; ++n) {
-        if (((n - s_begin) & (kExitEvery - 1)) == 0) {
-            const f2 r2 = fma2(X, X, mul2(Y, Y));
-            const f2 dot = fma2(X, VX, mul2(Y, VY));
-            const f2 v2 = fma2(VX, VX, mul2(VY, VY));
-            const float irem = tab[(size_t)n * C_COUNT + C_IREM];
-            const bool fin0 = !act0 || escapes(f2lo(r2), f2lo(dot), f2lo(v2), h2.R2, R, irem);
-            const bool fin1 = !act1 || escapes(f2hi(r2), f2hi(dot), f2hi(v2), h2.R2, R, irem);
-            done |= fin0 && fin1;
-            if (__all_sync(0xffffffffu, done)) break;
+    int n = s_begin;
+    for (;;) {
+        for (; n < s_end; ++n) {
+            const float4* c4 = reinterpret_cast<const float4*>(tab + (size_t)n * C_COUNT);
+            if (!rk4_step_x2<GTAB, NARROW, true>(X, Y, VX, VY, c4, h2)) break;
         }
-        rk4_step_x2<GTAB, NARROW>(X, Y, VX, VY,
-                                  reinterpret_cast<const float4*>(tab + (size_t)n * C_COUNT), h2);
+        if (n >= s_end) return;
+        bool rational;
+        int k = 0;
+        do {
+            if ((k++ & (kExitEvery - 1)) == 0) {
+                const f2 r2 = fma2(X, X, mul2(Y, Y));
+                const f2 dot = fma2(X, VX, mul2(Y, VY));
+                const f2 v2 = fma2(VX, VX, mul2(VY, VY));
+                const float irem = tab[(size_t)n * C_COUNT + C_IREM];
+                const bool fin0 = !act0 || escapes(f2lo(r2), f2lo(dot), f2lo(v2), h2.R2, R, irem);
+                const bool fin1 = !act1 || escapes(f2hi(r2), f2hi(dot), f2hi(v2), h2.R2, R, irem);
+                done |= fin0 && fin1;
+                if (__all_sync(0xffffffffu, done)) return;
+            }
+            const float4* c4 = reinterpret_cast<const float4*>(tab + (size_t)n * C_COUNT);
+            rational = rk4_step_x2<GTAB, NARROW, false>(X, Y, VX, VY, c4, h2);
+            ++n;
+        } while (n < s_end && !rational);
     }
 }
 

@@ -1,0 +1,58 @@
+"""Every step loop of the trajectory kernel against the counting launch, which
+integrates each trajectory alone with the general force (every branch tested
+per lane, no vote): the same n/nbar, error estimate and q_i, bit for bit."""
+import numpy as np
+import pytest
+
+from paper_2410_08267_gb300 import nuprof as nu
+from paper_2410_08267_gb300 import workloads as W
+
+from gpu_common import require_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def gpu():
+    return require_gpu()
+
+
+def _both(pb, block, tpt):
+    """Results of a normal run and of the counting run of one request."""
+    h = nu.create(pb, block=block, tpt=tpt, flags=nu.NU_FLAG_KEEP_QI)
+    b = nu.nu_batch_create([h])
+    try:
+        nu.nu_batch_run(b)
+        runs = [(*nu.nu_profile_result(h, pb.n_out), nu.nu_profile_qi(h, pb.n_traj))]
+        nu.nu_batch_branch_counts(b)
+        runs.append((*nu.nu_profile_result(h, pb.n_out), nu.nu_profile_qi(h, pb.n_traj)))
+        return runs
+    finally:
+        nu.nu_batch_destroy(b)
+        nu.nu_profile_destroy(h)
+
+
+PLAIN = W.plain_small(precision=W.MIXED)[0]
+CASES = {
+    # whole warps that stay in the NFW part, leave it and come back
+    "core_and_edge": PLAIN.replace(radii=np.geomspace(1.0, 3000.0, 7), n_steps=203),
+    "wide_fit_edge_at_its_end": PLAIN.replace(c=16.0, n_steps=120),
+    "narrow_fit_edge_at_its_end": PLAIN.replace(c=8.0, n_steps=120),
+    "logarithm_above_16": PLAIN.replace(c=25.0, n_steps=120),
+    "edge_below_one": PLAIN.replace(c=0.5, n_steps=120),
+    # the NFW edge lies beyond R before the onset: the bounds of the stages differ
+    "past_the_onset": PLAIN.replace(z_end=6.0, n_steps=150),
+    "no_halo": PLAIN.replace(M_h=0.0, n_steps=9),
+    "one_step": PLAIN.replace(n_steps=1),
+    # r^2 overflows float32 (and y is NaN) for one radius; the others share its launch
+    "radius_out_of_float_range": PLAIN.replace(radii=np.array([5.0, 1e25, 80.0]), n_steps=40),
+    "ragged_33": PLAIN.replace(n_q=3, n_mu=11, n_steps=65),
+    "ragged_257": PLAIN.replace(n_q=257, n_mu=1, n_steps=64),
+}
+
+
+@pytest.mark.parametrize("name", CASES)
+@pytest.mark.parametrize("block,tpt", [(128, 3), (64, 3)])
+def test_packed_loop_is_bitwise_the_counting_loop(name, block, tpt):
+    for a, b in zip(*_both(CASES[name], block, tpt)):
+        assert np.array_equal(a, b, equal_nan=True)
