@@ -110,11 +110,9 @@ extern "C" {
 #define NU_FLAG_GRAPH    2 /* batches: capture the launch in a CUDA graph      */
 #define NU_FLAG_TIMING   4 /* batches: record CUDA events around the trajectory
                               kernel (read with nu_batch_kernel_ms)            */
-#define NU_FLAG_GTAB     8 /* runs and batches: read the per-step coefficient
-                              table in place through the L1 cache instead of
-                              staging it in shared memory (frees shared memory,
-                              so more CTAs fit on an SM); results are identical.
-                              A table larger than 227 KB is always read this way */
+#define NU_FLAG_GTAB     8 /* accepted without effect: named where the kernels find
+                              the per-step coefficient table, which no kernel
+                              stages as a whole any more                       */
 #define NU_FLAG_VERIFY  16 /* mixed precision only: the request is also run in
                               the FP64 mode (same grids and steps) on the GPU,
                               and err_est then reports, per result, the error
@@ -181,12 +179,13 @@ typedef struct nu_opts {
     int precision;       /* NU_FP64 or NU_MIXED                                   */
     double z_end;        /* end of the backward integration; <= 0 -> the paper's z_i */
     int radii_unit;      /* NU_RADII_*                                            */
-    int block;           /* threads per CTA: 0 (default 256) or 64..512, multiple of 32 */
-    int tpt;             /* trajectories per thread: 0 (default 1), 1, 2, or 3 =
-                            two per thread in packed FP32x2 arithmetic (mixed
-                            precision; results bitwise those of 2).  The fastest
-                            mixed-precision shape on GB300 is block 128, tpt 3
-                            with NU_FLAG_GTAB; nu_autotune finds it            */
+    int block;           /* 0 (default 256) or 64..512, multiple of 32            */
+    int tpt;             /* 0 (default 1), 1, 2, or 3 (mixed precision only; as 2).
+                            block x tpt trajectories (tpt 3: block x 2) are a tile,
+                            whose sums are added in order, so the shape fixes the
+                            rounding of the sums.  How a launch runs its tiles
+                            (kernel, threads, split) the library chooses from the
+                            precision and the launch's size, with the same bits   */
     int flags;           /* NU_FLAG_*                                             */
     nu_alloc_fn alloc;
     nu_free_fn free;
@@ -196,10 +195,8 @@ typedef struct nu_opts {
                             (nu_profile_compute_noalloc); 0 -> 60000 ms      */
 } nu_opts;
 
-#define NU_MAX_STEPS 3000  /* the per-step coefficient table (80 B per step in FP32,
-                              160 B in FP64) is staged in
-                              shared memory when it fits in 227 KB and read
-                              through the L1 cache otherwise                     */
+#define NU_MAX_STEPS 3000  /* the per-step coefficient table takes 80 B per step
+                              (160 B in FP64)                                  */
 
 typedef struct nu_profile nu_profile;
 typedef struct nu_batch nu_batch;
@@ -218,7 +215,7 @@ typedef struct nu_plan_info {
     long long h2d_bytes;     /* bytes create() copies host -> device          */
     long long traj_steps;    /* n_traj * n_steps                              */
     long long device_bytes;  /* device memory create() will allocate          */
-    int n_tiles;             /* work tiles of one run                         */
+    int n_tiles;             /* tiles of the shape in one run                 */
     int tile;                /* trajectories per tile (block * tpt)           */
     int precision;           /* NU_FP64 or NU_MIXED                           */
     int n_steps;             /* RK4 steps                                     */
@@ -324,11 +321,10 @@ NU_API int nu_batch_kernel_ms(nu_batch* b, float* ms);
 NU_API int nu_batch_branch_counts(nu_batch* b, void* stream, long long* counts);
 
 /* Launch-shape autotuner: times the batch of requests `hs` with each candidate
- * launch shape (threads per CTA x trajectories per thread x table source:
- * 256x1, 512x1, 256x2 staged in shared memory; 256x1, 384x1 through L1; and for
- * mixed precision the packed 256x3 and 128x3 through L1 and 256x3 staged; one
- * warm-up and the median of three runs) and reports the
- * fastest.  With cache_path != NULL, a JSON-lines cache keyed by GPU name,
+ * shape (block x tpt: 256x1, 512x1, 256x2, 256x1, 384x1, and for mixed precision
+ * 256x3, 128x3, 256x3, some of them with NU_FLAG_GTAB; one warm-up and the median
+ * of three runs) and reports the fastest.  The library chooses the kernel and its
+ * threads by itself, so shapes of one tile run alike.  With cache_path != NULL, a JSON-lines cache keyed by GPU name,
  * precision, step-count and trajectory-count buckets (powers of two) is read
  * first and appended to after tuning.  Results of different shapes agree to
  * rounding, not bit for bit (the reduction order changes).  All requests must
@@ -336,7 +332,7 @@ NU_API int nu_batch_branch_counts(nu_batch* b, void* stream, long long* counts);
 typedef struct nu_tune_result {
     int block;               /* best threads per CTA                          */
     int tpt;                 /* best trajectories per thread                  */
-    int flags;               /* best table source (0 or NU_FLAG_GTAB)         */
+    int flags;               /* the best candidate's flags                    */
     float best_ms;           /* trajectory-kernel time of one run with it     */
     int from_cache;          /* 1 if read from the cache (no timing done)     */
     int n_candidates;
@@ -468,7 +464,7 @@ NU_API void nu_server_destroy(nu_server* s);
  *   returns NU_ETIMEDOUT and its work keeps the array; later calls on that
  *   device first wait (again bounded) for that work, so keep its stream alive
  *   until a later call has returned something other than NU_ETIMEDOUT.
- *   Errors: NU_EINVAL, NU_ENOTSUP (the packed shape tpt = 3, a mass-reuse
+ *   Errors: NU_EINVAL, NU_ENOTSUP (the shape tpt = 3, a mass-reuse
  *   relic or a tabulated f: this entry point computes one closed-form
  *   distribution for one mass), NU_ETOOBIG (the request's device buffers, or
  *   its host tables, need more than NU_NOALLOC_MAX_BYTES, e.g. too many

@@ -83,11 +83,10 @@ int sm_count()
     return v;
 }
 
-int persistent_grid(int precision, int tpt, int block, size_t smem, int n_tiles, int* grid,
-                    bool gtab = false)
+int persistent_grid(const LaunchShape& shape, int n_tiles, int* grid)
 {
     int per_sm = 0;
-    const int rc = max_ctas_per_sm(precision, tpt, block, smem, &per_sm, gtab);
+    const int rc = max_ctas_per_sm(shape, &per_sm);
     if (rc != NU_OK) return rc;
     const int sms = sm_count();
     if (per_sm < 1 || sms < 1) return NU_ECUDA;
@@ -106,9 +105,8 @@ struct nu_profile {
     Derived d;
     nu_plan_info info;
     int n_radii = 0;
-    int tiles_per_seg = 0;
-    int n_tiles = 0;
-    size_t smem = 0;
+    LaunchShape shape;
+    int n_tiles = 0;                // of a launch of this request alone
     DeviceBlock mem;
     DevProblem hdp;                 // host copy (device pointers inside)
     DevProblem* d_prob = nullptr;
@@ -121,8 +119,9 @@ struct nu_profile {
 struct nu_batch {
     std::vector<nu_profile*> hs;
     int precision = NU_MIXED, tpt = 1, block = 256;
-    int n_tiles = 0;
-    size_t smem = 0;
+    LaunchShape shape;
+    int n_tiles = 0;                // of the launch
+    int n_tiles_asked = 0;          // of the shape asked for
     int grid = 0;
     DeviceBlock mem;
     DevProblem* d_probs = nullptr;
@@ -133,7 +132,6 @@ struct nu_batch {
     unsigned long long* d_tallies = nullptr;   // [5], allocated at the first count
     bool use_graph = false;
     bool timing = false;
-    bool gtab = false;
     cudaEvent_t t0 = nullptr, t1 = nullptr;
     bool timed_run = false;
     cudaGraphExec_t exec = nullptr;
@@ -145,7 +143,7 @@ namespace {
 
 int plan_common(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic* relic,
                 const double* radii, int n_radii, const nu_pgrid* grid, const nu_opts* opts_in,
-                nu_opts& o, Derived& d, nu_plan_info& info, int& tiles_per_seg)
+                nu_opts& o, Derived& d, nu_plan_info& info)
 {
     resolve_opts(opts_in, o);
     int rc = validate(cosmo, halo, relic, radii, n_radii, grid, &o);
@@ -154,7 +152,7 @@ int plan_common(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic* reli
     if (rc != NU_OK) return rc;
     const long long seg = (long long)grid->n_q * grid->n_mu;
     const int tile = o.block * traj_per_thread(o.tpt);
-    tiles_per_seg = (int)((seg + tile - 1) / tile);
+    const long long tiles_per_seg = (seg + tile - 1) / tile;
     std::memset(&info, 0, sizeof(info));
     info.R_kpc = d.R;
     info.r200_kpc = d.r200;
@@ -179,7 +177,7 @@ int plan_common(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic* reli
                                           &twin_h2d);
         info.h2d_bytes += twin_h2d;
     }
-    const long long nt = (long long)tiles_per_seg * n_radii;
+    const long long nt = tiles_per_seg * n_radii;
     if (nt > (1LL << 30)) return NU_EINVAL;
     info.n_tiles = (int)nt;
     info.tile = tile;
@@ -255,16 +253,13 @@ private:
 int launch_profile(nu_profile* h, cudaStream_t s)
 {
     int grid = 0;
-    const bool gtab = (h->opts.flags & NU_FLAG_GTAB) != 0;
-    int rc = persistent_grid(h->opts.precision, h->opts.tpt, h->opts.block, h->smem, h->n_tiles, &grid,
-                             gtab);
+    const int rc = persistent_grid(h->shape, h->n_tiles, &grid);
     if (rc != NU_OK) return rc;
     if (cudaMemsetAsync(h->d_ctrl, 0, 2 * sizeof(unsigned), s) != cudaSuccess) {
         cudaGetLastError();
         return NU_ECUDA;
     }
-    return launch_traj(h->opts.precision, h->opts.tpt, h->opts.block, grid, h->smem, h->d_prob,
-                       h->d_prefix, 1, h->n_tiles, h->d_ctrl, s, gtab);
+    return launch_traj(h->shape, grid, h->d_prob, h->d_prefix, 1, h->n_tiles, h->d_ctrl, s);
 }
 
 // err = |mixed - fp64| / |fp64| per result (0 where both are 0)
@@ -381,8 +376,7 @@ int nu_profile_plan(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic* 
     nu_opts o;
     Derived d;
     nu_plan_info tmp;
-    int tps = 0;
-    const int rc = plan_common(cosmo, halo, relic, radii, n_radii, p_grid, opts, o, d, tmp, tps);
+    const int rc = plan_common(cosmo, halo, relic, radii, n_radii, p_grid, opts, o, d, tmp);
     if (rc != NU_OK) return rc;
     *info = tmp;
     return NU_OK;
@@ -396,8 +390,7 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
     nu_opts o;
     Derived d;
     nu_plan_info info;
-    int tps = 0;
-    int rc = plan_common(cosmo, halo, relic, radii, n_radii, p_grid, opts, o, d, info, tps);
+    int rc = plan_common(cosmo, halo, relic, radii, n_radii, p_grid, opts, o, d, info);
     if (rc != NU_OK) return rc;
 
     std::unique_ptr<nu_profile> h(new (std::nothrow) nu_profile());
@@ -412,9 +405,8 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
     h->d = d;
     h->info = info;
     h->n_radii = n_radii;
-    h->tiles_per_seg = tps;
-    h->n_tiles = info.n_tiles;
-    h->smem = coef_smem_bytes(o.precision, o.n_steps);
+    h->shape = plan_shape(o.precision, info.tile, info.n_traj);
+    h->n_tiles = tiles_of(h->shape, (long long)p_grid->n_q * p_grid->n_mu) * n_radii;
 
     // ---- host tables (FP64) ----
     const int nq = p_grid->n_q, nmu = p_grid->n_mu, N = o.n_steps;
@@ -514,8 +506,7 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
     P.n_q = nq;
     P.n_mu = nmu;
     P.n_steps = N;
-    P.tiles_per_seg = tps;
-    P.tile = o.block * traj_per_thread(o.tpt);
+    set_tiles(P, h->shape);
     P.precision = o.precision;
     P.n_mass = nm;
 
@@ -721,28 +712,29 @@ int nu_batch_create(nu_profile* const* hs, int n, const nu_opts* opts, nu_batch*
         b->hs.push_back(hs[i]);
     }
     if (b->tpt == kTptPacked && b->precision != NU_MIXED) return NU_EINVAL;
-    for (int i = 0; i < n; ++i) {
-        b->smem = std::max(b->smem, coef_smem_bytes(b->precision, hs[i]->opts.n_steps));
-    }
     const int tile = b->block * traj_per_thread(b->tpt);
+    long long n_traj = 0;
+    for (int i = 0; i < n; ++i) n_traj += hs[i]->info.n_traj;
+    b->shape = plan_shape(b->precision, tile, n_traj);
     std::vector<DevProblem> descs(n);
     std::vector<int> prefix(n + 1, 0);
+    long long asked = 0;
     for (int i = 0; i < n; ++i) {
         descs[i] = hs[i]->hdp;
+        set_tiles(descs[i], b->shape);
         const long long seg = (long long)hs[i]->grid.n_q * hs[i]->grid.n_mu;
-        descs[i].tile = tile;
-        descs[i].tiles_per_seg = (int)((seg + tile - 1) / tile);
+        asked += (seg + tile - 1) / tile * hs[i]->n_radii;
         const long long next = (long long)prefix[i] + (long long)descs[i].tiles_per_seg * hs[i]->n_radii;
         if (next > (1LL << 30)) return NU_EINVAL;
         prefix[i + 1] = (int)next;
     }
     b->n_tiles = prefix[n];
+    b->n_tiles_asked = (int)asked;
 
     nu_opts o;
     resolve_opts(opts, o);
     if (opts) b->use_graph = (opts->flags & NU_FLAG_GRAPH) != 0;
     if (opts) b->timing = (opts->flags & NU_FLAG_TIMING) != 0;
-    if (opts) b->gtab = (opts->flags & NU_FLAG_GTAB) != 0;
     if (b->timing && (cudaEventCreate(&b->t0) != cudaSuccess || cudaEventCreate(&b->t1) != cudaSuccess)) {
         cudaGetLastError();
         return NU_ECUDA;
@@ -773,7 +765,7 @@ int nu_batch_create(nu_profile* const* hs, int n, const nu_opts* opts, nu_batch*
     b->d_ctrl = reinterpret_cast<unsigned*>(base + o_ctrl);
     b->d_probs = reinterpret_cast<DevProblem*>(base + o_probs);
     b->d_prefix = reinterpret_cast<int*>(base + o_pref);
-    rc = persistent_grid(b->precision, b->tpt, b->block, b->smem, b->n_tiles, &b->grid, b->gtab);
+    rc = persistent_grid(b->shape, b->n_tiles, &b->grid);
     if (rc != NU_OK) {
         b->mem.release();
         return rc;
@@ -787,8 +779,8 @@ static int batch_enqueue(nu_batch* b, cudaStream_t s, bool timed)
 {
     if (cudaMemsetAsync(b->d_ctrl, 0, 2 * sizeof(unsigned), s) != cudaSuccess) return NU_ECUDA;
     if (timed && cudaEventRecord(b->t0, s) != cudaSuccess) return NU_ECUDA;
-    int rc = launch_traj(b->precision, b->tpt, b->block, b->grid, b->smem, b->d_probs,
-                         b->d_prefix, (int)b->hs.size(), b->n_tiles, b->d_ctrl, s, b->gtab);
+    int rc = launch_traj(b->shape, b->grid, b->d_probs, b->d_prefix, (int)b->hs.size(), b->n_tiles,
+                         b->d_ctrl, s);
     if (rc != NU_OK) return rc;
     if (timed && cudaEventRecord(b->t1, s) != cudaSuccess) return NU_ECUDA;
     for (nu_profile* h : b->hs)           // verified requests: their FP64 runs follow
@@ -873,8 +865,8 @@ int nu_batch_branch_counts(nu_batch* b, void* stream, long long* counts)
         cudaMemsetAsync(b->d_ctrl, 0, 2 * sizeof(unsigned), s) != cudaSuccess)
         rc = NU_ECUDA;
     if (rc == NU_OK)
-        rc = launch_traj_tally(b->precision, b->tpt, b->block, b->grid, b->smem, b->d_probs,
-                               b->d_prefix, (int)b->hs.size(), b->n_tiles, b->d_ctrl, b->d_tallies, s);
+        rc = launch_traj_tally(b->precision, b->shape, b->grid, b->d_probs, b->d_prefix,
+                               (int)b->hs.size(), b->n_tiles, b->d_ctrl, b->d_tallies, s);
     if (rc == NU_OK && (cudaMemcpyAsync(host, b->d_tallies, sizeof(host), cudaMemcpyDeviceToHost, s) !=
                             cudaSuccess ||
                         cudaStreamSynchronize(s) != cudaSuccess))
@@ -891,7 +883,7 @@ int nu_batch_info(const nu_batch* b, int* n_tiles, long long* traj_steps, long l
                   int* grid)
 {
     if (!b) return NU_EINVAL;
-    if (n_tiles) *n_tiles = b->n_tiles;
+    if (n_tiles) *n_tiles = b->n_tiles_asked;
     if (traj_steps) *traj_steps = b->traj_steps;
     if (h2d_bytes) *h2d_bytes = b->h2d_bytes;
     if (grid) *grid = b->grid;

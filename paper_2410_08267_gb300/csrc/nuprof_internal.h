@@ -47,11 +47,6 @@ enum CoefSlot {
 static_assert(C_COUNT == 20, "coefficient table layout");
 static_assert(C_COUNT % 4 == 0, "a step of the FP32 table is whole 16-byte words");
 
-// Largest dynamic shared memory of one CTA (GB300: 227 KB).  A table that does
-// not fit is read through the L1 cache instead of being staged (same values,
-// same results).
-constexpr size_t kMaxStagedSmem = 232448;
-
 // Halo and background quantities derived on the host in FP64 (Sec. II.B).
 struct Derived {
     double H0, rho_bar0, R, z_i, r200, r_s, Ic;
@@ -116,6 +111,7 @@ struct DevProblem {
     double ftab_scale;      // (n_ftab - 1) / ln(q_last / q_first)
     int n_radii, n_q, n_mu, n_steps;
     int tiles_per_seg, tile;
+    int group;              // tiles that make one tile of the request's shape
     int precision;
     int n_mass;
     // Chunked integration (serving): when `state` is set, a launch advances
@@ -166,20 +162,40 @@ nu_profile* profile_twin(const nu_profile* h);
 int profile_twin_run(nu_profile* h, void* stream);
 int profile_twin_query(const nu_profile* h);
 
-// Kernel launch helpers (traj_kernel.cu).
-int launch_traj(int precision, int tpt, int block, int grid, size_t smem_bytes,
-                const DevProblem* d_probs, const int* d_tile_prefix, int n_probs, int n_tiles,
-                unsigned* d_tile_counter, void* stream, bool gtab = false,
-                QueueCtl* d_queue = nullptr);
-int launch_traj_tally(int precision, int tpt, int block, int grid, size_t smem_bytes,
-                      const DevProblem* d_probs, const int* d_tile_prefix, int n_probs, int n_tiles,
-                      unsigned* d_tile_counter, unsigned long long* d_tallies, void* stream);
-int max_ctas_per_sm(int precision, int tpt, int block, size_t smem_bytes, int* out,
-                    bool gtab = false);
+// Kernel launch helpers (traj_kernel.cu).  A request's or batch's shape
+// (nu_opts.block x tpt) fixes its tile, whose sums are added in order, and so the
+// rounding of its results; how a launch runs such tiles is chosen by plan_shape.
+enum TrajKernelKind { kPacked, kRing, kFp64, kGeneralF32, kCountF32, kCountF64 };
+struct LaunchShape {
+    int kernel;      // TrajKernelKind
+    int threads;     // of a CTA
+    int tile;        // trajectories a CTA claims at a time
+    int group;       // such tiles in one tile of the asked shape
+};
+LaunchShape plan_shape(int precision, int tile, long long n_traj);
+LaunchShape whole_tiles(int precision, int tile);
+constexpr long long kLargeLaunch = 1LL << 34;   // n_traj of a launch of unknown size
+// Tiles of one radius with n_seg trajectories.
+inline int tiles_of(const LaunchShape& s, long long n_seg)
+{
+    return (int)((n_seg + s.tile - 1) / s.tile);
+}
+inline void set_tiles(DevProblem& P, const LaunchShape& s)
+{
+    P.tile = s.tile;
+    P.group = s.group;
+    P.tiles_per_seg = tiles_of(s, (long long)P.n_q * P.n_mu);
+}
+int launch_traj(const LaunchShape& shape, int grid, const DevProblem* d_probs,
+                const int* d_tile_prefix, int n_probs, int n_tiles, unsigned* d_tile_counter,
+                void* stream, QueueCtl* d_queue = nullptr);
+int launch_traj_tally(int precision, const LaunchShape& shape, int grid, const DevProblem* d_probs,
+                      const int* d_tile_prefix, int n_probs, int n_tiles, unsigned* d_tile_counter,
+                      unsigned long long* d_tallies, void* stream);
+int max_ctas_per_sm(const LaunchShape& shape, int* out);
 // Smallest tile (block 64 x 1 trajectory): request buffers of tile sums are
 // sized for it, so a batch may run any tile shape over existing requests.
 constexpr int kMinTile = 64;
-size_t coef_smem_bytes(int precision, int n_steps);
 // Trajectories per thread of a tile shape: tpt 3 is two trajectories per
 // thread in packed FP32x2 arithmetic (mixed precision only).
 inline int traj_per_thread(int tpt) { return tpt == 3 ? 2 : tpt; }

@@ -103,15 +103,13 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
 
     const int nq = p_grid->n_q, nmu = p_grid->n_mu, N = o.n_steps;
     const long long seg = (long long)nq * nmu;
-    const int tile = o.block * o.tpt;
-    const long long tps_ll = (seg + tile - 1) / tile;
-    const long long n_tiles_ll = tps_ll * n_radii;
-    if (n_tiles_ll > (1LL << 30)) return NU_ETOOBIG;
-    const int tps = (int)tps_ll, n_tiles = (int)n_tiles_ll;
-
-    // Device layout (the same order as the buffers of nu_profile_create).
+    // Device layout (the same order as the buffers of nu_profile_create), with the
+    // tiles of a launch of this size or, where their sums do not fit the array,
+    // with the whole ones of the shape.
     const bool fp64 = o.precision == NU_FP64;
     const size_t sz = fp64 ? sizeof(double) : sizeof(float);
+    LaunchShape shape;
+    int tps = 0, n_tiles = 0;
     size_t off = 0;
     auto carve = [&](size_t bytes) { size_t at = off; off += up256(bytes); return at; };
     const size_t o_ctrl = carve(4 * sizeof(unsigned));
@@ -127,11 +125,21 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
     const size_t o_wmu = carve((size_t)nmu * sizeof(double));
     const size_t o_mass = carve(3 * sizeof(double));      // mass scale 1, two normalisations
     const size_t upload_end = off;
-    const size_t o_part = carve((size_t)n_radii * tps * 2 * sizeof(double));
     const size_t o_cnt = carve((size_t)n_radii * sizeof(unsigned));
     const size_t o_out = carve((size_t)n_radii * sizeof(double));
     const size_t o_err = carve((size_t)n_radii * sizeof(double));
-    if (off > kArenaBytes) return NU_ETOOBIG;             // the device array
+    const size_t o_part = off;
+    for (bool whole : {false, true}) {
+        shape = whole ? whole_tiles(o.precision, o.block * o.tpt)
+                      : plan_shape(o.precision, o.block * o.tpt, seg * n_radii);
+        const long long tiles = (seg + shape.tile - 1) / shape.tile * n_radii;
+        if (tiles > (1LL << 30)) continue;
+        n_tiles = (int)tiles;
+        tps = tiles_of(shape, seg);
+        off = o_part + up256((size_t)n_radii * tps * 2 * sizeof(double));
+        if (off <= kArenaBytes) break;
+    }
+    if (tps == 0 || off > kArenaBytes) return NU_ETOOBIG;             // the device array
     // Host layout of the static staging buffer: the upload image, then the
     // FP64 tables and the read-back results.
     size_t hoff = upload_end;
@@ -220,8 +228,7 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
     P.n_q = nq;
     P.n_mu = nmu;
     P.n_steps = N;
-    P.tiles_per_seg = tps;
-    P.tile = tile;
+    set_tiles(P, shape);
     P.precision = o.precision;
     P.n_mass = 1;
 
@@ -249,8 +256,7 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
     put_into<double>(st, o_mass, mass, 3);
 
     int per_sm = 0, sms = 0;
-    const size_t smem = coef_smem_bytes(o.precision, N);
-    rc = max_ctas_per_sm(o.precision, o.tpt, o.block, smem, &per_sm);
+    rc = max_ctas_per_sm(shape, &per_sm);
     if (rc != NU_OK) return rc;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_id) != cudaSuccess ||
         per_sm < 1) {
@@ -270,8 +276,7 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
         if (wait_bounded(s, timeout_ms) != NU_OK) pend = {true, s};
         return NU_ECUDA;
     }
-    rc = launch_traj(o.precision, o.tpt, o.block, grid, smem,
-                     reinterpret_cast<const DevProblem*>(dev + o_prob),
+    rc = launch_traj(shape, grid, reinterpret_cast<const DevProblem*>(dev + o_prob),
                      reinterpret_cast<const int*>(dev + o_pref), 1, n_tiles,
                      reinterpret_cast<unsigned*>(dev + o_ctrl), stream);
     if (rc != NU_OK) cudaGetLastError();

@@ -348,9 +348,7 @@ void nu_server::deliver_verified()
 void nu_server::run()
 {
     cudaSetDevice(device);
-    const int tpt = o.tpt;
-    const int tile = o.block * traj_per_thread(tpt);
-    const bool gtab = (o.flags & NU_FLAG_GTAB) != 0;
+    const int tile = o.block * traj_per_thread(o.tpt);
     int slot = 0;
     for (;;) {
         {
@@ -397,20 +395,19 @@ void nu_server::run()
         double traj_active = 0.0;
         for (const Active& a : active) traj_active += (double)profile_n_traj(a.h);
         int chunk = o.chunk_steps;
+        // (requests may join a resident launch later, so its size is not known)
+        const LaunchShape shape = plan_shape(o.precision, tile, o.resident ? kLargeLaunch
+                                                                          : (long long)traj_active);
         if (chunk > 0 && traj_active * chunk > o.step_budget)
             chunk = std::max(1, (int)(o.step_budget / traj_active));
         std::vector<DevProblem> desc(active.size());
         std::vector<int> early_st(active.size(), 0);   // 1: signals this launch, 2: delivered
         std::vector<int> prefix(active.size() + 1, 0);
         long long steps_this = 0;
-        size_t smem = 0;                          // the largest table staged this launch
         for (size_t i = 0; i < active.size(); ++i) {
             const Active& a = active[i];
-            smem = std::max(smem, coef_smem_bytes(o.precision, a.n_steps));
             DevProblem d = profile_desc(a.h);
-            const long long seg = (long long)d.n_q * d.n_mu;
-            d.tile = tile;
-            d.tiles_per_seg = (int)((seg + tile - 1) / tile);
+            set_tiles(d, shape);
             d.state = a.state;
             d.step_begin = a.progress;
             d.step_end = std::min(a.n_steps, a.progress + (chunk > 0 ? chunk : a.n_steps));
@@ -436,11 +433,8 @@ void nu_server::run()
             (h_flags && cudaMemsetAsync(d_counts, 0, n * sizeof(unsigned), compute) != cudaSuccess))
             rc = NU_ECUDA;
         int grid = 0, per_sm = 0, sms = 0;
-        // a resident launch stages tables up to the largest a request may have
-        // (requests join it later), so that its shared memory fits any of them
         const bool res = o.resident != 0;
-        if (res) smem = std::max(smem, coef_smem_bytes(o.precision, NU_MAX_STEPS));
-        if (rc == NU_OK) rc = max_ctas_per_sm(o.precision, tpt, o.block, smem, &per_sm, gtab);
+        if (rc == NU_OK) rc = max_ctas_per_sm(shape, &per_sm);
         if (rc == NU_OK && (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
                             per_sm < 1))
             rc = NU_ECUDA;
@@ -455,8 +449,8 @@ void nu_server::run()
             // a resident launch keeps every CTA: the ones without work wait for
             // requests that join
             grid = res ? per_sm * sms : std::max(1, std::min(prefix[n], per_sm * sms));
-            rc = launch_traj(o.precision, tpt, o.block, grid, smem, d_desc[slot], d_prefix[slot], n,
-                             prefix[n], d_ctrl, compute, gtab, res ? d_q : nullptr);
+            rc = launch_traj(shape, grid, d_desc[slot], d_prefix[slot], n, prefix[n], d_ctrl, compute,
+                             res ? d_q : nullptr);
         }
         const auto t_launch = Clock::now();
         auto t_publish = t_launch;               // resident: the last time work joined
@@ -484,9 +478,7 @@ void nu_server::run()
                 Active& a = staged[k];
                 const int i = (int)active.size();
                 DevProblem d = profile_desc(a.h);
-                const long long seg = (long long)d.n_q * d.n_mu;
-                d.tile = tile;
-                d.tiles_per_seg = (int)((seg + tile - 1) / tile);
+                set_tiles(d, shape);
                 d.state = a.state;
                 d.step_begin = 0;
                 d.step_end = a.n_steps;

@@ -6,8 +6,7 @@
 // growing NFW halo (App. A).  The state (x, y, vx, vy) stays in registers for
 // the whole integration; the per-step coefficients (background, growth,
 // coupling at the three RK stage times, built in FP64 on the host) are read as
-// warp-uniform vector loads, either staged once per request into shared memory
-// or (GTAB) in place through the L1 cache.  At the end the Liouville map
+// warp-uniform vector loads through the L1 cache.  At the end the Liouville map
 // f0 = f_init(P_i) (Sec. II.C) and the weight of the trajectory in
 // Eq. localdensity are applied, once per relic mass read from the trajectory
 // (Sec. III), and each tile's sum is formed by a warp-shuffle + shared-memory tree.  Tile sums land in a per-request
@@ -20,6 +19,7 @@
 // one request, so uneven batches of requests share one launch.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <type_traits>
@@ -131,16 +131,100 @@ __device__ __forceinline__ float nfw_I_log(float y, float u)
 // I = -ln(1-t) - t = t^2 sum_{k>=0} t^k/(k+2), a series of positive terms; for
 // t < 1/2 (y < 1) it is summed by Horner through k = 50 (truncation below
 // 1e-16 relative), above that the two terms no longer cancel badly.
-__device__ __forceinline__ double nfw_I(double y)
+//
+// An FP64 operation holds a scheduler's FP64 unit for 64 cycles here, where an FP32
+// or integer one takes one or two: the FP64 force is bound by the number of its
+// FP64 operations, one warp on a scheduler is enough to keep the unit busy, and
+// work moved off it is free.  So:
+// * Horner's recurrence p <- t p + 1/(k+2) forgets its start by a factor t a step.
+//   It starts in FP32, whose relative error 2^-22 is multiplied by t^J in the J
+//   FP64 steps that remain; J is the smallest multiple of 4 that makes that
+//   2^-93, 2^-40 of an ulp of the sum.  So the sum has the bits of the whole
+//   recurrence but where a rounding lies within 2^-40 ulp of a tie.
+// * Non-negative numbers are ordered as their bits, so tests are integer ones.
+// * t is the correctly rounded quotient from Newton's iteration and Markstein's
+//   final correction (IBM J. Res. Dev. 34, 1990): the seed is an FP32 reciprocal.
+constexpr float kSeriesBits = 71.0f;       // 93 - 22
+constexpr int kSeriesTail = 20;            // FP32 terms: 2^-23 at the largest t that uses them
+constexpr int kSeriesMaxJ = 48;            // above: the whole recurrence
+
+__constant__ float c_series[kSeriesMaxJ + kSeriesTail] = {   // 1/(k+2)
+#define NU_INV4(k) 1.0f / ((k) + 2), 1.0f / ((k) + 3), 1.0f / ((k) + 4), 1.0f / ((k) + 5)
+#define NU_INV16(k) NU_INV4(k), NU_INV4((k) + 4), NU_INV4((k) + 8), NU_INV4((k) + 12)
+    NU_INV16(0), NU_INV16(16), NU_INV16(32), NU_INV16(48), NU_INV4(64)
+#undef NU_INV16
+#undef NU_INV4
+};
+
+// a < b for doubles that are not negative (NaN: false for a NaN a)
+__device__ __forceinline__ bool less_nonneg(double a, double b)
 {
-    const double t = y / (1.0 + y);
-    if (t < 0.5) {
-        double p = 1.0 / 52.0;
-#pragma unroll   // fully: the coefficients 1/(k+2) become compile-time constants
-        for (int k = 49; k >= 0; --k) p = fma(p, t, 1.0 / (double)(k + 2));
-        return (t * t) * p;
+    return __double_as_longlong(a) < __double_as_longlong(b);
+}
+
+// float of a positive double, truncated (values below the float range: about 1e-38),
+// and double of a positive float; integer operations only.
+__device__ __forceinline__ float trunc_f32(double v)
+{
+    const int hi = max(__double2hiint(v), 0x38100000);
+    return __uint_as_float(((unsigned)(hi - 0x38000000) << 3) | ((unsigned)__double2loint(v) >> 29));
+}
+__device__ __forceinline__ double widen_f32(float v)
+{
+    const unsigned b = __float_as_uint(v);
+    return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+
+// y / u for 0 <= y < u and 1 <= u (6 FP64 operations).
+__device__ __forceinline__ double quotient(double y, double u)
+{
+    const double r0 = widen_f32(rcp_approx(trunc_f32(u)));   // 1/u to 2^-22
+    const double e = fma(-u, r0, 1.0);
+    const double r = fma(r0, fma(e, e, e), r0);               // to an ulp
+    const double q = y * r;
+    return fma(fma(-q, u, y), r, q);                          // the remainder is exact
+}
+
+template <int K>
+__device__ __forceinline__ double series4(double p, double t)   // terms K + 3 .. K
+{
+    p = fma(p, t, 1.0 / (K + 5));
+    p = fma(p, t, 1.0 / (K + 4));
+    p = fma(p, t, 1.0 / (K + 3));
+    return fma(p, t, 1.0 / (K + 2));
+}
+
+// sum_{k=0}^{50} t^k/(k+2) for 0 < t <= t_max < 1/2.
+__device__ __forceinline__ double nfw_series(double t, float t_max)
+{
+    const int need = (int)(kSeriesBits * rcp_approx(-lg2_approx(t_max))) + 1;
+    const int J = max(8, (need + 3) & ~3);
+    double p;
+    if (J > kSeriesMaxJ) {
+        p = 1.0 / 52.0;
+        p = fma(p, t, 1.0 / 51.0);
+        p = fma(p, t, 1.0 / 50.0);
+    } else {
+        const float tf = trunc_f32(t);
+        float s = c_series[J + kSeriesTail - 1];
+#pragma unroll
+        for (int i = kSeriesTail - 2; i >= 0; --i) s = fmaf(s, tf, c_series[J + i]);
+        p = widen_f32(s);
     }
-    return log1p(y) - t;
+    switch (min(J, kSeriesMaxJ)) {
+    case 48: p = series4<44>(p, t);   // fallthrough, as all below
+    case 44: p = series4<40>(p, t);
+    case 40: p = series4<36>(p, t);
+    case 36: p = series4<32>(p, t);
+    case 32: p = series4<28>(p, t);
+    case 28: p = series4<24>(p, t);
+    case 24: p = series4<20>(p, t);
+    case 20: p = series4<16>(p, t);
+    case 16: p = series4<12>(p, t);
+    case 12: p = series4<8>(p, t);
+    default: p = series4<4>(p, t);
+    }
+    return series4<0>(p, t);
 }
 
 // Steps between two tests of the early exit (a power of two).
@@ -261,24 +345,35 @@ __device__ __forceinline__ float accel_m(float x, float y, float S, float Yq, fl
     return m;
 }
 
-template <class Ctr = NoTally>
+// FP64.  WARP: every lane of the warp is here (the integration loops), and the
+// series' length is that of the lane that needs most.
+template <class Ctr = NoTally, bool WARP = true>
 __device__ __forceinline__ double accel_m(double x, double y, double S, double Q, double,
                                           const HaloF64& hc, Ctr& ctr)
 {
     const double r2 = fma(x, x, y * y);
-    double m = 0.0;
-    if (r2 < hc.R2) {
-        const double rinv = rsqrt(fmax(r2, 1e-200));
-        const double rinv3 = rinv * rinv * rinv;
-        double sel = 1.0;
-        if (r2 < Q) {
-            const double ys = (r2 * rinv) * S;
+    const bool in = less_nonneg(r2, hc.R2), nfw = in && less_nonneg(r2, Q);
+    double m = 0.0, rinv = 0.0, ys = 0.0, t = 0.0, sel = 1.0;
+    if (in) rinv = rsqrt(less_nonneg(r2, 1e-200) ? 1e-200 : r2);
+    bool series = false;
+    if (nfw) {
+        ys = (r2 * rinv) * S;
+        t = quotient(ys, 1.0 + ys);
+        series = less_nonneg(t, 0.5);
+    }
+    unsigned t_max = series ? __float_as_uint(trunc_f32(t)) : 0u;
+    if (WARP) t_max = __reduce_max_sync(0xffffffffu, t_max);
+    if (in) {
+        if (nfw) {
             ctr.add(ys < 1.0 ? 2 : 3);
-            sel = nfw_I(ys) * hc.invIc;
+            // the truncated t_max is one float below t at most
+            const double I = series ? (t * t) * nfw_series(t, __uint_as_float(t_max + 1u))
+                                    : log1p(ys) - t;
+            sel = I * hc.invIc;
         } else {
             ctr.add(1);
         }
-        m = fma(sel, rinv3, -hc.invR3);
+        m = fma(sel, rinv * rinv * rinv, -hc.invR3);
     } else {
         ctr.add(0);
     }
@@ -441,15 +536,57 @@ __device__ __forceinline__ float max3_nan(float a, float b, float c)
     return r;
 }
 
-struct HaloX2 {
-    f2 invIc, neg_invR3;
-    float R2, c;
-};
+// The operations of a step for one trajectory (float) and for two (f2): the same
+// roundings, so both forms of the step below give a trajectory the same bits.
+__device__ __forceinline__ float fmav(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ f2 fmav(f2 a, f2 b, f2 c) { return fma2(a, b, c); }
+__device__ __forceinline__ float mulv(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ f2 mulv(f2 a, f2 b) { return mul2(a, b); }
+__device__ __forceinline__ float addv(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ f2 addv(f2 a, f2 b) { return add2(a, b); }
+__device__ __forceinline__ float rsqrtv(float a) { return rsqrt_approx(a); }
+__device__ __forceinline__ f2 rsqrtv(f2 a) { return pk(rsqrt_approx(f2lo(a)), rsqrt_approx(f2hi(a))); }
+__device__ __forceinline__ float rcpv(float a) { return rcp_approx(a); }
+__device__ __forceinline__ f2 rcpv(f2 a) { return pk(rcp_approx(f2lo(a)), rcp_approx(f2hi(a))); }
+__device__ __forceinline__ float rcp_negv(float a) { return rcp_approx(-a); }
+__device__ __forceinline__ f2 rcp_negv(f2 a) { return pk(rcp_approx(-f2lo(a)), rcp_approx(-f2hi(a))); }
+__device__ __forceinline__ float lg2v(float a) { return lg2_approx(a); }
+__device__ __forceinline__ f2 lg2v(f2 a) { return pk(lg2_approx(f2lo(a)), lg2_approx(f2hi(a))); }
+template <class V> __device__ __forceinline__ V splat(float a);
+template <> __device__ __forceinline__ float splat<float>(float a) { return a; }
+template <> __device__ __forceinline__ f2 splat<f2>(float a) { return dup(a); }
+// largest of all values, NaN if one of them is NaN
+__device__ __forceinline__ float max_nan(float a) { return a; }
+__device__ __forceinline__ float max_nan(f2 a) { return max3_nan(f2lo(a), f2hi(a), f2hi(a)); }
+__device__ __forceinline__ float max_nan(float a, float b, float c, float d)
+{
+    return max3_nan(max3_nan(a, b, c), d, d);
+}
+__device__ __forceinline__ float max_nan(f2 a, f2 b, f2 c, f2 d)
+{
+    const float m = max3_nan(f2lo(a), f2hi(a), f2lo(b)), n = max3_nan(f2hi(b), f2lo(c), f2hi(c));
+    return max3_nan(max3_nan(m, n, f2lo(d)), f2hi(d), f2hi(d));
+}
 
-// N(y) and D(y) of the rational g for both lanes (see nfw_N16, nfw_D16 and
-// nfw_N8, nfw_D8); NARROW selects the fit.
+template <class V>
+struct HaloV {
+    V invIc, neg_invR3;
+    float R2, R, c;
+};
+template <class V>
+__device__ __forceinline__ HaloV<V> halo_of(const HaloF32& h)
+{
+    return {splat<V>(h.invIc), splat<V>(-h.invR3), h.R2, h.R, h.c};
+}
+
+// N(y) and D(y) of the rational g (see nfw_N16, nfw_D16 and nfw_N8, nfw_D8);
+// NARROW selects the fit.
 template <bool NARROW>
-__device__ __forceinline__ f2 nfw_N_x2(f2 y)
+__device__ __forceinline__ float nfw_N(float y) { return NARROW ? nfw_N8(y) : nfw_N16(y); }
+template <bool NARROW>
+__device__ __forceinline__ float nfw_D(float y) { return NARROW ? nfw_D8(y) : nfw_D16(y); }
+template <bool NARROW>
+__device__ __forceinline__ f2 nfw_N(f2 y)
 {
     f2 p;
     if constexpr (NARROW) {
@@ -468,7 +605,7 @@ __device__ __forceinline__ f2 nfw_N_x2(f2 y)
     return p;
 }
 template <bool NARROW>
-__device__ __forceinline__ f2 nfw_D_x2(f2 y)
+__device__ __forceinline__ f2 nfw_D(f2 y)
 {
     f2 p;
     if constexpr (NARROW) {
@@ -488,241 +625,234 @@ __device__ __forceinline__ f2 nfw_D_x2(f2 y)
     return p;
 }
 
-// I(y) on the logarithm branch for both lanes (see nfw_I_log).
-__device__ __forceinline__ f2 nfw_I_log_x2(f2 y, f2 u)
+// One force evaluation: accel_m (FP32) without branches.
+//   kRational   the value on the rational branch of the NFW part
+//   kSelect     each lane's own branch, but not the logarithm; `logarithm` is set
+//               where a lane is on it
+//   kSelectLog  each lane's own branch
+enum StepForm { kRational, kSelect, kSelectLog };
+
+template <StepForm FORM>
+__device__ __forceinline__ float branch_of(float r2, float ys, float Yq, float R2, float c, float mq,
+                                           float ml, float ms, bool& logarithm)
 {
-    const float ua = f2lo(u), ub = f2hi(u);
-    const f2 lg = pk(lg2_approx(ua), lg2_approx(ub));
-    const f2 rn = pk(rcp_approx(-ua), rcp_approx(-ub));
-    return fma2(lg, dup(0.693147180559945309f), mul2(y, rn));
+    const bool in = r2 < R2, nfw = ys < c;
+    if constexpr (FORM == kSelect) logarithm |= in && nfw && !(ys < Yq);
+    const float mn = FORM == kSelectLog && nfw ? ml : ms;
+    return ys < Yq ? mq : in ? mn : 0.0f;
+}
+template <StepForm FORM>
+__device__ __forceinline__ f2 branch_of(f2 r2, f2 ys, float Yq, float R2, float c, f2 mq, f2 ml, f2 ms,
+                                        bool& logarithm)
+{
+    return pk(branch_of<FORM>(f2lo(r2), f2lo(ys), Yq, R2, c, f2lo(mq), f2lo(ml), f2lo(ms), logarithm),
+              branch_of<FORM>(f2hi(r2), f2hi(ys), Yq, R2, c, f2hi(mq), f2hi(ml), f2hi(ms), logarithm));
 }
 
-// Geometry of one force evaluation for both lanes of a register pair:
-// guarded r^2, 1/r, rs = S/r and y = r^2 rs.
-struct Geo2 {
-    f2 r2, rinv, rs, ys;
-};
-
-__device__ __forceinline__ Geo2 geometry_x2(f2 x, f2 y, f2 S)
+template <bool NARROW, StepForm FORM, class V>
+__device__ __forceinline__ V m_form(V x, V y, V S, float Yq, V T, const HaloV<V>& hc, V& ys,
+                                    bool& logarithm)
 {
-    Geo2 g;
-    g.r2 = fma2(x, x, fma2(y, y, dup(kR2Guard)));
-    g.rinv = pk(rsqrt_approx(f2lo(g.r2)), rsqrt_approx(f2hi(g.r2)));
-    g.rs = mul2(g.rinv, S);
-    g.ys = mul2(g.r2, g.rs);
-    return g;
-}
-
-// Per-branch formulas of accel_m for both lanes (FP32, the same operations).
-template <bool NARROW>
-__device__ __forceinline__ f2 m_rational_x2(const Geo2& g, f2 T, const HaloX2& hc)
-{
-    const f2 nr = mul2(nfw_N_x2<NARROW>(g.ys), mul2(g.rs, T));
-    const f2 d = nfw_D_x2<NARROW>(g.ys);
-    return fma2(nr, pk(rcp_approx(f2lo(d)), rcp_approx(f2hi(d))), hc.neg_invR3);
-}
-__device__ __forceinline__ f2 m_log_x2(const Geo2& g, f2 rinv2, const HaloX2& hc)
-{
-    const f2 sel = mul2(nfw_I_log_x2(g.ys, fma2(g.r2, g.rs, dup(1.0f))), hc.invIc);
-    return fma2(sel, mul2(rinv2, g.rinv), hc.neg_invR3);
-}
-__device__ __forceinline__ f2 m_shell_x2(const Geo2& g, f2 rinv2, const HaloX2& hc)
-{
-    return fma2(rinv2, g.rinv, hc.neg_invR3);
-}
-// shell or beyond R (0), for lanes outside the NFW edge
-__device__ __forceinline__ f2 m_out_x2(const Geo2& g, const HaloX2& hc)
-{
-    const f2 ms = m_shell_x2(g, mul2(g.rinv, g.rinv), hc);
-    return pk(f2lo(g.r2) < hc.R2 ? f2lo(ms) : 0.0f, f2hi(g.r2) < hc.R2 ? f2hi(ms) : 0.0f);
-}
-// any mix of branches: each formula that some lane of the warp needs,
-// evaluated for both lanes and selected per lane (q0, q1: on the rational branch)
-template <bool NARROW>
-__device__ __forceinline__ f2 m_mixed_x2(const Geo2& g, f2 T, const HaloX2& hc, bool need_log,
-                                         bool q0, bool q1)
-{
-    const f2 rinv2 = mul2(g.rinv, g.rinv);
-    const f2 mq = m_rational_x2<NARROW>(g, T, hc);
-    const f2 ml = need_log ? m_log_x2(g, rinv2, hc) : dup(0.0f);
-    const f2 ms = m_shell_x2(g, rinv2, hc);
-    const bool n0 = f2lo(g.ys) < hc.c, n1 = f2hi(g.ys) < hc.c;
-    const bool in0 = f2lo(g.r2) < hc.R2, in1 = f2hi(g.r2) < hc.R2;
-    return pk(!in0 ? 0.0f : q0 ? f2lo(mq) : n0 ? f2lo(ml) : f2lo(ms),
-              !in1 ? 0.0f : q1 ? f2hi(mq) : n1 ? f2hi(ml) : f2hi(ms));
-}
-
-// m = Mhat/r^3 at two independent points (a, b) of both lanes: lane by lane
-// the values of accel_m (FP32).  Within one RK4 step the first two stages'
-// positions depend only on the step's start state, and so do the last two
-// given the first two, so their force evaluations are independent and run
-// interleaved.  One warp vote covers all four lane-evaluations (the two
-// points of a pair almost always share their branch): every one on the
-// rational branch of the NFW part (y < Yq, which implies r < R), every one
-// outside the NFW edge (shell or beyond R), or any mix (each formula that a
-// lane needs evaluated for all and selected per lane).  Returns whether every
-// one was on the rational branch.  All lanes of the warp execute this function
-// together (the integration loop is warp-uniform).
-template <bool NARROW>
-__device__ __forceinline__ bool accel_m_pair_x2(f2 xa, f2 ya, f2 Sa, float Ya, f2 Ta,
-                                                f2 xb, f2 yb, f2 Sb, float Yb, f2 Tb,
-                                                const HaloX2& hc, f2& ma, f2& mb)
-{
-    const Geo2 ga = geometry_x2(xa, ya, Sa);
-    const Geo2 gb = geometry_x2(xb, yb, Sb);
-    const bool qa0 = f2lo(ga.ys) < Ya, qa1 = f2hi(ga.ys) < Ya;
-    const bool qb0 = f2lo(gb.ys) < Yb, qb1 = f2hi(gb.ys) < Yb;
-    const unsigned full = 0xffffffffu;
-    if (__all_sync(full, qa0 && qa1 && qb0 && qb1)) {
-        ma = m_rational_x2<NARROW>(ga, Ta, hc);
-        mb = m_rational_x2<NARROW>(gb, Tb, hc);
-        return true;
+    const V r2 = fmav(x, x, fmav(y, y, splat<V>(kR2Guard)));
+    const V rinv = rsqrtv(r2);
+    const V rs = mulv(rinv, S);
+    ys = mulv(r2, rs);
+    const V mq = fmav(mulv(nfw_N<NARROW>(ys), mulv(rs, T)), rcpv(nfw_D<NARROW>(ys)), hc.neg_invR3);
+    if constexpr (FORM == kRational) return mq;
+    const V rinv2 = mulv(rinv, rinv);
+    const V ms = fmav(rinv2, rinv, hc.neg_invR3);
+    V ml = ms;
+    if constexpr (FORM == kSelectLog) {
+        const V u = fmav(r2, rs, splat<V>(1.0f));
+        const V I = fmav(lg2v(u), splat<V>(0.693147180559945309f), mulv(ys, rcp_negv(u)));
+        ml = fmav(mulv(I, hc.invIc), mulv(rinv2, rinv), hc.neg_invR3);
     }
-    // lanes inside R and inside the NFW edge
-    const bool na0 = f2lo(ga.r2) < hc.R2 && f2lo(ga.ys) < hc.c;
-    const bool na1 = f2hi(ga.r2) < hc.R2 && f2hi(ga.ys) < hc.c;
-    const bool nb0 = f2lo(gb.r2) < hc.R2 && f2lo(gb.ys) < hc.c;
-    const bool nb1 = f2hi(gb.r2) < hc.R2 && f2hi(gb.ys) < hc.c;
-    if (__all_sync(full, !(na0 || na1 || nb0 || nb1))) {
-        ma = m_out_x2(ga, hc);
-        mb = m_out_x2(gb, hc);
-        return false;
-    }
-    // a lane of the NFW part above the rational branch (only halos with c > 16)
-    const bool la = (na0 && !qa0) || (na1 && !qa1);
-    const bool lb = (nb0 && !qb0) || (nb1 && !qb1);
-    const bool need_log = __any_sync(full, la || lb);
-    ma = m_mixed_x2<NARROW>(ga, Ta, hc, need_log, qa0, qa1);
-    mb = m_mixed_x2<NARROW>(gb, Tb, hc, need_log, qb0, qb1);
-    return false;
+    return branch_of<FORM>(r2, ys, Yq, hc.R2, hc.c, mq, ml, ms, logarithm);
 }
 
-// Four consecutive slots of a step's coefficients.
-template <bool GTAB>
-__device__ __forceinline__ float4 coef4(const float4* c4, int q)
+// One RK4 step: every value is formed by the operations of rk4_step.  The four
+// force evaluations run as two independent pairs: within a step the positions of
+// the first two stages depend only on its start state, and those of the last two
+// on it and the first pair's forces.
+// kRational and kSelect return false and leave the state as it was where a lane of
+// the warp is on another branch (kRational) or on the logarithm (kSelect), found
+// out with one vote near the step's end.  For kRational the bounds of the four
+// evaluations do not rise from stage to stage (S falls with z), so the largest y
+// against the last stage's bound decides, and a NaN (r^2 out of range, far beyond
+// R) decides against it.  `rational` says whether this lane's last evaluation was
+// on the rational branch.
+template <bool NARROW, StepForm FORM, class V>
+__device__ __forceinline__ bool rk4_form(V& x, V& y, V& vx, V& vy, const float4* row,
+                                         const HaloV<V>& hc, bool& rational)
 {
-    return GTAB ? __ldg(&c4[q]) : c4[q];
-}
+    const float4 q0 = row[0];                        // MA1 MA2 MA3 B1
+    const V MA1 = splat<V>(q0.x), MA2 = splat<V>(q0.y), MA3 = splat<V>(q0.z), B1 = splat<V>(q0.w);
+    const V X2 = fmav(MA1, vx, x), Y2 = fmav(MA1, vy, y);
+    const float4 q2 = row[2];                        // W1 W2 S0 S1
+    const float4 q3 = row[3];                        // S2 Q0 Q1 Q2
+    const float4 q4 = row[4];                        // T0 T1 T2 IREM
+    const V S0 = splat<V>(q2.z), S1 = splat<V>(q2.w), T0 = splat<V>(q4.x), T1 = splat<V>(q4.y);
+    V y1, y2, y3, y4;
+    bool logarithm = false;
+    const V m1 = m_form<NARROW, FORM>(x, y, S0, q3.y, T0, hc, y1, logarithm);
+    const V m2 = m_form<NARROW, FORM>(X2, Y2, S1, q3.z, T1, hc, y2, logarithm);
+    const float4 q1 = row[1];                        // B2 B3 B4 W0
+    const V p1 = mulv(B1, m1);
+    const V VX2 = fmav(p1, x, vx), VY2 = fmav(p1, y, vy);
+    const V p2 = mulv(splat<V>(q1.x), m2);
+    const V VX3 = fmav(p2, X2, vx), VY3 = fmav(p2, Y2, vy);
+    const V X3 = fmav(MA2, VX2, x), Y3 = fmav(MA2, VY2, y);
+    const V X4 = fmav(MA3, VX3, x), Y4 = fmav(MA3, VY3, y);
 
-// One RK4 step of both trajectories: every value is formed by the operations of
-// rk4_step.  c4 points at the step's C_COUNT coefficients; each group of four is
-// loaded where it is first needed, which keeps the table out of registers.  The
-// four force evaluations run as two independent pairs (stages 1 and 2, then 3
-// and 4).
-//
-// RATIONAL takes every evaluation of the warp to be on the rational branch of
-// the NFW part, as it mostly is, and finds out with one vote near
-// the step's end; where that was not so it returns false and leaves the state
-// as it was.  The bounds of the four evaluations do not rise from stage to stage
-// (S falls with z), so the largest of the eight y against the last stage's
-// bound decides, and a NaN (r^2 out of range far beyond R) decides against it.
-// Otherwise each pair votes, and the return value says whether every evaluation
-// was on the rational branch.
-template <bool GTAB, bool NARROW, bool RATIONAL>
-__device__ __forceinline__ bool rk4_step_x2(f2& x, f2& y, f2& vx, f2& vy, const float4* c4,
-                                            const HaloX2& hc)
-{
-    const float4 q0 = coef4<GTAB>(c4, 0);          // MA1 MA2 MA3 B1
-    const f2 MA1 = dup(q0.x), MA2 = dup(q0.y), MA3 = dup(q0.z), B1 = dup(q0.w);
-    const f2 X2 = fma2(MA1, vx, x), Y2 = fma2(MA1, vy, y);
-    const float4 q2 = coef4<GTAB>(c4, 2);          // W1 W2 S0 S1
-    const float4 q3 = coef4<GTAB>(c4, 3);          // S2 Q0 Q1 Q2
-    const float4 q4 = coef4<GTAB>(c4, 4);          // T0 T1 T2 IREM
-    const f2 S0 = dup(q2.z), S1 = dup(q2.w), T0 = dup(q4.x), T1 = dup(q4.y);
-    f2 m1, m2;
-    float y_max = 0.0f;
-    bool rational = true;
-    if constexpr (RATIONAL) {
-        const Geo2 g1 = geometry_x2(x, y, S0), g2 = geometry_x2(X2, Y2, S1);
-        m1 = m_rational_x2<NARROW>(g1, T0, hc);
-        m2 = m_rational_x2<NARROW>(g2, T1, hc);
-        y_max = max3_nan(f2lo(g1.ys), f2hi(g1.ys), f2lo(g2.ys));
-        y_max = max3_nan(y_max, f2hi(g2.ys), y_max);
+    const V S2 = splat<V>(q3.x), T2 = splat<V>(q4.z);
+    const V m3 = m_form<NARROW, FORM>(X3, Y3, S1, q3.z, T1, hc, y3, logarithm);
+    const V m4 = m_form<NARROW, FORM>(X4, Y4, S2, q3.w, T2, hc, y4, logarithm);
+    if constexpr (FORM == kRational) {
+        if (!__all_sync(0xffffffffu, max_nan(y1, y2, y3, y4) < q3.w)) return false;
     } else {
-        rational = accel_m_pair_x2<NARROW>(x, y, S0, q3.y, T0, X2, Y2, S1, q3.z, T1, hc, m1, m2);
+        if (FORM == kSelect && __any_sync(0xffffffffu, logarithm)) return false;
+        rational = max_nan(y4) < q3.w;
     }
-    const float4 q1 = coef4<GTAB>(c4, 1);          // B2 B3 B4 W0
-    const f2 p1 = mul2(B1, m1);
-    const f2 VX2 = fma2(p1, x, vx), VY2 = fma2(p1, y, vy);
-    const f2 p2 = mul2(dup(q1.x), m2);
-    const f2 VX3 = fma2(p2, X2, vx), VY3 = fma2(p2, Y2, vy);
-    const f2 X3 = fma2(MA2, VX2, x), Y3 = fma2(MA2, VY2, y);
-    const f2 X4 = fma2(MA3, VX3, x), Y4 = fma2(MA3, VY3, y);
 
-    const f2 S2 = dup(q3.x), T2 = dup(q4.z);
-    f2 m3, m4;
-    if constexpr (RATIONAL) {
-        const Geo2 g3 = geometry_x2(X3, Y3, S1), g4 = geometry_x2(X4, Y4, S2);
-        m3 = m_rational_x2<NARROW>(g3, T1, hc);
-        m4 = m_rational_x2<NARROW>(g4, T2, hc);
-        y_max = max3_nan(y_max, f2lo(g3.ys), f2hi(g3.ys));
-        y_max = max3_nan(y_max, f2lo(g4.ys), f2hi(g4.ys));
-        if (!__all_sync(0xffffffffu, y_max < q3.w)) return false;
-    } else {
-        rational &= accel_m_pair_x2<NARROW>(X3, Y3, S1, q3.z, T1, X4, Y4, S2, q3.w, T2, hc, m3, m4);
-    }
-    const f2 B3 = dup(q1.y), B4 = dup(q1.z), W0 = dup(q1.w), W1 = dup(q2.x), W2 = dup(q2.y);
-    const f2 p3 = mul2(B3, m3);
-    const f2 VX4 = fma2(p3, X3, vx), VY4 = fma2(p3, Y3, vy);
-    const f2 p4 = mul2(B4, m4);
-
-    const f2 nx = fma2(W2, VX4, fma2(W1, add2(VX2, VX3), fma2(W0, vx, x)));
-    const f2 ny = fma2(W2, VY4, fma2(W1, add2(VY2, VY3), fma2(W0, vy, y)));
-    const f2 p2x2 = mul2(p2, dup(2.0f));   // exact doubling
-    const f2 third = dup(1.0f / 3.0f);
-    const f2 tx = fma2(p3, X3, fma2(p2x2, X2, mul2(p1, x)));
-    const f2 ty = fma2(p3, Y3, fma2(p2x2, Y2, mul2(p1, y)));
-    vx = fma2(p4, X4, fma2(tx, third, vx));
-    vy = fma2(p4, Y4, fma2(ty, third, vy));
+    const V B3 = splat<V>(q1.y), B4 = splat<V>(q1.z);
+    const V W0 = splat<V>(q1.w), W1 = splat<V>(q2.x), W2 = splat<V>(q2.y);
+    const V p3 = mulv(B3, m3);
+    const V VX4 = fmav(p3, X3, vx), VY4 = fmav(p3, Y3, vy);
+    const V p4 = mulv(B4, m4);
+    const V nx = fmav(W2, VX4, fmav(W1, addv(VX2, VX3), fmav(W0, vx, x)));
+    const V ny = fmav(W2, VY4, fmav(W1, addv(VY2, VY3), fmav(W0, vy, y)));
+    const V p2x2 = mulv(p2, splat<V>(2.0f));         // exact doubling
+    const V third = splat<V>(1.0f / 3.0f);
+    const V tx = fmav(p3, X3, fmav(p2x2, X2, mulv(p1, x)));
+    const V ty = fmav(p3, Y3, fmav(p2x2, Y2, mulv(p1, y)));
+    vx = fmav(p4, X4, fmav(tx, third, vx));
+    vy = fmav(p4, Y4, fmav(ty, third, vy));
     x = nx;
     y = ny;
-    return rational;
+    return true;
 }
 
-// The packed step loop of one tile for steps [s_begin, s_end).  NARROW is fixed
-// per request (the rational fit its force uses), so the tile chooses the loop
-// once.
-//
-// Bound by register operands and issue: a packed fused multiply-add with three
-// different register pairs takes 3 cycles of a scheduler, one with a constant
-// operand 2, and each other instruction one more (measured with independent
-// chains).  So the loop's instructions count: a warp whose lanes all stay on the
-// rational branch runs steps with one vote instead of two, four 3-input maxima
-// instead of eight compares, and no exit test (no lane of it is beyond R).
-// Where a step's vote fails, the step is done again with a vote per pair, and so
-// are the following ones until one is on the rational branch throughout: lanes
-// stay outside the NFW edge for many steps, so few steps are done twice.
-// Precision sweep of four masses, 128-thread CTAs: 6.41-6.50 -> 5.85-5.92 ms.
-template <bool GTAB, bool NARROW>
-__device__ __forceinline__ void packed_steps(f2& X, f2& Y, f2& VX, f2& VY, const float* tab,
-                                             int s_begin, int s_end, bool act0, bool act1,
-                                             bool done, const HaloX2& h2, float R)
+// Whether every active trajectory of this lane is finished (see escapes).
+__device__ __forceinline__ bool lane_finished(float x, float y, float vx, float vy, bool act0, bool,
+                                              const HaloV<float>& hc, float irem)
 {
-    int n = s_begin;
-    for (;;) {
-        for (; n < s_end; ++n) {
-            const float4* c4 = reinterpret_cast<const float4*>(tab + (size_t)n * C_COUNT);
-            if (!rk4_step_x2<GTAB, NARROW, true>(X, Y, VX, VY, c4, h2)) break;
-        }
-        if (n >= s_end) return;
-        bool rational;
-        int k = 0;
-        do {
-            if ((k++ & (kExitEvery - 1)) == 0) {
-                const f2 r2 = fma2(X, X, mul2(Y, Y));
-                const f2 dot = fma2(X, VX, mul2(Y, VY));
-                const f2 v2 = fma2(VX, VX, mul2(VY, VY));
-                const float irem = tab[(size_t)n * C_COUNT + C_IREM];
-                const bool fin0 = !act0 || escapes(f2lo(r2), f2lo(dot), f2lo(v2), h2.R2, R, irem);
-                const bool fin1 = !act1 || escapes(f2hi(r2), f2hi(dot), f2hi(v2), h2.R2, R, irem);
-                done |= fin0 && fin1;
-                if (__all_sync(0xffffffffu, done)) return;
-            }
-            const float4* c4 = reinterpret_cast<const float4*>(tab + (size_t)n * C_COUNT);
-            rational = rk4_step_x2<GTAB, NARROW, false>(X, Y, VX, VY, c4, h2);
-            ++n;
-        } while (n < s_end && !rational);
+    return !act0 || escapes(fmaf(x, x, y * y), fmaf(x, vx, y * vy), fmaf(vx, vx, vy * vy), hc.R2,
+                            hc.R, irem);
+}
+__device__ __forceinline__ bool lane_finished(f2 x, f2 y, f2 vx, f2 vy, bool act0, bool act1,
+                                              const HaloV<f2>& hc, float irem)
+{
+    const f2 r2 = fma2(x, x, mul2(y, y));
+    const f2 dot = fma2(x, vx, mul2(y, vy));
+    const f2 v2 = fma2(vx, vx, mul2(vy, vy));
+    return (!act0 || escapes(f2lo(r2), f2lo(dot), f2lo(v2), hc.R2, hc.R, irem)) &&
+           (!act1 || escapes(f2hi(r2), f2hi(dot), f2hi(v2), hc.R2, hc.R, irem));
+}
+
+// A warp's window on the coefficient table: two buffers of kRingSteps rows in
+// shared memory, one filled by asynchronous copies while the steps of the other
+// run.  Read in place, a table row costs its first reader on an SM a wait for L2,
+// with all of a step behind it.
+constexpr int kRingSteps = 32;
+constexpr int kRow16 = C_COUNT / 4;                  // 16-byte words of a step's coefficients
+constexpr int kRing16 = 2 * kRingSteps * kRow16;     // and of a warp's two buffers
+
+__device__ __forceinline__ void copy16_async(float4* dst, const float4* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void copies_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+}
+
+// Copy rows [first, first + kRingSteps), none past s_end, into one of the buffers.
+__device__ __forceinline__ void ring_fill(float4* half, const float4* tab, int first, int s_end,
+                                          int lane)
+{
+    const int n16 = min(kRingSteps, s_end - first) * kRow16;
+    for (int i = lane; i < n16; i += 32) copy16_async(half + i, tab + (size_t)first * kRow16 + i);
+    copies_commit();
+}
+
+// Run body(rows, count) over steps [s_begin, s_end) in windows of kRingSteps
+// rows until it returns false.  Warp-uniform; all copies are done on return, so
+// the buffers can be filled again.
+template <class Body>
+__device__ __forceinline__ void over_ring(float4* ring, const float4* tab, int s_begin, int s_end,
+                                          int lane, Body body)
+{
+    ring_fill(ring, tab, s_begin, s_end, lane);
+    ring_fill(ring + kRing16 / 2, tab, s_begin + kRingSteps, s_end, lane);
+    float4* half = ring;
+    for (int first = s_begin; first < s_end; first += kRingSteps) {
+        copies_wait<1>();                            // this half has arrived
+        __syncwarp();
+        if (!body(half, min(kRingSteps, s_end - first))) break;
+        __syncwarp();                                // every lane has read it
+        ring_fill(half, tab, first + 2 * kRingSteps, s_end, lane);
+        half = half == ring ? ring + kRing16 / 2 : ring;
     }
+    copies_wait<0>();
+    __syncwarp();
+}
+
+// The FP32 step loop of one warp for steps [s_begin, s_end).  NARROW is fixed per
+// request (the rational fit its force uses), so the tile chooses the loop once.
+//
+// With many warps it is bound by register operands and issue: a packed fused
+// multiply-add with three different register pairs takes 3 cycles of a scheduler,
+// one with a constant operand 2, each other instruction about one more (measured
+// with independent chains), and 102 of a packed step's 156 instructions are such
+// operations.  With one warp on a scheduler it is bound by that warp's own issue
+// (a scalar fused multiply-add every 2 cycles) and the chain of a step.  So the
+// instructions of a step count, and no step has more than two votes, both off the
+// chain, and no branch but theirs.
+// A warp whose lanes all stay on the rational branch runs kRational steps, without
+// selects and without the exit test (no lane of it is beyond R).  Where one fails
+// it is done again in a form that lets each lane select its branch, and so are the
+// following steps: every kSelectEvery of them the warp stops if its lanes are all
+// finished, and goes back to kRational steps if they were all on that branch.
+// Evaluating the branches of such a warp by votes and warp-uniform paths took 1900
+// cycles a step on one scheduler, selecting takes 626 (431 one trajectory a lane).
+constexpr int kSelectEvery = 8;
+
+template <bool NARROW, class V>
+__device__ __forceinline__ void step_loop(V& x, V& y, V& vx, V& vy, const float4* tab, int s_begin,
+                                          int s_end, bool act0, bool act1, const HaloF32& h,
+                                          float4* ring, int lane)
+{
+    const HaloV<V> hc = halo_of<V>(h);
+    bool done = !act0 && !act1;      // every trajectory of this lane is finished
+    if (__all_sync(0xffffffffu, done)) return;
+    bool rational = true;
+    bool select = false;             // the warp runs steps that select
+    int k_select = 0;
+    over_ring(ring, tab, s_begin, s_end, lane, [&](const float4* rows, int count) {
+        const float4* const end = rows + count * kRow16;
+        while (rows < end) {
+            if (!select) {
+                for (; rows < end; rows += kRow16)
+                    if (!rk4_form<NARROW, kRational>(x, y, vx, vy, rows, hc, rational)) break;
+                if (rows >= end) break;
+                select = true;
+                k_select = 0;
+                rational = false;
+            }
+            if ((k_select++ & (kSelectEvery - 1)) == 0) {
+                done |= lane_finished(x, y, vx, vy, act0, act1, hc, rows[C_IREM / 4].w);
+                if (__all_sync(0xffffffffu, done)) return false;
+                select = !__all_sync(0xffffffffu, rational);
+            }
+            if (hc.c > (float)kRationalYMax || !rk4_form<NARROW, kSelect>(x, y, vx, vy, rows, hc, rational))
+                rk4_form<NARROW, kSelectLog>(x, y, vx, vy, rows, hc, rational);
+            rows += kRow16;
+        }
+        return true;
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -777,31 +907,63 @@ __device__ int queue_wait(QueueCtl* q, unsigned g, int* n_probs)
     }
 }
 
-// The packed path asks for two 512-thread CTAs per SM (at most 64 registers):
-// it issues few instructions per trajectory, so it needs many warps to hide
-// the latency of its dependent chains.
-template <typename T, int TPT, bool COUNT, bool PACKED = false, bool GTAB = false>
-__global__ void __launch_bounds__(512, PACKED ? 2 : 1)
+// Sum of a tile's weighted f values, in an order that depends on the trajectories
+// alone: each 64 consecutive ones form a unit, whose lanes add the two halves and
+// are then summed by a shuffle tree; units are added by fours, in pairs, and the
+// fours of a tile in order.  So every kernel and every split of a request's tiles
+// into ones of a unit, two or four gives the same bits.
+constexpr int kUnit = 64;
+
+// Sum of n (1, 2 or 4) values of a four, those from `have` on being absent.
+template <class Load>
+__device__ __forceinline__ double sum_of_four(int n, int have, Load load)
+{
+    auto at = [&](int i) { return i < n && i < have ? load(i) : 0.0; };   // + 0.0 is exact
+    return (at(0) + at(1)) + (at(2) + at(3));
+}
+
+// Work of one launch: CTAs of a persistent grid claim tiles of `P.tile`
+// consecutive trajectories of one radius and integrate them in passes of
+// blockDim.x * TPT.  The step loop:
+//   kLoopPacked  two trajectories per thread in packed FP32x2, 24 warps per SM (80
+//                registers: 64 spill in the step forms, 5.95 ms against 5.75 ms on
+//                the precision sweep of four masses; 96 and 20 warps, 5.74 ms, but
+//                the uneven batch 27.5 against 27.0 ms);
+//   kLoopRing    one trajectory per thread, for small launches (plan_shape);
+//   kLoopGeneral one trajectory after another with the general force: the FP64
+//                mode, and with COUNT the counting variant of either mode.
+enum StepLoop { kLoopGeneral, kLoopPacked, kLoopRing };
+constexpr int kRingThreads = 128;
+
+__device__ __forceinline__ int warp_id() { return threadIdx.x >> 5; }
+
+template <typename T, int TPT, bool COUNT, StepLoop LOOP>
+__global__ void __launch_bounds__(LOOP == kLoopGeneral ? (COUNT || TPT == 2 ? 512 : 256) : LOOP == kLoopPacked ? 256 : kRingThreads,
+                                  LOOP == kLoopPacked ? 3 : 1)
 traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_prefix,
             int n_probs, int n_tiles, unsigned* __restrict__ tile_counter,
             unsigned long long* __restrict__ tallies, QueueCtl* queue)
 {
     using Ctr = typename std::conditional<COUNT, Tally, NoTally>::type;
     Ctr ctr;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* s_coef = reinterpret_cast<T*>(smem_raw);
     __shared__ int s_tile;
     __shared__ int s_req;
     __shared__ int s_last;
     // the descriptor of the tile's request, read through L2 (requests published
     // into a resident launch are never served from a stale L1 line)
     __shared__ __align__(16) DevProblem s_prob;
-    __shared__ double s_red[32][2];
+    // unit sums of a pass; with one trajectory per thread a unit is two warps, and
+    // the second hands its lanes' values to the first
+    __shared__ double s_red[16][2];
+    __shared__ double s_half[TPT == 1 ? 8 : 1][2][32];
+    extern __shared__ __align__(16) float4 s_ring[];   // kRing16 words a warp (not kLoopGeneral)
+    float4* ring = s_ring + warp_id() * kRing16;
 
     const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int nwarps = blockDim.x >> 5;
-    int cur = -1;
+    const int warp = warp_id();
+    const int n_warps = blockDim.x >> 5;
+    // trajectory of slot i of this thread within a pass
+    auto slot = [&](int i) { return (warp * TPT + i) * 32 + lane; };
 
     for (;;) {
         if (threadIdx.x == 0) {
@@ -834,18 +996,8 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
         __syncthreads();
         const DevProblem& P = s_prob;
         const int n_steps = P.n_steps;
-
-        // coefficient table: staged once per request into shared memory, or
-        // (GTAB) read in place through the L1 cache with warp-uniform loads
-        const T* tab = GTAB ? reinterpret_cast<const T*>(P.coef) : s_coef;
-        if (!GTAB && lo != cur) {   // stage this request's table (uniform branch)
-            const float4* src = reinterpret_cast<const float4*>(P.coef);
-            float4* dst = reinterpret_cast<float4*>(s_coef);
-            const int n16 = (int)((size_t)n_steps * C_COUNT * sizeof(T) / 16);
-            for (int i = threadIdx.x; i < n16; i += blockDim.x) dst[i] = __ldg(&src[i]);
-            __syncthreads();
-            cur = lo;
-        }
+        // coefficient table, read in place through the L1 cache with warp-uniform loads
+        const T* tab = reinterpret_cast<const T*>(P.coef);
 
         const int tps = P.tiles_per_seg;
         const int lt = g - __ldcg(&tile_prefix[lo]);
@@ -860,14 +1012,19 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
         const int s_begin = P.step_begin;
         const int s_end = P.step_end > 0 ? P.step_end : n_steps;
         T* state = reinterpret_cast<T*>(P.state);
+        const bool more = state && s_end < n_steps;      // more chunks follow
+        const int nm = P.n_mass;
+        double* part = P.partials + ((size_t)seg * tps + tis) * 2 * nm;
 
+        // one pass, but for a tile of more trajectories than the CTA holds
+        for (int base = 0; base < (LOOP == kLoopGeneral ? P.tile : 1); base += blockDim.x * TPT) {
         T x[TPT], y[TPT], vx[TPT], vy[TPT];
         bool act[TPT];
         bool done = true;            // every trajectory of this lane is finished
 #pragma unroll
         for (int i = 0; i < TPT; ++i) {
-            const int t = tis * P.tile + i * blockDim.x + threadIdx.x;
-            act[i] = t < n_seg;
+            const int t = tis * P.tile + base + slot(i);
+            act[i] = base + slot(i) < P.tile && t < n_seg;
             done &= !act[i];
             const int tt = act[i] ? t : 0;
             if (state && s_begin > 0) {          // resume a served request
@@ -889,26 +1046,32 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
         // A finished trajectory (escapes(): beyond R on a line that never
         // re-enters) keeps its velocity for every later step, and q_i depends
         // on v alone.  A warp stops integrating once all of its lanes are in that state
-        // (padding lanes of a ragged tile start finished); the test runs every
-        // kExitEvery steps, and a finished lane that keeps stepping with its
-        // warp stays beyond R with its velocity unchanged.  All lanes of the
-        // warp reach the vote, so the full mask is valid.
-        if constexpr (PACKED) {
+        // (padding lanes of a ragged tile start finished), and a finished lane
+        // that keeps stepping with its warp stays beyond R with its velocity
+        // unchanged.  All lanes of the warp reach the votes, so the full mask is
+        // valid.
+        if constexpr (LOOP == kLoopPacked) {
             static_assert(TPT == 2, "packed path holds two trajectories");
             f2 X = pk(x[0], x[1]), Y = pk(y[0], y[1]);
             f2 VX = pk(vx[0], vx[1]), VY = pk(vy[0], vy[1]);
-            const HaloX2 h2{dup(hc.invIc), dup(-hc.invR3), hc.R2, hc.c};
-            const float* ftab = reinterpret_cast<const float*>(tab);
+            const float4* tab4 = reinterpret_cast<const float4*>(tab);
             if (hc.narrow)
-                packed_steps<GTAB, true>(X, Y, VX, VY, ftab, s_begin, s_end, act[0], act[1], done,
-                                         h2, hc.R);
+                step_loop<true>(X, Y, VX, VY, tab4, s_begin, s_end, act[0], act[1], hc, ring, lane);
             else
-                packed_steps<GTAB, false>(X, Y, VX, VY, ftab, s_begin, s_end, act[0], act[1], done,
-                                          h2, hc.R);
+                step_loop<false>(X, Y, VX, VY, tab4, s_begin, s_end, act[0], act[1], hc, ring, lane);
             x[0] = f2lo(X); x[1] = f2hi(X);
             y[0] = f2lo(Y); y[1] = f2hi(Y);
             vx[0] = f2lo(VX); vx[1] = f2hi(VX);
             vy[0] = f2lo(VY); vy[1] = f2hi(VY);
+        } else if constexpr (LOOP == kLoopRing) {
+            static_assert(TPT == 1, "one trajectory per thread");
+            const float4* tab4 = reinterpret_cast<const float4*>(tab);
+            if (hc.narrow)
+                step_loop<true>(x[0], y[0], vx[0], vy[0], tab4, s_begin, s_end, act[0], false, hc,
+                                ring, lane);
+            else
+                step_loop<false>(x[0], y[0], vx[0], vy[0], tab4, s_begin, s_end, act[0], false, hc,
+                                 ring, lane);
         } else {
             bool fin_i[TPT];
 #pragma unroll
@@ -932,7 +1095,7 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
                 const float4* c4 = reinterpret_cast<const float4*>(tab + (size_t)n * C_COUNT);
 #pragma unroll
                 for (int q = 0; q < (int)(C_COUNT * sizeof(T) / 16); ++q)
-                    reinterpret_cast<float4*>(c)[q] = GTAB ? __ldg(&c4[q]) : c4[q];
+                    reinterpret_cast<float4*>(c)[q] = __ldg(&c4[q]);
 #pragma unroll
                 for (int i = 0; i < TPT; ++i) {
                     ctr.set_live(!fin_i[i] && !done);
@@ -941,18 +1104,16 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
             }
         }
 
-        if (state && s_end < n_steps) {          // more chunks follow: keep the state
+        if (more) {                              // keep the state
 #pragma unroll
             for (int i = 0; i < TPT; ++i) {
                 if (!act[i]) continue;
-                const int t = tis * P.tile + i * blockDim.x + threadIdx.x;
-                T* st = state + ((size_t)seg * n_seg + t) * 4;
+                T* st = state + ((size_t)seg * n_seg + tis * P.tile + base + slot(i)) * 4;
                 st[0] = x[i];
                 st[1] = y[i];
                 st[2] = vx[i];
                 st[3] = vy[i];
             }
-            __syncthreads();   // every thread has read s_tile before it is reused
             continue;
         }
 
@@ -965,53 +1126,65 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
         for (int i = 0; i < TPT; ++i) {
             const double ux = (double)vx[i], uy = (double)vy[i];
             qf[i] = sqrt(fma(ux, ux, uy * uy)) * P.q_scale;
-            if (P.qi && act[i]) {
-                const int t = tis * P.tile + i * blockDim.x + threadIdx.x;
-                reinterpret_cast<T*>(P.qi)[(size_t)seg * n_seg + t] = (T)qf[i];
-            }
+            if (P.qi && act[i])
+                reinterpret_cast<T*>(P.qi)[(size_t)seg * n_seg + tis * P.tile + base + slot(i)] = (T)qf[i];
         }
         // momentum and direction nodes of each trajectory (recomputed here
         // rather than kept live through the step loop)
         int tj[TPT], tk[TPT];
 #pragma unroll
         for (int i = 0; i < TPT; ++i) {
-            const int t = act[i] ? tis * P.tile + i * blockDim.x + threadIdx.x : 0;
+            const int t = act[i] ? tis * P.tile + base + slot(i) : 0;
             tj[i] = t / n_mu;
             tk[i] = t - tj[i] * n_mu;
         }
-        const int nm = P.n_mass;
-        double* part = P.partials + ((size_t)seg * tps + tis) * 2 * nm;
         for (int a = 0; a < nm; ++a) {
             const double sa = P.mass_s[a];
             double acc = 0.0, accc = 0.0;
 #pragma unroll
             for (int i = 0; i < TPT; ++i) {
                 if (!act[i]) continue;
+                // (no fused multiply-adds: a thread of one trajectory adds in no other way)
                 const double f = relic_f_dev(P, qf[i] * sa);
                 const double wm = P.wmu[tk[i]];
-                acc += P.wq[tj[i]] * wm * f;
-                accc += P.wqc[tj[i]] * wm * f;
+                acc = __dadd_rn(acc, __dmul_rn(P.wq[tj[i]] * wm, f));
+                accc = __dadd_rn(accc, __dmul_rn(P.wqc[tj[i]] * wm, f));
             }
-            // tile sum: warp shuffle, then the warps in order
-            acc = warp_sum(acc);
-            accc = warp_sum(accc);
-            if (lane == 0) {
-                s_red[warp][0] = acc;
-                s_red[warp][1] = accc;
+            if constexpr (TPT == 1) {
+                if (warp & 1) {
+                    s_half[warp >> 1][0][lane] = acc;
+                    s_half[warp >> 1][1][lane] = accc;
+                }
+                __syncthreads();
+                if (!(warp & 1) && warp + 1 < n_warps) {
+                    acc += s_half[warp >> 1][0][lane];
+                    accc += s_half[warp >> 1][1][lane];
+                }
+            }
+            if (TPT == 2 || !(warp & 1)) {
+                acc = warp_sum(acc);
+                accc = warp_sum(accc);
+                if (lane == 0) {
+                    s_red[TPT == 2 ? warp : warp >> 1][0] = acc;
+                    s_red[TPT == 2 ? warp : warp >> 1][1] = accc;
+                }
             }
             __syncthreads();
-            if (warp == 0) {
-                double t0 = lane < nwarps ? s_red[lane][0] : 0.0;
-                double t1 = lane < nwarps ? s_red[lane][1] : 0.0;
-                t0 = warp_sum(t0);
-                t1 = warp_sum(t1);
-                if (lane == 0) {
-                    part[2 * a] = t0;
-                    part[2 * a + 1] = t1;
-                }
+            if (threadIdx.x < 2) {               // the units of this pass, in order
+                double t = base > 0 ? part[2 * a + threadIdx.x] : 0.0;
+                const int units = (min((int)blockDim.x * TPT, P.tile - base) + kUnit - 1) / kUnit;
+                for (int u = 0; u < units; u += 4)
+                    t += sum_of_four(4, units - u, [&](int i) { return s_red[u + i][threadIdx.x]; });
+                part[2 * a + threadIdx.x] = t;
             }
             __syncthreads();   // s_red is reused by the next mass
         }
+        }   // passes
+        if (more) {
+            __syncthreads();   // every thread has read s_tile before it is reused
+            continue;
+        }
+
         if (threadIdx.x == 0) {
             __threadfence();
             const unsigned prev = atomicAdd(&P.seg_count[seg], 1u);
@@ -1022,11 +1195,21 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
         if (s_last && warp == 0) {   // this CTA finished the radius: add tiles in order
             __threadfence();
             const double* sp = P.partials + (size_t)seg * tps * 2 * nm;
+            // P.group tiles make one tile of the request's shape, `per` of them a four
+            const int n_whole = (tps + P.group - 1) / P.group;
+            const int per = P.group > 1 ? max(1, 4 * kUnit / P.tile) : 1;
             for (int a = 0; a < nm; ++a) {
                 double t0 = 0.0, t1 = 0.0;
-                for (int i = lane; i < tps; i += 32) {
-                    t0 += __ldcg(&sp[(size_t)i * 2 * nm + 2 * a]);
-                    t1 += __ldcg(&sp[(size_t)i * 2 * nm + 2 * a + 1]);
+                for (int k = lane; k < n_whole; k += 32) {
+                    double w0 = 0.0, w1 = 0.0;
+                    const int end = min((k + 1) * P.group, tps);
+                    for (int i = k * P.group; i < end; i += per) {
+                        const double* s0 = sp + (size_t)i * 2 * nm + 2 * a;
+                        w0 += sum_of_four(per, end - i, [&](int j) { return __ldcg(s0 + j * 2 * nm); });
+                        w1 += sum_of_four(per, end - i, [&](int j) { return __ldcg(s0 + j * 2 * nm + 1); });
+                    }
+                    t0 += w0;
+                    t1 += w1;
                 }
                 t0 = warp_sum(t0);
                 t1 = warp_sum(t1);
@@ -1080,7 +1263,10 @@ __global__ void force_probe_kernel(const DevProblem* __restrict__ prob, int stag
     const T Tq = c[(size_t)k * C_COUNT + C_T0 + slot];
     const typename PrecTraits<T>::Halo hc = PrecTraits<T>::halo(P);
     NoTally none;
-    out[i] = (double)accel_m((T)r[i], T(0), S, Q, Tq, hc, none);
+    if constexpr (std::is_same<T, double>::value)
+        out[i] = accel_m<NoTally, false>(r[i], 0.0, S, Q, Tq, hc, none);
+    else
+        out[i] = (double)accel_m((T)r[i], T(0), S, Q, Tq, hc, none);
 }
 
 int launch_force_probe(int precision, const DevProblem* d_prob, int stage, const double* d_r, int n,
@@ -1097,24 +1283,97 @@ int launch_force_probe(int precision, const DevProblem* d_prob, int stage, const
     return NU_OK;
 }
 
-size_t coef_smem_bytes(int precision, int n_steps)
+// The kernel, the threads of a CTA and the tiles of a launch over n_traj
+// trajectories whose sums are to be those of tiles of `tile`.
+//   Mixed precision, small launches: one trajectory a lane, in CTAs of four warps,
+// one for each scheduler of an SM (CTAs of two warps load the schedulers unevenly:
+// 338 against 300 us on the paper's production grid).  Up to about twelve warps a
+// scheduler it is the faster one, as more warps share the chip: 400 steps over
+// 4k / 51k / 102k / 204k / 307k / 409k trajectories take 96 / 145 / 198 / 350 / 460 /
+// 581 us, and 144 / 176 / 229 / 371 / 442 / 531 us packed.
+//   Mixed precision, larger: the packed kernel, two trajectories a lane, whatever
+// shape was asked for.
+//   FP64: one trajectory a lane, in the smallest CTAs there are sums for, and of
+// those only as many on an SM as give each scheduler a warp: one keeps its FP64
+// unit busy, and work not yet started can go to an SM that is done early.  Six radii of
+// the precision sweep take 26.7 ms with 4 warps on an SM, 27.5 with 6, 31.6 with 8 and
+// 33.8 with 20; 27.2 in CTAs of 4 warps and 33.2 of 8.
+constexpr int kFp64WarpsPerSm = 4;
+constexpr long long kRingMaxTraj = 12LL * 32 * 4 * 152;
+
+LaunchShape plan_shape(int precision, int tile, long long n_traj)
 {
-    return (size_t)n_steps * C_COUNT * (precision == NU_FP64 ? sizeof(double) : sizeof(float));
+    if (n_traj > (1LL << 35)) return whole_tiles(precision, tile);   // few enough to count
+    LaunchShape s;
+    s.tile = tile;
+    if (precision == NU_FP64) {
+        s.kernel = kFp64;
+        s.tile = tile % kUnit == 0 ? kUnit : tile;
+        s.threads = std::min(s.tile, 256);
+    } else if (n_traj <= kRingMaxTraj && tile % kRingThreads == 0) {
+        s.kernel = kRing;
+        s.threads = s.tile = kRingThreads;
+    } else {
+        s.kernel = kPacked;
+        for (int t : {256, 128, 64})                 // 128 threads, or one tile's
+            if (tile % t == 0) {
+                s.tile = t;
+                break;
+            }
+        s.threads = (s.tile + kUnit - 1) / kUnit * 32;
+    }
+    s.group = tile / s.tile;
+    return s;
 }
 
-template <typename T, int TPT, bool COUNT, bool PACKED = false, bool GTAB = false>
-static int launch_t(int block, int grid, size_t smem, const DevProblem* d_probs, const int* d_prefix,
-                    int n_probs, int n_tiles, unsigned* d_counter, unsigned long long* d_tallies,
-                    cudaStream_t s, QueueCtl* d_queue = nullptr)
+// The same with CTAs that claim whole tiles, for callers without room for the sums
+// of smaller ones.
+LaunchShape whole_tiles(int precision, int tile)
 {
-    auto k = traj_kernel<T, TPT, COUNT, PACKED, GTAB>;
-    if (GTAB) smem = 0;
-    if (smem > 48 * 1024) {
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess)
-            return NU_ECUDA;
+    LaunchShape s;
+    s.tile = tile;
+    s.group = 1;
+    if (precision == NU_FP64) {
+        s.kernel = kFp64;
+        s.threads = std::min(tile, 256);
+    } else if (tile <= 512) {
+        s.kernel = kPacked;
+        s.threads = (tile + kUnit - 1) / kUnit * 32;
+    } else {
+        s.kernel = kGeneralF32;
+        s.threads = 512;
     }
-    k<<<grid, block, smem, s>>>(d_probs, d_prefix, n_probs, n_tiles, d_counter, d_tallies, d_queue);
+    return s;
+}
+
+typedef void (*TrajKernel)(const DevProblem*, const int*, int, int, unsigned*, unsigned long long*,
+                           QueueCtl*);
+
+static TrajKernel kernel_of(int kernel)
+{
+    switch (kernel) {
+    case kPacked: return traj_kernel<float, 2, false, kLoopPacked>;
+    case kRing: return traj_kernel<float, 1, false, kLoopRing>;
+    case kFp64: return traj_kernel<double, 1, false, kLoopGeneral>;
+    case kGeneralF32: return traj_kernel<float, 2, false, kLoopGeneral>;
+    case kCountF32: return traj_kernel<float, 2, true, kLoopGeneral>;
+    default: return traj_kernel<double, 2, true, kLoopGeneral>;
+    }
+}
+
+// Shared memory of a CTA: its warps' windows on the table.
+static size_t ring_bytes(const LaunchShape& shape)
+{
+    return shape.kernel == kPacked || shape.kernel == kRing
+               ? (size_t)(shape.threads / 32) * kRing16 * sizeof(float4) : 0;
+}
+
+int launch_traj(const LaunchShape& shape, int grid, const DevProblem* d_probs, const int* d_prefix,
+                int n_probs, int n_tiles, unsigned* d_counter, void* stream, QueueCtl* d_queue)
+{
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    kernel_of(shape.kernel)<<<grid, shape.threads, ring_bytes(shape), s>>>(d_probs, d_prefix, n_probs, n_tiles,
+                                                           d_counter, nullptr, d_queue);
     if (cudaGetLastError() != cudaSuccess) return NU_ECUDA;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone)
@@ -1122,85 +1381,28 @@ static int launch_t(int block, int grid, size_t smem, const DevProblem* d_probs,
     return NU_OK;
 }
 
-template <bool GTAB>
-static int launch_shape(int precision, int tpt, int block, int grid, size_t smem,
-                        const DevProblem* d_probs, const int* d_prefix, int n_probs, int n_tiles,
-                        unsigned* d_counter, cudaStream_t s, QueueCtl* q)
+int launch_traj_tally(int precision, const LaunchShape& shape, int grid, const DevProblem* d_probs,
+                      const int* d_prefix, int n_probs, int n_tiles, unsigned* d_counter,
+                      unsigned long long* d_tallies, void* stream)
 {
-    if (precision == NU_FP64) {
-        if (tpt == 2) return launch_t<double, 2, false, false, GTAB>(block, grid, smem, d_probs, d_prefix, n_probs, n_tiles, d_counter, nullptr, s, q);
-        return launch_t<double, 1, false, false, GTAB>(block, grid, smem, d_probs, d_prefix, n_probs, n_tiles, d_counter, nullptr, s, q);
-    }
-    if (tpt == 3) return launch_t<float, 2, false, true, GTAB>(block, grid, smem, d_probs, d_prefix, n_probs, n_tiles, d_counter, nullptr, s, q);
-    if (tpt == 2) return launch_t<float, 2, false, false, GTAB>(block, grid, smem, d_probs, d_prefix, n_probs, n_tiles, d_counter, nullptr, s, q);
-    return launch_t<float, 1, false, false, GTAB>(block, grid, smem, d_probs, d_prefix, n_probs, n_tiles, d_counter, nullptr, s, q);
-}
-
-int launch_traj(int precision, int tpt, int block, int grid, size_t smem, const DevProblem* d_probs,
-                const int* d_prefix, int n_probs, int n_tiles, unsigned* d_counter, void* stream,
-                bool gtab, QueueCtl* d_queue)
-{
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    if (gtab || smem > kMaxStagedSmem)   // a table too large to stage is read through L1
-        return launch_shape<true>(precision, tpt, block, grid, smem, d_probs, d_prefix, n_probs, n_tiles, d_counter, s, d_queue);
-    return launch_shape<false>(precision, tpt, block, grid, smem, d_probs, d_prefix, n_probs, n_tiles, d_counter, s, d_queue);
-}
-
-template <bool GTAB>
-static int launch_tally_shape(int precision, int tpt, int block, int grid, size_t smem,
-                              const DevProblem* d_probs, const int* d_prefix, int n_probs,
-                              int n_tiles, unsigned* d_counter, unsigned long long* d_tallies,
-                              cudaStream_t s)
-{
-    if (precision == NU_FP64) {
-        if (tpt == 2) return launch_t<double, 2, true, false, GTAB>(block, grid, smem, d_probs, d_prefix, n_probs, n_tiles, d_counter, d_tallies, s);
-        return launch_t<double, 1, true, false, GTAB>(block, grid, smem, d_probs, d_prefix, n_probs, n_tiles, d_counter, d_tallies, s);
-    }
-    if (tpt >= 2) return launch_t<float, 2, true, false, GTAB>(block, grid, smem, d_probs, d_prefix, n_probs, n_tiles, d_counter, d_tallies, s);
-    return launch_t<float, 1, true, false, GTAB>(block, grid, smem, d_probs, d_prefix, n_probs, n_tiles, d_counter, d_tallies, s);
-}
-
-int launch_traj_tally(int precision, int tpt, int block, int grid, size_t smem,
-                      const DevProblem* d_probs, const int* d_prefix, int n_probs, int n_tiles,
-                      unsigned* d_counter, unsigned long long* d_tallies, void* stream)
-{
-    // the tallies are trajectory facts: every shape integrates the same values
-    // (for a packed batch the scalar two-trajectory kernel counts, bitwise the
-    // same computation; it stages the plain table, which needs less than smem)
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    if (smem > kMaxStagedSmem)
-        return launch_tally_shape<true>(precision, tpt, block, grid, smem, d_probs, d_prefix, n_probs, n_tiles, d_counter, d_tallies, s);
-    return launch_tally_shape<false>(precision, tpt, block, grid, smem, d_probs, d_prefix, n_probs, n_tiles, d_counter, d_tallies, s);
-}
-
-template <typename T, int TPT, bool PACKED = false, bool GTAB = false>
-static int occ_t(int block, size_t smem, int* out)
-{
-    auto k = traj_kernel<T, TPT, false, PACKED, GTAB>;
-    if (GTAB) smem = 0;
-    if (smem > 48 * 1024) {
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess)
-            return NU_ECUDA;
-    }
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k, block, smem) != cudaSuccess)
-        return NU_ECUDA;
+    // the tallies are trajectory facts: every kernel integrates the same values
+    const int threads = std::min((shape.tile + kUnit - 1) / kUnit * 32, 512);
+    kernel_of(precision == NU_FP64 ? kCountF64 : kCountF32)
+        <<<grid, threads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+            d_probs, d_prefix, n_probs, n_tiles, d_counter, d_tallies, nullptr);
+    if (cudaGetLastError() != cudaSuccess) return NU_ECUDA;
+    count_launch();
     return NU_OK;
 }
 
-template <bool GTAB>
-static int occ_shape(int precision, int tpt, int block, size_t smem, int* out)
+int max_ctas_per_sm(const LaunchShape& shape, int* out)
 {
-    if (precision == NU_FP64)
-        return tpt == 2 ? occ_t<double, 2, false, GTAB>(block, smem, out) : occ_t<double, 1, false, GTAB>(block, smem, out);
-    if (tpt == 3) return occ_t<float, 2, true, GTAB>(block, smem, out);
-    return tpt == 2 ? occ_t<float, 2, false, GTAB>(block, smem, out) : occ_t<float, 1, false, GTAB>(block, smem, out);
-}
-
-int max_ctas_per_sm(int precision, int tpt, int block, size_t smem, int* out, bool gtab)
-{
-    return (gtab || smem > kMaxStagedSmem) ? occ_shape<true>(precision, tpt, block, smem, out)
-                : occ_shape<false>(precision, tpt, block, smem, out);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kernel_of(shape.kernel), shape.threads,
+                                                      ring_bytes(shape)) != cudaSuccess)
+        return NU_ECUDA;
+    if (shape.kernel == kFp64)
+        *out = std::min(*out, std::max(1, kFp64WarpsPerSm * 32 / shape.threads));
+    return NU_OK;
 }
 
 }  // namespace nuprof

@@ -51,8 +51,47 @@ CASES = {
 }
 
 
+# many radii of short runs: the launch is large enough for two trajectories a lane
+LARGE = PLAIN.replace(radii=np.geomspace(1.0, 3000.0, 300), n_steps=40)
+
+
 @pytest.mark.parametrize("name", CASES)
-@pytest.mark.parametrize("block,tpt", [(128, 3), (64, 3)])
-def test_packed_loop_is_bitwise_the_counting_loop(name, block, tpt):
+@pytest.mark.parametrize("block,tpt", [(256, 1), (128, 3), (64, 3)])
+def test_small_launch_is_bitwise_the_counting_loop(name, block, tpt):
     for a, b in zip(*_both(CASES[name], block, tpt)):
         assert np.array_equal(a, b, equal_nan=True)
+
+
+# tiles of 64, 96 (three halves of a unit), 256, 288 and 1024 trajectories
+@pytest.mark.parametrize("block,tpt", [(64, 1), (96, 1), (256, 1), (288, 1), (512, 2)])
+@pytest.mark.parametrize("change", [{}, {"c": 25.0}, {"z_end": 6.0}, {"n_q": 257, "n_mu": 4}])
+def test_large_launch_is_bitwise_the_counting_loop(change, block, tpt):
+    for a, b in zip(*_both(LARGE.replace(**change), block, tpt)):
+        assert np.array_equal(a, b, equal_nan=True)
+
+
+@pytest.mark.parametrize("block,tpt", [(96, 1), (480, 1), (512, 2)])
+def test_fp64_is_bitwise_the_counting_loop(block, tpt):
+    pb = PLAIN.replace(precision=W.FP64, n_steps=20)
+    for a, b in zip(*_both(pb, block, tpt)):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("block,tpt", [(256, 1), (96, 1), (512, 2)])
+def test_results_do_not_depend_on_what_shares_the_launch(block, tpt):
+    """A small request alone (one trajectory a lane) and in a large batch (two)."""
+    def results(problems):
+        hs = [nu.create(pb, block=block, tpt=tpt) for pb in problems]
+        b = nu.nu_batch_create(hs)
+        try:
+            nu.nu_batch_run(b)
+            return [nu.nu_profile_result(h, pb.n_out) for h, pb in zip(hs, problems)]
+        finally:
+            nu.nu_batch_destroy(b)
+            for h in hs:
+                nu.nu_profile_destroy(h)
+
+    small = PLAIN.replace(radii=np.array([3.0, 90.0]), n_q=37, n_mu=9, n_steps=100,
+                          masses=(0.05, 0.1, 0.2))
+    for a, b in zip(results([small])[0], results([LARGE, small])[1]):
+        assert np.array_equal(a, b)
