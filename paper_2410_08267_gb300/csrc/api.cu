@@ -405,7 +405,9 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
     h->d = d;
     h->info = info;
     h->n_radii = n_radii;
-    h->shape = plan_shape(o.precision, info.tile, info.n_traj);
+    LaunchSize size;
+    size.add(n_radii, (long long)p_grid->n_q * p_grid->n_mu);
+    h->shape = plan_shape(o.precision, info.tile, size);
     h->n_tiles = tiles_of(h->shape, (long long)p_grid->n_q * p_grid->n_mu) * n_radii;
 
     // ---- host tables (FP64) ----
@@ -713,9 +715,10 @@ int nu_batch_create(nu_profile* const* hs, int n, const nu_opts* opts, nu_batch*
     }
     if (b->tpt == kTptPacked && b->precision != NU_MIXED) return NU_EINVAL;
     const int tile = b->block * traj_per_thread(b->tpt);
-    long long n_traj = 0;
-    for (int i = 0; i < n; ++i) n_traj += hs[i]->info.n_traj;
-    b->shape = plan_shape(b->precision, tile, n_traj);
+    LaunchSize size;
+    for (int i = 0; i < n; ++i)
+        size.add(hs[i]->n_radii, (long long)hs[i]->grid.n_q * hs[i]->grid.n_mu);
+    b->shape = plan_shape(b->precision, tile, size);
     std::vector<DevProblem> descs(n);
     std::vector<int> prefix(n + 1, 0);
     long long asked = 0;

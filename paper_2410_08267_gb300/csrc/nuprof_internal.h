@@ -22,11 +22,11 @@ enum CoefSlot {
     C_MA1 = 0,   // -(h/2) A(z_a)        X2 = x + C_MA1 v
     C_MA2,       // -(h/2) A(z_m)        X3 = x + C_MA2 V2
     C_MA3,       // -h A(z_m)            X4 = x + C_MA3 V3
+    C_W0,        // -(h/6) A(z_a)        x' = x + W0 v + W1 (V2+V3) + W2 V4
     C_B1,        // (h/2) B F (z_a)      V2 = v + C_B1 m1 x
     C_B2,        // (h/2) B F (z_m)      V3 = v + C_B2 m2 X2
+    C_B4,        // (h/6) B F (z_b)      (before C_B3: pairs of stages are read as pairs)
     C_B3,        // h B F (z_m)          V4 = v + C_B3 m3 X3
-    C_B4,        // (h/6) B F (z_b)
-    C_W0,        // -(h/6) A(z_a)        x' = x + W0 v + W1 (V2+V3) + W2 V4
     C_W1,        // -(h/3) A(z_m)
     C_W2,        // -(h/6) A(z_b)
     C_S0,        // 1/((1+z_a) r_s)      NFW argument scale
@@ -172,9 +172,17 @@ struct LaunchShape {
     int tile;        // trajectories a CTA claims at a time
     int group;       // such tiles in one tile of the asked shape
 };
-LaunchShape plan_shape(int precision, int tile, long long n_traj);
+struct LaunchSize {
+    long long n_traj = 0, tiles128 = 0, tiles256 = 0;   // and tiles of 128 and of 256
+    void add(long long n_radii, long long n_seg)        // a request's radii, trajectories of one
+    {
+        n_traj += n_radii * n_seg;
+        tiles128 += n_radii * ((n_seg + 127) / 128);
+        tiles256 += n_radii * ((n_seg + 255) / 256);
+    }
+};
+LaunchShape plan_shape(int precision, int tile, const LaunchSize& size);
 LaunchShape whole_tiles(int precision, int tile);
-constexpr long long kLargeLaunch = 1LL << 34;   // n_traj of a launch of unknown size
 // Tiles of one radius with n_seg trajectories.
 inline int tiles_of(const LaunchShape& s, long long n_seg)
 {

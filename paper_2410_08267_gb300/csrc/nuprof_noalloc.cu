@@ -129,9 +129,11 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
     const size_t o_out = carve((size_t)n_radii * sizeof(double));
     const size_t o_err = carve((size_t)n_radii * sizeof(double));
     const size_t o_part = off;
+    LaunchSize size;
+    size.add(n_radii, seg);
     for (bool whole : {false, true}) {
         shape = whole ? whole_tiles(o.precision, o.block * o.tpt)
-                      : plan_shape(o.precision, o.block * o.tpt, seg * n_radii);
+                      : plan_shape(o.precision, o.block * o.tpt, size);
         const long long tiles = (seg + shape.tile - 1) / shape.tile * n_radii;
         if (tiles > (1LL << 30)) continue;
         n_tiles = (int)tiles;

@@ -395,9 +395,14 @@ void nu_server::run()
         double traj_active = 0.0;
         for (const Active& a : active) traj_active += (double)profile_n_traj(a.h);
         int chunk = o.chunk_steps;
-        // (requests may join a resident launch later, so its size is not known)
-        const LaunchShape shape = plan_shape(o.precision, tile, o.resident ? kLargeLaunch
-                                                                          : (long long)traj_active);
+        LaunchSize size;
+        for (const Active& a : active) {
+            const DevProblem& d = profile_desc(a.h);
+            size.add(d.n_radii, (long long)d.n_q * d.n_mu);
+        }
+        // (requests may join a resident launch later: it is taken to fill the chip)
+        if (o.resident) size.tiles256 = std::max(size.tiles256, 1LL << 20);
+        const LaunchShape shape = plan_shape(o.precision, tile, size);
         if (chunk > 0 && traj_active * chunk > o.step_budget)
             chunk = std::max(1, (int)(o.step_budget / traj_active));
         std::vector<DevProblem> desc(active.size());

@@ -536,55 +536,18 @@ __device__ __forceinline__ float max3_nan(float a, float b, float c)
     return r;
 }
 
-// The operations of a step for one trajectory (float) and for two (f2): the same
-// roundings, so both forms of the step below give a trajectory the same bits.
-__device__ __forceinline__ float fmav(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ f2 fmav(f2 a, f2 b, f2 c) { return fma2(a, b, c); }
-__device__ __forceinline__ float mulv(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ f2 mulv(f2 a, f2 b) { return mul2(a, b); }
-__device__ __forceinline__ float addv(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ f2 addv(f2 a, f2 b) { return add2(a, b); }
-__device__ __forceinline__ float rsqrtv(float a) { return rsqrt_approx(a); }
-__device__ __forceinline__ f2 rsqrtv(f2 a) { return pk(rsqrt_approx(f2lo(a)), rsqrt_approx(f2hi(a))); }
-__device__ __forceinline__ float rcpv(float a) { return rcp_approx(a); }
-__device__ __forceinline__ f2 rcpv(f2 a) { return pk(rcp_approx(f2lo(a)), rcp_approx(f2hi(a))); }
-__device__ __forceinline__ float rcp_negv(float a) { return rcp_approx(-a); }
-__device__ __forceinline__ f2 rcp_negv(f2 a) { return pk(rcp_approx(-f2lo(a)), rcp_approx(-f2hi(a))); }
-__device__ __forceinline__ float lg2v(float a) { return lg2_approx(a); }
-__device__ __forceinline__ f2 lg2v(f2 a) { return pk(lg2_approx(f2lo(a)), lg2_approx(f2hi(a))); }
-template <class V> __device__ __forceinline__ V splat(float a);
-template <> __device__ __forceinline__ float splat<float>(float a) { return a; }
-template <> __device__ __forceinline__ f2 splat<f2>(float a) { return dup(a); }
-// largest of all values, NaN if one of them is NaN
-__device__ __forceinline__ float max_nan(float a) { return a; }
-__device__ __forceinline__ float max_nan(f2 a) { return max3_nan(f2lo(a), f2hi(a), f2hi(a)); }
-__device__ __forceinline__ float max_nan(float a, float b, float c, float d)
-{
-    return max3_nan(max3_nan(a, b, c), d, d);
-}
-__device__ __forceinline__ float max_nan(f2 a, f2 b, f2 c, f2 d)
-{
-    const float m = max3_nan(f2lo(a), f2hi(a), f2lo(b)), n = max3_nan(f2hi(b), f2lo(c), f2hi(c));
-    return max3_nan(max3_nan(m, n, f2lo(d)), f2hi(d), f2hi(d));
-}
+__device__ __forceinline__ f2 rsqrt2(f2 a) { return pk(rsqrt_approx(f2lo(a)), rsqrt_approx(f2hi(a))); }
+__device__ __forceinline__ f2 rcp2(f2 a) { return pk(rcp_approx(f2lo(a)), rcp_approx(f2hi(a))); }
+__device__ __forceinline__ f2 rcp_neg2(f2 a) { return pk(rcp_approx(-f2lo(a)), rcp_approx(-f2hi(a))); }
+__device__ __forceinline__ f2 lg2_2(f2 a) { return pk(lg2_approx(f2lo(a)), lg2_approx(f2hi(a))); }
 
-template <class V>
-struct HaloV {
-    V invIc, neg_invR3;
+struct HaloX2 {
+    f2 invIc, neg_invR3;
     float R2, R, c;
 };
-template <class V>
-__device__ __forceinline__ HaloV<V> halo_of(const HaloF32& h)
-{
-    return {splat<V>(h.invIc), splat<V>(-h.invR3), h.R2, h.R, h.c};
-}
 
-// N(y) and D(y) of the rational g (see nfw_N16, nfw_D16 and nfw_N8, nfw_D8);
-// NARROW selects the fit.
-template <bool NARROW>
-__device__ __forceinline__ float nfw_N(float y) { return NARROW ? nfw_N8(y) : nfw_N16(y); }
-template <bool NARROW>
-__device__ __forceinline__ float nfw_D(float y) { return NARROW ? nfw_D8(y) : nfw_D16(y); }
+// N(y) and D(y) of the rational g for both halves (see nfw_N16, nfw_D16 and nfw_N8,
+// nfw_D8); NARROW selects the fit.
 template <bool NARROW>
 __device__ __forceinline__ f2 nfw_N(f2 y)
 {
@@ -625,129 +588,181 @@ __device__ __forceinline__ f2 nfw_D(f2 y)
     return p;
 }
 
-// One force evaluation: accel_m (FP32) without branches.
+// Two force evaluations, one in each half of the pairs: accel_m (FP32) without
+// branches, from r^2 on.
 //   kRational   the value on the rational branch of the NFW part
-//   kSelect     each lane's own branch, but not the logarithm; `logarithm` is set
-//               where a lane is on it
-//   kSelectLog  each lane's own branch
+//   kSelect     each half's own branch, where none is the logarithm: the bounds Yq
+//               are c then, so no y lies between them and c
+//   kSelectLog  each half's own branch
 enum StepForm { kRational, kSelect, kSelectLog };
 
 template <StepForm FORM>
 __device__ __forceinline__ float branch_of(float r2, float ys, float Yq, float R2, float c, float mq,
-                                           float ml, float ms, bool& logarithm)
+                                           float ml, float ms)
 {
-    const bool in = r2 < R2, nfw = ys < c;
-    if constexpr (FORM == kSelect) logarithm |= in && nfw && !(ys < Yq);
-    const float mn = FORM == kSelectLog && nfw ? ml : ms;
-    return ys < Yq ? mq : in ? mn : 0.0f;
-}
-template <StepForm FORM>
-__device__ __forceinline__ f2 branch_of(f2 r2, f2 ys, float Yq, float R2, float c, f2 mq, f2 ml, f2 ms,
-                                        bool& logarithm)
-{
-    return pk(branch_of<FORM>(f2lo(r2), f2lo(ys), Yq, R2, c, f2lo(mq), f2lo(ml), f2lo(ms), logarithm),
-              branch_of<FORM>(f2hi(r2), f2hi(ys), Yq, R2, c, f2hi(mq), f2hi(ml), f2hi(ms), logarithm));
+    const float mn = FORM == kSelectLog && ys < c ? ml : ms;
+    return ys < Yq ? mq : r2 < R2 ? mn : 0.0f;
 }
 
-template <bool NARROW, StepForm FORM, class V>
-__device__ __forceinline__ V m_form(V x, V y, V S, float Yq, V T, const HaloV<V>& hc, V& ys,
-                                    bool& logarithm)
+template <bool NARROW, StepForm FORM>
+__device__ __forceinline__ f2 m_form(f2 r2, f2 S, float Yq0, float Yq1, f2 T, const HaloX2& hc, f2& ys)
 {
-    const V r2 = fmav(x, x, fmav(y, y, splat<V>(kR2Guard)));
-    const V rinv = rsqrtv(r2);
-    const V rs = mulv(rinv, S);
-    ys = mulv(r2, rs);
-    const V mq = fmav(mulv(nfw_N<NARROW>(ys), mulv(rs, T)), rcpv(nfw_D<NARROW>(ys)), hc.neg_invR3);
+    const f2 rinv = rsqrt2(r2);
+    const f2 rs = mul2(rinv, S);
+    ys = mul2(r2, rs);
+    const f2 mq = fma2(mul2(nfw_N<NARROW>(ys), mul2(rs, T)), rcp2(nfw_D<NARROW>(ys)), hc.neg_invR3);
     if constexpr (FORM == kRational) return mq;
-    const V rinv2 = mulv(rinv, rinv);
-    const V ms = fmav(rinv2, rinv, hc.neg_invR3);
-    V ml = ms;
+    const f2 rinv2 = mul2(rinv, rinv);
+    const f2 ms = fma2(rinv2, rinv, hc.neg_invR3);
+    f2 ml = ms;
     if constexpr (FORM == kSelectLog) {
-        const V u = fmav(r2, rs, splat<V>(1.0f));
-        const V I = fmav(lg2v(u), splat<V>(0.693147180559945309f), mulv(ys, rcp_negv(u)));
-        ml = fmav(mulv(I, hc.invIc), mulv(rinv2, rinv), hc.neg_invR3);
+        const f2 u = fma2(r2, rs, dup(1.0f));
+        const f2 I = fma2(lg2_2(u), dup(0.693147180559945309f), mul2(ys, rcp_neg2(u)));
+        ml = fma2(mul2(I, hc.invIc), mul2(rinv2, rinv), hc.neg_invR3);
     }
-    return branch_of<FORM>(r2, ys, Yq, hc.R2, hc.c, mq, ml, ms, logarithm);
+    return pk(branch_of<FORM>(f2lo(r2), f2lo(ys), Yq0, hc.R2, hc.c, f2lo(mq), f2lo(ml), f2lo(ms)),
+              branch_of<FORM>(f2hi(r2), f2hi(ys), Yq1, hc.R2, hc.c, f2hi(mq), f2hi(ml), f2hi(ms)));
 }
 
-// One RK4 step: every value is formed by the operations of rk4_step.  The four
-// force evaluations run as two independent pairs: within a step the positions of
-// the first two stages depend only on its start state, and those of the last two
-// on it and the first pair's forces.
-// kRational and kSelect return false and leave the state as it was where a lane of
-// the warp is on another branch (kRational) or on the logarithm (kSelect), found
-// out with one vote near the step's end.  For kRational the bounds of the four
-// evaluations do not rise from stage to stage (S falls with z), so the largest y
-// against the last stage's bound decides, and a NaN (r^2 out of range, far beyond
-// R) decides against it.  `rational` says whether this lane's last evaluation was
-// on the rational branch.
-template <bool NARROW, StepForm FORM, class V>
-__device__ __forceinline__ bool rk4_form(V& x, V& y, V& vx, V& vy, const float4* row,
-                                         const HaloV<V>& hc, bool& rational)
-{
-    const float4 q0 = row[0];                        // MA1 MA2 MA3 B1
-    const V MA1 = splat<V>(q0.x), MA2 = splat<V>(q0.y), MA3 = splat<V>(q0.z), B1 = splat<V>(q0.w);
-    const V X2 = fmav(MA1, vx, x), Y2 = fmav(MA1, vy, y);
-    const float4 q2 = row[2];                        // W1 W2 S0 S1
-    const float4 q3 = row[3];                        // S2 Q0 Q1 Q2
-    const float4 q4 = row[4];                        // T0 T1 T2 IREM
-    const V S0 = splat<V>(q2.z), S1 = splat<V>(q2.w), T0 = splat<V>(q4.x), T1 = splat<V>(q4.y);
-    V y1, y2, y3, y4;
-    bool logarithm = false;
-    const V m1 = m_form<NARROW, FORM>(x, y, S0, q3.y, T0, hc, y1, logarithm);
-    const V m2 = m_form<NARROW, FORM>(X2, Y2, S1, q3.z, T1, hc, y2, logarithm);
-    const float4 q1 = row[1];                        // B2 B3 B4 W0
-    const V p1 = mulv(B1, m1);
-    const V VX2 = fmav(p1, x, vx), VY2 = fmav(p1, y, vy);
-    const V p2 = mulv(splat<V>(q1.x), m2);
-    const V VX3 = fmav(p2, X2, vx), VY3 = fmav(p2, Y2, vy);
-    const V X3 = fmav(MA2, VX2, x), Y3 = fmav(MA2, VY2, y);
-    const V X4 = fmav(MA3, VX3, x), Y4 = fmav(MA3, VY3, y);
-
-    const V S2 = splat<V>(q3.x), T2 = splat<V>(q4.z);
-    const V m3 = m_form<NARROW, FORM>(X3, Y3, S1, q3.z, T1, hc, y3, logarithm);
-    const V m4 = m_form<NARROW, FORM>(X4, Y4, S2, q3.w, T2, hc, y4, logarithm);
-    if constexpr (FORM == kRational) {
-        if (!__all_sync(0xffffffffu, max_nan(y1, y2, y3, y4) < q3.w)) return false;
-    } else {
-        if (FORM == kSelect && __any_sync(0xffffffffu, logarithm)) return false;
-        rational = max_nan(y4) < q3.w;
+// One RK4 step of a lane's trajectories: every value is formed by the operations of
+// rk4_step.  The four force evaluations run as two independent pairs: within a step
+// the positions of the first two stages depend only on its start state, and those
+// of the last two on it and the first pair's forces.
+// A kRational step returns false and leaves the state as it was where a lane of the
+// warp is on another branch, found out with one vote near the step's end: the
+// bounds of the four evaluations do not rise from stage to stage (S falls with z),
+// so the largest y against the last stage's bound decides, and a NaN (r^2 out of
+// range, far beyond R) decides against it.  Other steps clear `rational` where this
+// lane's last evaluation was on another branch.
+//
+// Two trajectories of a lane: the halves of every pair are theirs.
+struct TwoTrajectories {
+    f2 x, y, vx, vy;
+    __device__ __forceinline__ TwoTrajectories(const float* x_, const float* y_, const float* vx_,
+                                               const float* vy_)
+        : x(pk(x_[0], x_[1])), y(pk(y_[0], y_[1])), vx(pk(vx_[0], vx_[1])), vy(pk(vy_[0], vy_[1]))
+    {
     }
+    __device__ __forceinline__ void store(float* x_, float* y_, float* vx_, float* vy_) const
+    {
+        x_[0] = f2lo(x); x_[1] = f2hi(x);
+        y_[0] = f2lo(y); y_[1] = f2hi(y);
+        vx_[0] = f2lo(vx); vx_[1] = f2hi(vx);
+        vy_[0] = f2lo(vy); vy_[1] = f2hi(vy);
+    }
+    // Whether every active trajectory of this lane is finished (see escapes).
+    __device__ __forceinline__ bool finished(const bool* act, const HaloX2& hc, float irem) const
+    {
+        const f2 r2 = fma2(x, x, mul2(y, y));
+        const f2 dot = fma2(x, vx, mul2(y, vy));
+        const f2 v2 = fma2(vx, vx, mul2(vy, vy));
+        return (!act[0] || escapes(f2lo(r2), f2lo(dot), f2lo(v2), hc.R2, hc.R, irem)) &&
+               (!act[1] || escapes(f2hi(r2), f2hi(dot), f2hi(v2), hc.R2, hc.R, irem));
+    }
+    template <bool NARROW, StepForm FORM>
+    __device__ __forceinline__ bool step(const float4* row, const HaloX2& hc, bool& rational)
+    {
+        auto r2 = [](f2 a, f2 b) { return fma2(a, a, fma2(b, b, dup(kR2Guard))); };
+        const float4 q0 = row[0];                    // MA1 MA2 MA3 W0
+        const f2 MA1 = dup(q0.x), MA2 = dup(q0.y), MA3 = dup(q0.z), W0 = dup(q0.w);
+        const f2 X2 = fma2(MA1, vx, x), Y2 = fma2(MA1, vy, y);
+        const float4 q2 = row[2];                    // W1 W2 S0 S1
+        const float4 q3 = row[3];                    // S2 Q0 Q1 Q2
+        const float4 q4 = row[4];                    // T0 T1 T2 IREM
+        const f2 S1 = dup(q2.w), T1 = dup(q4.y);
+        f2 y1, y2, y3, y4;
+        const f2 m1 = m_form<NARROW, FORM>(r2(x, y), dup(q2.z), q3.y, q3.y, dup(q4.x), hc, y1);
+        const f2 m2 = m_form<NARROW, FORM>(r2(X2, Y2), S1, q3.z, q3.z, T1, hc, y2);
+        const float4 q1 = row[1];                    // B1 B2 B4 B3
+        const f2 p1 = mul2(dup(q1.x), m1);
+        const f2 VX2 = fma2(p1, x, vx), VY2 = fma2(p1, y, vy);
+        const f2 p2 = mul2(dup(q1.y), m2);
+        const f2 VX3 = fma2(p2, X2, vx), VY3 = fma2(p2, Y2, vy);
+        const f2 X3 = fma2(MA2, VX2, x), Y3 = fma2(MA2, VY2, y);
+        const f2 X4 = fma2(MA3, VX3, x), Y4 = fma2(MA3, VY3, y);
 
-    const V B3 = splat<V>(q1.y), B4 = splat<V>(q1.z);
-    const V W0 = splat<V>(q1.w), W1 = splat<V>(q2.x), W2 = splat<V>(q2.y);
-    const V p3 = mulv(B3, m3);
-    const V VX4 = fmav(p3, X3, vx), VY4 = fmav(p3, Y3, vy);
-    const V p4 = mulv(B4, m4);
-    const V nx = fmav(W2, VX4, fmav(W1, addv(VX2, VX3), fmav(W0, vx, x)));
-    const V ny = fmav(W2, VY4, fmav(W1, addv(VY2, VY3), fmav(W0, vy, y)));
-    const V p2x2 = mulv(p2, splat<V>(2.0f));         // exact doubling
-    const V third = splat<V>(1.0f / 3.0f);
-    const V tx = fmav(p3, X3, fmav(p2x2, X2, mulv(p1, x)));
-    const V ty = fmav(p3, Y3, fmav(p2x2, Y2, mulv(p1, y)));
-    vx = fmav(p4, X4, fmav(tx, third, vx));
-    vy = fmav(p4, Y4, fmav(ty, third, vy));
-    x = nx;
-    y = ny;
-    return true;
-}
+        const f2 m3 = m_form<NARROW, FORM>(r2(X3, Y3), S1, q3.z, q3.z, T1, hc, y3);
+        const f2 m4 = m_form<NARROW, FORM>(r2(X4, Y4), dup(q3.x), q3.w, q3.w, dup(q4.z), hc, y4);
+        if constexpr (FORM == kRational) {
+            const float a = max3_nan(f2lo(y1), f2hi(y1), f2lo(y2));
+            const float b = max3_nan(f2hi(y2), f2lo(y3), f2hi(y3));
+            const float y_max = max3_nan(max3_nan(a, b, f2lo(y4)), f2hi(y4), f2hi(y4));
+            if (!__all_sync(0xffffffffu, y_max < q3.w)) return false;
+        } else {
+            rational = rational && f2lo(y4) < q3.w && f2hi(y4) < q3.w;
+        }
 
-// Whether every active trajectory of this lane is finished (see escapes).
-__device__ __forceinline__ bool lane_finished(float x, float y, float vx, float vy, bool act0, bool,
-                                              const HaloV<float>& hc, float irem)
-{
-    return !act0 || escapes(fmaf(x, x, y * y), fmaf(x, vx, y * vy), fmaf(vx, vx, vy * vy), hc.R2,
-                            hc.R, irem);
-}
-__device__ __forceinline__ bool lane_finished(f2 x, f2 y, f2 vx, f2 vy, bool act0, bool act1,
-                                              const HaloV<f2>& hc, float irem)
-{
-    const f2 r2 = fma2(x, x, mul2(y, y));
-    const f2 dot = fma2(x, vx, mul2(y, vy));
-    const f2 v2 = fma2(vx, vx, mul2(vy, vy));
-    return (!act0 || escapes(f2lo(r2), f2lo(dot), f2lo(v2), hc.R2, hc.R, irem)) &&
-           (!act1 || escapes(f2hi(r2), f2hi(dot), f2hi(v2), hc.R2, hc.R, irem));
-}
+        const f2 W1 = dup(q2.x), W2 = dup(q2.y);
+        const f2 p3 = mul2(dup(q1.w), m3);
+        const f2 VX4 = fma2(p3, X3, vx), VY4 = fma2(p3, Y3, vy);
+        const f2 p4 = mul2(dup(q1.z), m4);
+        const f2 nx = fma2(W2, VX4, fma2(W1, add2(VX2, VX3), fma2(W0, vx, x)));
+        const f2 ny = fma2(W2, VY4, fma2(W1, add2(VY2, VY3), fma2(W0, vy, y)));
+        const f2 p2x2 = mul2(p2, dup(2.0f));         // exact doubling
+        const f2 third = dup(1.0f / 3.0f);
+        const f2 tx = fma2(p3, X3, fma2(p2x2, X2, mul2(p1, x)));
+        const f2 ty = fma2(p3, Y3, fma2(p2x2, Y2, mul2(p1, y)));
+        vx = fma2(p4, X4, fma2(tx, third, vx));
+        vy = fma2(p4, Y4, fma2(ty, third, vy));
+        x = nx;
+        y = ny;
+        return true;
+    }
+};
+
+// One trajectory of a lane: the halves of a position or velocity are its x and y,
+// and those of a force evaluation the two stages of a pair (1 and 2, then 4 and 3).
+// So a step takes few more instructions than half of two trajectories' step, which
+// is what a scheduler with few warps is bound by.
+struct OneTrajectory {
+    f2 r, v;
+    __device__ __forceinline__ OneTrajectory(const float* x, const float* y, const float* vx,
+                                             const float* vy)
+        : r(pk(x[0], y[0])), v(pk(vx[0], vy[0]))
+    {
+    }
+    __device__ __forceinline__ void store(float* x, float* y, float* vx, float* vy) const
+    {
+        x[0] = f2lo(r); y[0] = f2hi(r);
+        vx[0] = f2lo(v); vy[0] = f2hi(v);
+    }
+    __device__ __forceinline__ bool finished(const bool* act, const HaloX2& hc, float irem) const
+    {
+        const float x = f2lo(r), y = f2hi(r), vx = f2lo(v), vy = f2hi(v);
+        return !act[0] || escapes(fmaf(x, x, y * y), fmaf(x, vx, y * vy), fmaf(vx, vx, vy * vy), hc.R2,
+                                  hc.R, irem);
+    }
+    template <bool NARROW, StepForm FORM>
+    __device__ __forceinline__ bool step(const float4* row, const HaloX2& hc, bool& rational)
+    {
+        auto r2 = [](f2 a, f2 b) { return pk(guarded_r2(f2lo(a), f2hi(a)), guarded_r2(f2lo(b), f2hi(b))); };
+        const float4 q0 = row[0], q1 = row[1], q2 = row[2], q3 = row[3], q4 = row[4];
+        const f2 R2 = fma2(dup(q0.x), v, r);
+        f2 y12, y43;
+        const f2 m12 = m_form<NARROW, FORM>(r2(r, R2), pk(q2.z, q2.w), q3.y, q3.z, pk(q4.x, q4.y), hc, y12);
+        const f2 p12 = mul2(pk(q1.x, q1.y), m12);
+        const f2 p1 = dup(f2lo(p12)), p2 = dup(f2hi(p12));
+        const f2 V2 = fma2(p1, r, v);
+        const f2 V3 = fma2(p2, R2, v);
+        const f2 R3 = fma2(dup(q0.y), V2, r);
+        const f2 R4 = fma2(dup(q0.z), V3, r);
+        const f2 m43 = m_form<NARROW, FORM>(r2(R4, R3), pk(q3.x, q2.w), q3.w, q3.z, pk(q4.z, q4.y), hc, y43);
+        if constexpr (FORM == kRational) {
+            const float y_max = max3_nan(max3_nan(f2lo(y12), f2hi(y12), f2lo(y43)), f2hi(y43), f2hi(y43));
+            if (!__all_sync(0xffffffffu, y_max < q3.w)) return false;
+        } else {
+            rational = rational && f2lo(y43) < q3.w;
+        }
+        const f2 p43 = mul2(pk(q1.z, q1.w), m43);
+        const f2 p3 = dup(f2hi(p43)), p4 = dup(f2lo(p43));
+        const f2 V4 = fma2(p3, R3, v);
+        const f2 nr = fma2(dup(q2.y), V4, fma2(dup(q2.x), add2(V2, V3), fma2(dup(q0.w), v, r)));
+        const f2 t = fma2(p3, R3, fma2(dup(f2hi(p12) * 2.0f), R2, mul2(p1, r)));
+        v = fma2(p4, R4, fma2(t, dup(1.0f / 3.0f), v));
+        r = nr;
+        return true;
+    }
+};
 
 // A warp's window on the coefficient table: two buffers of kRingSteps rows in
 // shared memory, one filled by asynchronous copies while the steps of the other
@@ -820,35 +835,39 @@ __device__ __forceinline__ void over_ring(float4* ring, const float4* tab, int s
 // cycles a step on one scheduler, selecting takes 626 (431 one trajectory a lane).
 constexpr int kSelectEvery = 8;
 
-template <bool NARROW, class V>
-__device__ __forceinline__ void step_loop(V& x, V& y, V& vx, V& vy, const float4* tab, int s_begin,
-                                          int s_end, bool act0, bool act1, const HaloF32& h,
-                                          float4* ring, int lane)
+template <bool NARROW, class State>
+__device__ __forceinline__ void step_loop(State& s, const float4* tab, int s_begin, int s_end,
+                                          const bool* act, bool done, const HaloX2& hc, float4* ring,
+                                          int lane)
 {
-    const HaloV<V> hc = halo_of<V>(h);
-    bool done = !act0 && !act1;      // every trajectory of this lane is finished
     if (__all_sync(0xffffffffu, done)) return;
     bool rational = true;
     bool select = false;             // the warp runs steps that select
     int k_select = 0;
     over_ring(ring, tab, s_begin, s_end, lane, [&](const float4* rows, int count) {
         const float4* const end = rows + count * kRow16;
+        // a bound below c, which comes last in the window first: c > 16, or an NFW
+        // edge that lies beyond R
+        const bool logarithm = end[3 - kRow16].w < hc.c;
         while (rows < end) {
             if (!select) {
                 for (; rows < end; rows += kRow16)
-                    if (!rk4_form<NARROW, kRational>(x, y, vx, vy, rows, hc, rational)) break;
+                    if (!s.template step<NARROW, kRational>(rows, hc, rational)) break;
                 if (rows >= end) break;
                 select = true;
                 k_select = 0;
                 rational = false;
             }
             if ((k_select++ & (kSelectEvery - 1)) == 0) {
-                done |= lane_finished(x, y, vx, vy, act0, act1, hc, rows[C_IREM / 4].w);
+                done |= s.finished(act, hc, rows[C_IREM / 4].w);
                 if (__all_sync(0xffffffffu, done)) return false;
                 select = !__all_sync(0xffffffffu, rational);
+                rational = true;
             }
-            if (hc.c > (float)kRationalYMax || !rk4_form<NARROW, kSelect>(x, y, vx, vy, rows, hc, rational))
-                rk4_form<NARROW, kSelectLog>(x, y, vx, vy, rows, hc, rational);
+            if (logarithm)
+                s.template step<NARROW, kSelectLog>(rows, hc, rational);
+            else
+                s.template step<NARROW, kSelect>(rows, hc, rational);
             rows += kRow16;
         }
         return true;
@@ -1050,28 +1069,17 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
         // that keeps stepping with its warp stays beyond R with its velocity
         // unchanged.  All lanes of the warp reach the votes, so the full mask is
         // valid.
-        if constexpr (LOOP == kLoopPacked) {
-            static_assert(TPT == 2, "packed path holds two trajectories");
-            f2 X = pk(x[0], x[1]), Y = pk(y[0], y[1]);
-            f2 VX = pk(vx[0], vx[1]), VY = pk(vy[0], vy[1]);
+        if constexpr (LOOP != kLoopGeneral) {
+            using State = typename std::conditional<LOOP == kLoopPacked, TwoTrajectories, OneTrajectory>::type;
+            static_assert(TPT == (LOOP == kLoopPacked ? 2 : 1), "trajectories of a lane");
+            const HaloX2 h2{dup(hc.invIc), dup(-hc.invR3), hc.R2, hc.R, hc.c};
             const float4* tab4 = reinterpret_cast<const float4*>(tab);
+            State st(x, y, vx, vy);
             if (hc.narrow)
-                step_loop<true>(X, Y, VX, VY, tab4, s_begin, s_end, act[0], act[1], hc, ring, lane);
+                step_loop<true>(st, tab4, s_begin, s_end, act, done, h2, ring, lane);
             else
-                step_loop<false>(X, Y, VX, VY, tab4, s_begin, s_end, act[0], act[1], hc, ring, lane);
-            x[0] = f2lo(X); x[1] = f2hi(X);
-            y[0] = f2lo(Y); y[1] = f2hi(Y);
-            vx[0] = f2lo(VX); vx[1] = f2hi(VX);
-            vy[0] = f2lo(VY); vy[1] = f2hi(VY);
-        } else if constexpr (LOOP == kLoopRing) {
-            static_assert(TPT == 1, "one trajectory per thread");
-            const float4* tab4 = reinterpret_cast<const float4*>(tab);
-            if (hc.narrow)
-                step_loop<true>(x[0], y[0], vx[0], vy[0], tab4, s_begin, s_end, act[0], false, hc,
-                                ring, lane);
-            else
-                step_loop<false>(x[0], y[0], vx[0], vy[0], tab4, s_begin, s_end, act[0], false, hc,
-                                 ring, lane);
+                step_loop<false>(st, tab4, s_begin, s_end, act, done, h2, ring, lane);
+            st.store(x, y, vx, vy);
         } else {
             bool fin_i[TPT];
 #pragma unroll
@@ -1283,44 +1291,46 @@ int launch_force_probe(int precision, const DevProblem* d_prob, int stage, const
     return NU_OK;
 }
 
-// The kernel, the threads of a CTA and the tiles of a launch over n_traj
-// trajectories whose sums are to be those of tiles of `tile`.
-//   Mixed precision, small launches: one trajectory a lane, in CTAs of four warps,
-// one for each scheduler of an SM (CTAs of two warps load the schedulers unevenly:
-// 338 against 300 us on the paper's production grid).  Up to about twelve warps a
-// scheduler it is the faster one, as more warps share the chip: 400 steps over
-// 4k / 51k / 102k / 204k / 307k / 409k trajectories take 96 / 145 / 198 / 350 / 460 /
-// 581 us, and 144 / 176 / 229 / 371 / 442 / 531 us packed.
-//   Mixed precision, larger: the packed kernel, two trajectories a lane, whatever
-// shape was asked for.
+// The kernel, the threads of a CTA and the tiles of a launch whose sums are to be
+// those of tiles of `tile`.
+//   Mixed precision: one trajectory a lane or two (packed), each in CTAs of four
+// warps, one for each scheduler of an SM.  As a CTA is one warp more on every scheduler of
+// its SM, a step of a launch that fits the chip takes the time of the SM with most CTAs:
+// with w of them, about max(440, 270 + 125 w) cycles one trajectory a lane and
+// max(500, 90 + 300 w) packed, fitted to launches of 4k to 307k trajectories (400 steps
+// over 8k / 51k / 76k / 102k / 153k / 204k / 307k: 96 / 132 / 174 / 211 / 255 / 309 / 424 us
+// and 109 / 143 / 146 / 202 / 260 / 353 / 411 us packed).  The cheaper one is taken; a
+// launch that fills the chip runs packed.
 //   FP64: one trajectory a lane, in the smallest CTAs there are sums for, and of
 // those only as many on an SM as give each scheduler a warp: one keeps its FP64
 // unit busy, and work not yet started can go to an SM that is done early.  Six radii of
 // the precision sweep take 26.7 ms with 4 warps on an SM, 27.5 with 6, 31.6 with 8 and
 // 33.8 with 20; 27.2 in CTAs of 4 warps and 33.2 of 8.
 constexpr int kFp64WarpsPerSm = 4;
-constexpr long long kRingMaxTraj = 12LL * 32 * 4 * 152;
+constexpr int kSms = 152;
+constexpr int kPackedTile = 256;
+constexpr int kPackedCtas = 6;                       // on an SM
 
-LaunchShape plan_shape(int precision, int tile, long long n_traj)
+LaunchShape plan_shape(int precision, int tile, const LaunchSize& size)
 {
-    if (n_traj > (1LL << 35)) return whole_tiles(precision, tile);   // few enough to count
+    if (size.n_traj > (1LL << 35)) return whole_tiles(precision, tile);   // few enough to count
     LaunchShape s;
     s.tile = tile;
     if (precision == NU_FP64) {
         s.kernel = kFp64;
         s.tile = tile % kUnit == 0 ? kUnit : tile;
         s.threads = std::min(s.tile, 256);
-    } else if (n_traj <= kRingMaxTraj && tile % kRingThreads == 0) {
-        s.kernel = kRing;
-        s.threads = s.tile = kRingThreads;
     } else {
-        s.kernel = kPacked;
-        for (int t : {256, 128, 64})                 // 128 threads, or one tile's
+        const long long w1 = (size.tiles128 + kSms - 1) / kSms, w2 = (size.tiles256 + kSms - 1) / kSms;
+        const bool one = tile % kRingThreads == 0 && w2 <= kPackedCtas &&
+                         std::max(440LL, 270 + 125 * w1) < std::max(500LL, 90 + 300 * w2);
+        s.kernel = one ? kRing : kPacked;
+        for (int t : {one ? kRingThreads : kPackedTile, 128, 64})
             if (tile % t == 0) {
                 s.tile = t;
                 break;
             }
-        s.threads = (s.tile + kUnit - 1) / kUnit * 32;
+        s.threads = one ? s.tile : (s.tile + kUnit - 1) / kUnit * 32;
     }
     s.group = tile / s.tile;
     return s;
