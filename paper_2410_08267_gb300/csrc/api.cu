@@ -7,6 +7,8 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <iterator>
+#include <map>
 #include <memory>
 #include <mutex>
 #include <new>
@@ -111,7 +113,8 @@ struct nu_profile {
     DevProblem hdp;                 // host copy (device pointers inside)
     DevProblem* d_prob = nullptr;
     int* d_prefix = nullptr;
-    unsigned* d_ctrl = nullptr;     // [0] tile counter, [1] status
+    unsigned* d_ctrl = nullptr;     // control words (CtrlWord)
+    double* host_out = nullptr;     // results in mapped host memory, or none
     std::shared_ptr<RunEvent> last;
     nu_profile* twin = nullptr;     // NU_FLAG_VERIFY: the same request in the FP64 mode
 };
@@ -249,16 +252,93 @@ private:
     unsigned char* p_ = nullptr;
 };
 
-// Enqueue one handle's own launch (work counter and status cleared first).
+// Page-locked, mapped host memory in which the kernel leaves results besides device
+// memory, so that reading them takes no copy (a copy of 10 values costs the
+// caller 12 us).  One block of fixed size for the process, handed out first fit and
+// given back with the handle; a handle that finds no room reads its results by a
+// copy.
+class HostResults {
+public:
+    static double* take(size_t n) noexcept
+    {
+        try {
+            return take_first_fit(n);
+        } catch (...) {                                   // no memory for the list
+            return nullptr;
+        }
+    }
+    static void give(double* ptr) noexcept                // allocates nothing
+    {
+        if (!ptr) return;
+        std::lock_guard<std::mutex> g(mu());
+        Pool& p = pool();
+        auto node = p.taken.extract((size_t)(ptr - p.base));
+        auto next = p.free.lower_bound(node.key());
+        if (next != p.free.end() && next->first == node.key() + node.mapped()) {
+            node.mapped() += next->second;
+            next = p.free.erase(next);
+        }
+        if (next != p.free.begin()) {
+            auto prev = std::prev(next);
+            if (prev->first + prev->second == node.key()) {
+                prev->second += node.mapped();
+                return;
+            }
+        }
+        p.free.insert(std::move(node));
+    }
+
+private:
+    static double* take_first_fit(size_t n)
+    {
+        std::lock_guard<std::mutex> g(mu());
+        Pool& p = pool();
+        if (!p.base) {
+            if (p.failed || cudaHostAlloc(reinterpret_cast<void**>(&p.base), kDoubles * sizeof(double),
+                                          cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+                cudaGetLastError();
+                p.base = nullptr;
+                p.failed = true;
+                return nullptr;
+            }
+            p.free[0] = kDoubles;
+        }
+        n = (n + 15) & ~(size_t)15;
+        for (auto it = p.free.begin(); it != p.free.end(); ++it) {
+            if (it->second < n) continue;
+            const size_t off = it->first, len = it->second;
+            p.taken[off] = n;
+            if (len > n) p.free[off + n] = len - n;
+            p.free.erase(off);
+            return p.base + off;
+        }
+        return nullptr;
+    }
+
+    static constexpr size_t kDoubles = (size_t)1 << 17;   // 1 MiB
+    struct Pool {
+        double* base = nullptr;
+        bool failed = false;
+        std::map<size_t, size_t> free, taken;             // offset -> length
+    };
+    static std::mutex& mu()
+    {
+        static std::mutex m;
+        return m;
+    }
+    static Pool& pool()
+    {
+        static Pool p;
+        return p;
+    }
+};
+
+// Enqueue one handle's own launch.
 int launch_profile(nu_profile* h, cudaStream_t s)
 {
     int grid = 0;
     const int rc = persistent_grid(h->shape, h->n_tiles, &grid);
     if (rc != NU_OK) return rc;
-    if (cudaMemsetAsync(h->d_ctrl, 0, 2 * sizeof(unsigned), s) != cudaSuccess) {
-        cudaGetLastError();
-        return NU_ECUDA;
-    }
     return launch_traj(h->shape, grid, h->d_prob, h->d_prefix, 1, h->n_tiles, h->d_ctrl, s);
 }
 
@@ -281,6 +361,8 @@ int staging_reserve(size_t bytes)
     { Stage st(bytes); }   // grows the buffer; its lock is released before the size is read
     return Stage::capacity() >= bytes ? NU_OK : NU_ENOMEM;
 }
+
+void host_results_reserve() { HostResults::give(HostResults::take(1)); }
 
 const DevProblem& profile_desc(const nu_profile* h) { return h->hdp; }
 nu_profile* profile_twin(const nu_profile* h) { return h->twin; }
@@ -386,6 +468,15 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
                       const double* radii, int n_radii, const nu_pgrid* p_grid,
                       const nu_opts* opts, nu_profile** out)
 {
+    return profile_create(cosmo, halo, relic, radii, n_radii, p_grid, opts, out, true);
+}
+
+}  // extern "C"
+
+int nuprof::profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic* relic,
+                           const double* radii, int n_radii, const nu_pgrid* p_grid,
+                           const nu_opts* opts, nu_profile** out, bool host_results)
+{
     if (!out) return NU_EINVAL;
     nu_opts o;
     Derived d;
@@ -412,8 +503,8 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
 
     // ---- host tables (FP64) ----
     const int nq = p_grid->n_q, nmu = p_grid->n_mu, N = o.n_steps;
-    std::vector<double> coef, q, wq, wqc, mu, wmu;
-    coef_table(*cosmo, *halo, d, N, coef);
+    std::vector<double> q, wq, wqc, mu, wmu;
+    const std::shared_ptr<const CoefTable> coef = coef_table(*cosmo, *halo, d, N);
     log_nodes(nq, p_grid->q_min, p_grid->q_max, q, wq, wqc);
     gauss_legendre(nmu, mu, wmu);
     const double kT0 = kKB * cosmo->T0_K;                 // eV
@@ -443,7 +534,7 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
     const size_t sz = fp64 ? sizeof(double) : sizeof(float);
     size_t off = 0;
     auto carve = [&](size_t bytes) { size_t at = off; off += align256(bytes); return at; };
-    const size_t o_ctrl = carve(4 * sizeof(unsigned));
+    const size_t o_ctrl = carve(kCtrlWords * sizeof(unsigned));
     const size_t o_prob = carve(sizeof(DevProblem));
     const size_t o_pref = carve(2 * sizeof(int));
     const size_t o_coef = carve((size_t)N * C_COUNT * sz);
@@ -488,8 +579,10 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
     P.seg_count = reinterpret_cast<unsigned*>(base + o_cnt);
     P.out = reinterpret_cast<double*>(base + o_out);
     P.err = reinterpret_cast<double*>(base + o_err);
+    if (host_results) h->host_out = HostResults::take((size_t)2 * nm * n_radii);
+    P.host_out = h->host_out;
     P.qi = keep_qi ? static_cast<void*>(base + o_qi) : nullptr;
-    P.status = reinterpret_cast<int*>(base + o_ctrl + sizeof(unsigned));
+    P.status = reinterpret_cast<int*>(base + o_ctrl) + kCtrlStatus;
     P.q_scale = relic->m_eV / (kC * kT0);                 // Liouville map: q_i = m |v| / (c k_B T0)
     P.invIc = 1.0 / d.Ic;
     P.invR3 = d.R > 0.0 ? 1.0 / (d.R * d.R * d.R) : 0.0;
@@ -520,13 +613,13 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
         const int prefix[2] = {0, h->n_tiles};
         std::memcpy(stage + o_pref, prefix, sizeof(prefix));
         if (fp64) {
-            put<double>(stage, o_coef, coef.data(), coef.size());
+            std::memcpy(stage + o_coef, coef->f64.data(), coef->f64.size() * sizeof(double));
             put<double>(stage, o_x0, x0.data(), n_radii);
             put<double>(stage, o_v0, v0.data(), nq);
             put<double>(stage, o_mu, mu.data(), nmu);
             put<double>(stage, o_smu, smu.data(), nmu);
         } else {
-            fp32_table(coef.data(), N, d, reinterpret_cast<float*>(stage + o_coef));
+            std::memcpy(stage + o_coef, coef->f32.data(), coef->f32.size() * sizeof(float));
             put<float>(stage, o_x0, x0.data(), n_radii);
             put<float>(stage, o_v0, v0.data(), nq);
             put<float>(stage, o_mu, mu.data(), nmu);
@@ -547,6 +640,7 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
         if (cudaMemcpyAsync(base, stage, upload_end, cudaMemcpyHostToDevice, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess) {   // the staging buffer is reused after this
             cudaGetLastError();
+            HostResults::give(h->host_out);
             h->mem.release();
             return NU_ECUDA;
         }
@@ -560,8 +654,9 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
         o2.flags = 0;
         o2.block = 256;
         o2.tpt = 1;
-        rc = nu_profile_create(cosmo, halo, relic, radii, n_radii, p_grid, &o2, &h->twin);
+        rc = profile_create(cosmo, halo, relic, radii, n_radii, p_grid, &o2, &h->twin, false);
         if (rc != NU_OK) {
+            HostResults::give(h->host_out);
             h->mem.release();
             return rc;
         }
@@ -569,6 +664,8 @@ int nu_profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic
     *out = h.release();
     return NU_OK;
 }
+
+extern "C" {
 
 int nu_profile_run(nu_profile* h, void* stream)
 {
@@ -594,6 +691,13 @@ int nu_profile_result(nu_profile* h, double* n_over_nbar, double* err_est, int n
     if (cudaEventSynchronize(h->last->ev) != cudaSuccess) {
         cudaGetLastError();
         return NU_ECUDA;
+    }
+    if (h->host_out && !h->twin) {        // the run left them in host memory
+        for (int i = 0; i < n_radii; ++i)
+            if (!std::isfinite(h->host_out[i])) return NU_EDEVICE;
+        std::memcpy(n_over_nbar, h->host_out, n_radii * sizeof(double));
+        if (err_est) std::memcpy(err_est, h->host_out + n_radii, n_radii * sizeof(double));
+        return NU_OK;
     }
     // out and err are adjacent in the device layout: one copy brings both back
     Stage staging((size_t)2 * n_radii * sizeof(double));
@@ -641,12 +745,19 @@ int nu_profile_qi(nu_profile* h, double* qi, long long n)
         }
         return NU_OK;
     }
-    std::vector<float> tmp((size_t)total);
-    if (cudaMemcpy(tmp.data(), h->hdp.qi, total * sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess) {
-        cudaGetLastError();
-        return NU_ECUDA;
+    // through the page-locked buffer a part at a time, widened from there
+    const long long part = std::min(total, 1LL << 20);
+    Stage staging((size_t)part * sizeof(float));
+    const float* tmp = reinterpret_cast<const float*>(staging.data());
+    for (long long at = 0; at < total; at += part) {
+        const long long m = std::min(part, total - at);
+        if (cudaMemcpy(staging.data(), static_cast<const float*>(h->hdp.qi) + at, m * sizeof(float),
+                       cudaMemcpyDeviceToHost) != cudaSuccess) {
+            cudaGetLastError();
+            return NU_ECUDA;
+        }
+        for (long long i = 0; i < m; ++i) qi[at + i] = tmp[i];
     }
-    for (long long i = 0; i < total; ++i) qi[i] = tmp[(size_t)i];
     return NU_OK;
 }
 
@@ -684,6 +795,7 @@ void nu_profile_destroy(nu_profile* h)
     if (h->last) cudaEventSynchronize(h->last->ev);
     h->last.reset();
     nu_profile_destroy(h->twin);
+    HostResults::give(h->host_out);
     h->mem.release();
     delete h;
 }
@@ -744,7 +856,7 @@ int nu_batch_create(nu_profile* const* hs, int n, const nu_opts* opts, nu_batch*
     }
     size_t off = 0;
     auto carve = [&](size_t bytes) { size_t at = off; off += align256(bytes); return at; };
-    const size_t o_ctrl = carve(4 * sizeof(unsigned));
+    const size_t o_ctrl = carve(kCtrlWords * sizeof(unsigned));
     const size_t o_probs = carve((size_t)n * sizeof(DevProblem));
     const size_t o_pref = carve((size_t)(n + 1) * sizeof(int));
     int rc = b->mem.allocate(off, o);
@@ -780,7 +892,6 @@ int nu_batch_create(nu_profile* const* hs, int n, const nu_opts* opts, nu_batch*
 
 static int batch_enqueue(nu_batch* b, cudaStream_t s, bool timed)
 {
-    if (cudaMemsetAsync(b->d_ctrl, 0, 2 * sizeof(unsigned), s) != cudaSuccess) return NU_ECUDA;
     if (timed && cudaEventRecord(b->t0, s) != cudaSuccess) return NU_ECUDA;
     int rc = launch_traj(b->shape, b->grid, b->d_probs, b->d_prefix, (int)b->hs.size(), b->n_tiles,
                          b->d_ctrl, s);
@@ -864,8 +975,7 @@ int nu_batch_branch_counts(nu_batch* b, void* stream, long long* counts)
     }
     unsigned long long host[kTallies] = {0, 0, 0, 0, 0, 0};
     int rc = NU_OK;
-    if (cudaMemsetAsync(b->d_tallies, 0, sizeof(host), s) != cudaSuccess ||
-        cudaMemsetAsync(b->d_ctrl, 0, 2 * sizeof(unsigned), s) != cudaSuccess)
+    if (cudaMemsetAsync(b->d_tallies, 0, sizeof(host), s) != cudaSuccess)
         rc = NU_ECUDA;
     if (rc == NU_OK)
         rc = launch_traj_tally(b->precision, b->shape, b->grid, b->d_probs, b->d_prefix,

@@ -160,15 +160,19 @@ void fp32_table(const double* tab, int n_steps, const Derived& d, float* out)
 {
     const double c = d.r_s > 0.0 ? d.r200 / d.r_s : 0.0;
     const double ymax = std::min(c, kRationalYMax);
+    for (size_t i = 0; i < (size_t)n_steps * C_COUNT; ++i) out[i] = (float)tab[i];
     for (int n = 0; n < n_steps; ++n) {
         const double* t = tab + (size_t)n * C_COUNT;
-        for (int k = 0; k < C_COUNT; ++k) {
-            double v = t[k];
-            if (k >= C_Q0 && k <= C_Q2)
-                v = std::min(ymax, (1.0 - 1e-3) * d.R * t[C_S0 + (k - C_Q0)]);
-            out[(size_t)n * C_COUNT + k] = (float)v;
-        }
+        for (int k = 0; k < 3; ++k)
+            out[(size_t)n * C_COUNT + C_Q0 + k] = (float)std::min(ymax, (1.0 - 1e-3) * d.R * t[C_S0 + k]);
     }
+}
+
+// Redshift and expansion rate of half-step k.
+static StageBackground stage_background(const nu_cosmo& cosmo, const Derived& d, double h, long k)
+{
+    const double z = std::expm1(0.5 * h * (double)k);
+    return {std::exp(0.5 * h * (double)k), z, hubble(cosmo, d, z)};
 }
 
 // Eq. eoms in u = ln a: dx/du = (1+z)^2 v / H, dv/du = -gradPhi / H with
@@ -177,13 +181,12 @@ void fp32_table(const double* tab, int n_steps, const Derived& d, float* out)
 // -(n+1) h; each is computed from the integer step index (1+z = e^{k h/2}),
 // so no time variable is ever accumulated.
 void coef_table_into(const nu_cosmo& cosmo, const nu_halo& halo, const Derived& d, int n_steps,
-                     double* tab)
+                     double* tab, const StageBackground* grid)
 {
     const double h = std::log1p(d.z_end) / n_steps;
     auto stage = [&](long k, double& A, double& BF, double& S, double& Q) {
-        const double zp1 = std::exp(0.5 * h * (double)k);
-        const double z = std::expm1(0.5 * h * (double)k);
-        const double H = hubble(cosmo, d, z);
+        const StageBackground at = grid ? grid[k] : stage_background(cosmo, d, h, k);
+        const double zp1 = at.zp1, z = at.z, H = at.H;
         A = zp1 * zp1 / H;
         const double F = kG * coupling_kappa(halo, z) * zp1 * growth_xi(halo, d, z) * halo.M_h;
         BF = F / H;
@@ -262,28 +265,60 @@ TableKey table_key(const nu_cosmo& cosmo, const nu_halo& halo, const Derived& d,
 }
 }  // namespace
 
-void coef_table(const nu_cosmo& cosmo, const nu_halo& halo, const Derived& d, int n_steps,
-                std::vector<double>& tab)
+// The halos of a scan share their background and step grid: the last few are kept
+// too (an exponential pair and a square root a stage, most of the time of a table).
+static std::shared_ptr<const std::vector<StageBackground>> background(const nu_cosmo& cosmo,
+                                                                      const Derived& d, int n_steps)
+{
+    struct Kept {
+        double Om, h, z_end;
+        int n_steps;
+        std::shared_ptr<const std::vector<StageBackground>> grid;
+    };
+    constexpr size_t kKept = 8;
+    static std::mutex mu;
+    static std::vector<Kept> kept;                       // oldest first
+    {
+        std::lock_guard<std::mutex> g(mu);
+        for (const Kept& k : kept)
+            if (k.Om == cosmo.Om && k.h == cosmo.h && k.z_end == d.z_end && k.n_steps == n_steps)
+                return k.grid;
+    }
+    auto grid = std::make_shared<std::vector<StageBackground>>((size_t)2 * n_steps + 1);
+    const double h = std::log1p(d.z_end) / n_steps;
+    for (long k = 0; k <= 2L * n_steps; ++k) (*grid)[(size_t)k] = stage_background(cosmo, d, h, k);
+    std::lock_guard<std::mutex> g(mu);
+    if (kept.size() == kKept) kept.erase(kept.begin());
+    kept.push_back({cosmo.Om, cosmo.h, d.z_end, n_steps, grid});
+    return grid;
+}
+
+std::shared_ptr<const CoefTable> coef_table(const nu_cosmo& cosmo, const nu_halo& halo,
+                                            const Derived& d, int n_steps)
 {
     constexpr size_t kKept = 8;
     static std::mutex mu;
-    static std::vector<std::pair<TableKey, std::vector<double>>> kept;   // most recent last
+    static std::vector<std::pair<TableKey, std::shared_ptr<const CoefTable>>> kept;   // most recent last
     const TableKey key = table_key(cosmo, halo, d, n_steps);
     {
         std::lock_guard<std::mutex> g(mu);
         for (size_t i = 0; i < kept.size(); ++i) {
             if (kept[i].first == key) {
-                tab = kept[i].second;
                 std::rotate(kept.begin() + i, kept.begin() + i + 1, kept.end());
-                return;
+                return kept.back().second;
             }
         }
     }
-    tab.assign((size_t)n_steps * C_COUNT, 0.0);
-    coef_table_into(cosmo, halo, d, n_steps, tab.data());
+    auto tab = std::make_shared<CoefTable>();
+    tab->f64.resize((size_t)n_steps * C_COUNT);
+    tab->f32.resize((size_t)n_steps * C_COUNT);
+    coef_table_into(cosmo, halo, d, n_steps, tab->f64.data(),
+                    background(cosmo, d, n_steps)->data());
+    fp32_table(tab->f64.data(), n_steps, d, tab->f32.data());
     std::lock_guard<std::mutex> g(mu);
     if (kept.size() == kKept) kept.erase(kept.begin());
     kept.emplace_back(key, tab);
+    return tab;
 }
 
 // |P| nodes: log-spaced on [q_min, q_max]; the integral of P^2 f dP is taken

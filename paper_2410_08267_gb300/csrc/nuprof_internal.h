@@ -3,6 +3,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <memory>
 #include <vector>
 
 #include "nuprof.h"
@@ -62,14 +63,23 @@ double growth_xi(const nu_halo& halo, const Derived& d, double z);
 double coupling_kappa(const nu_halo& halo, double z);
 double relic_f(const nu_relic& relic, double q);
 // Host tables, written into caller memory (no allocation) or into vectors.
+struct StageBackground {
+    double zp1, z, H;        // 1+z, z and H(z)
+};
 void coef_table_into(const nu_cosmo& cosmo, const nu_halo& halo, const Derived& d, int n_steps,
-                     double* table);   // [n_steps][C_COUNT]
+                     double* table,   // [n_steps][C_COUNT]
+                     const StageBackground* grid = nullptr);   // [2 n_steps + 1], or none
 // Largest y of the FP32 force's rational approximation of I(y)/y^2.
 constexpr double kRationalYMax = 16.0;
 // FP32 copy of a coefficient table; see host_model.cpp.
 void fp32_table(const double* tab, int n_steps, const Derived& d, float* out);
-void coef_table(const nu_cosmo& cosmo, const nu_halo& halo, const Derived& d, int n_steps,
-                std::vector<double>& table);
+// The table in both precisions, kept for the requests of a scan that share it.
+struct CoefTable {
+    std::vector<double> f64;   // [n_steps][C_COUNT]
+    std::vector<float> f32;
+};
+std::shared_ptr<const CoefTable> coef_table(const nu_cosmo& cosmo, const nu_halo& halo,
+                                            const Derived& d, int n_steps);
 void log_nodes_into(int n, double q_min, double q_max, double* q, double* wl, double* wl_coarse);
 void log_nodes(int n, double q_min, double q_max, std::vector<double>& q,
                std::vector<double>& wl, std::vector<double>& wl_coarse);
@@ -78,6 +88,9 @@ void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w);
 void resolve_opts(const nu_opts* in, nu_opts& out);
 long long device_bytes(int precision, int n_steps, int n_radii, int n_q, int n_mu,
                        int tiles_per_seg, bool keep_qi, int n_mass, int n_ftab, long long* h2d_bytes);
+// Control words of a launch: the next tile to claim, the status, the CTAs that have
+// left.  Zero before the first launch; each launch leaves them so.
+enum CtrlWord { kCtrlNext = 0, kCtrlStatus, kCtrlLeft, kCtrlWords = 4 };
 // Number of masses read from one trajectory set (Sec. III mass reuse).
 inline int relic_n_mass(const nu_relic& r) { return r.n_masses > 0 ? r.n_masses : 1; }
 
@@ -97,8 +110,9 @@ struct DevProblem {
     unsigned* seg_count;    // [n_radii] tiles finished (reset by the finisher)
     double* out;            // [n_mass][n_radii] n/nbar
     double* err;            // [n_mass][n_radii] relative quadrature-error estimate
+    double* host_out;       // out and err once more, in mapped host memory (optional)
     void* qi;               // [n_radii][n_q][n_mu] final q in the state precision (optional)
-    int* status;            // bit 0: non-finite sum
+    int* status;            // bit 0: non-finite sums so far
     double q_scale;         // q_i = |v| * q_scale (fiducial mass)
     double invIc, invR3, R2;
     double c_nfw;           // concentration: the NFW edge in y = r / (r_s (1+z))
@@ -144,6 +158,11 @@ struct QueueCtl {
 };
 
 // Accessors used by the request server (api.cu).
+// nu_profile_create without results in mapped host memory: nothing in it may
+// allocate page-locked memory while a resident launch waits on the host.
+int profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_relic* relic,
+                   const double* radii, int n_radii, const nu_pgrid* p_grid, const nu_opts* opts,
+                   nu_profile** out, bool host_results);
 const DevProblem& profile_desc(const nu_profile* h);
 int profile_n_radii(const nu_profile* h);
 int profile_n_out(const nu_profile* h);   // n_mass * n_radii result values
@@ -155,6 +174,7 @@ int profile_read(const nu_profile* h, double* out, double* err, void* stream);
 // the host).
 size_t staging_capacity();
 int staging_reserve(size_t bytes);
+void host_results_reserve();   // page-lock the block of results in host memory
 // NU_FLAG_VERIFY: the FP64 twin of a handle (nullptr without the flag), a
 // launch of the twin alone with an event after it, and a query of that event
 // (NU_OK done, NU_EAGAIN running, NU_EBUSY never run, NU_ECUDA).
@@ -165,7 +185,7 @@ int profile_twin_query(const nu_profile* h);
 // Kernel launch helpers (traj_kernel.cu).  A request's or batch's shape
 // (nu_opts.block x tpt) fixes its tile, whose sums are added in order, and so the
 // rounding of its results; how a launch runs such tiles is chosen by plan_shape.
-enum TrajKernelKind { kPacked, kRing, kFp64, kGeneralF32, kCountF32, kCountF64 };
+enum TrajKernelKind { kPacked, kRing, kFp64, kGeneralF32, kCountF32, kCountF64, kKernelKinds };
 struct LaunchShape {
     int kernel;      // TrajKernelKind
     int threads;     // of a CTA

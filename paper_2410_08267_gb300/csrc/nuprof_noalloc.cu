@@ -112,7 +112,7 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
     int tps = 0, n_tiles = 0;
     size_t off = 0;
     auto carve = [&](size_t bytes) { size_t at = off; off += up256(bytes); return at; };
-    const size_t o_ctrl = carve(4 * sizeof(unsigned));
+    const size_t o_ctrl = carve(kCtrlWords * sizeof(unsigned));
     const size_t o_prob = carve(sizeof(DevProblem));
     const size_t o_pref = carve(2 * sizeof(int));
     const size_t o_coef = carve((size_t)N * C_COUNT * sz);
@@ -218,7 +218,7 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
     P.out = reinterpret_cast<double*>(dev + o_out);
     P.err = reinterpret_cast<double*>(dev + o_err);
     P.qi = nullptr;
-    P.status = reinterpret_cast<int*>(dev + o_ctrl + sizeof(unsigned));
+    P.status = reinterpret_cast<int*>(dev + o_ctrl) + kCtrlStatus;
     P.q_scale = relic->m_eV / (kC * kT0);
     P.invIc = 1.0 / d.Ic;
     P.invR3 = d.R > 0.0 ? 1.0 / (d.R * d.R * d.R) : 0.0;
@@ -268,8 +268,7 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
     const int grid = n_tiles < per_sm * sms ? n_tiles : per_sm * sms;
 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    // The array keeps the previous call's contents: the control words (work
-    // counter, status) are part of the zeroed upload and the per-radius
+    // The array keeps the previous call's contents: the control words are part of the zeroed upload and the per-radius
     // completion counters are cleared explicitly.
     if (cudaMemcpyAsync(dev, st, upload_end, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemsetAsync(dev + o_cnt, 0, (size_t)n_radii * sizeof(unsigned), s) != cudaSuccess) {

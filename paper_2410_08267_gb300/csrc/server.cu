@@ -286,8 +286,8 @@ bool nu_server::admit_one()
     void* state = nullptr;
     if (rc == NU_OK) {
         state = arena.alloc(state_bytes);
-        if (state) rc = nu_profile_create(&p.cosmo, &p.halo, &p.relic, p.radii.data(),
-                                          (int)p.radii.size(), &p.grid, &p.opts, &h);
+        if (state) rc = profile_create(&p.cosmo, &p.halo, &p.relic, p.radii.data(),
+                                       (int)p.radii.size(), &p.grid, &p.opts, &h, false);
         if (!state || rc == NU_ENOMEM) {
             arena.release(state);
             if (h) nu_profile_destroy(h);
@@ -434,7 +434,7 @@ void nu_server::run()
                             compute) != cudaSuccess ||
             cudaMemcpyAsync(d_prefix[slot], prefix.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice,
                             compute) != cudaSuccess ||
-            cudaMemsetAsync(d_ctrl, 0, 2 * sizeof(unsigned), compute) != cudaSuccess ||
+            cudaMemsetAsync(d_ctrl, 0, kCtrlWords * sizeof(unsigned), compute) != cudaSuccess ||
             (h_flags && cudaMemsetAsync(d_counts, 0, n * sizeof(unsigned), compute) != cudaSuccess))
             rc = NU_ECUDA;
         int grid = 0, per_sm = 0, sms = 0;
@@ -747,6 +747,7 @@ int nu_server_create(const nu_server_opts* opts, nu_server** out)
         // room for typical uploads, so that admissions during a launch never
         // have to grow the staging buffer
         staging_reserve((size_t)16 << 20);
+        host_results_reserve();
     }
     if (cudaStreamCreateWithFlags(&s->compute, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&s->upload, cudaStreamNonBlocking) != cudaSuccess ||

@@ -960,7 +960,7 @@ template <typename T, int TPT, bool COUNT, StepLoop LOOP>
 __global__ void __launch_bounds__(LOOP == kLoopGeneral ? (COUNT || TPT == 2 ? 512 : 256) : LOOP == kLoopPacked ? 256 : kRingThreads,
                                   LOOP == kLoopPacked ? 3 : 1)
 traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_prefix,
-            int n_probs, int n_tiles, unsigned* __restrict__ tile_counter,
+            int n_probs, int n_tiles, unsigned* __restrict__ ctrl,
             unsigned long long* __restrict__ tallies, QueueCtl* queue)
 {
     using Ctr = typename std::conditional<COUNT, Tally, NoTally>::type;
@@ -986,7 +986,7 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
 
     for (;;) {
         if (threadIdx.x == 0) {
-            const unsigned claimed = atomicAdd(tile_counter, 1u);
+            const unsigned claimed = atomicAdd(&ctrl[kCtrlNext], 1u);
             int np = n_probs;
             int t = queue ? queue_wait(queue, claimed, &np)
                           : (claimed < (unsigned)n_tiles ? (int)claimed : -1);
@@ -1225,7 +1225,12 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
                     const double ratio = t0 * P.norms[2 * a];
                     const double ratio_c = t1 * P.norms[2 * a + 1];
                     P.out[(size_t)a * P.n_radii + seg] = ratio;
-                    P.err[(size_t)a * P.n_radii + seg] = fabs(ratio - ratio_c) / (3.0 * fabs(ratio));
+                    const double err = fabs(ratio - ratio_c) / (3.0 * fabs(ratio));
+                    P.err[(size_t)a * P.n_radii + seg] = err;
+                    if (P.host_out) {
+                        P.host_out[(size_t)a * P.n_radii + seg] = ratio;
+                        P.host_out[(size_t)(nm + a) * P.n_radii + seg] = err;
+                    }
                     if (!isfinite(ratio)) atomicOr(P.status, 1);
                 }
             }
@@ -1241,6 +1246,11 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
             }
         }
         // the next iteration's first __syncthreads orders s_tile/s_last reuse
+    }
+    // the last CTA to leave makes the counters ready for the next launch
+    if (threadIdx.x == 0 && atomicAdd(&ctrl[kCtrlLeft], 1u) == gridDim.x - 1u) {
+        ctrl[kCtrlNext] = 0u;
+        ctrl[kCtrlLeft] = 0u;
     }
     if constexpr (COUNT) {
 #pragma unroll
@@ -1407,11 +1417,16 @@ int launch_traj_tally(int precision, const LaunchShape& shape, int grid, const D
 
 int max_ctas_per_sm(const LaunchShape& shape, int* out)
 {
+    // asked for by every run: kept, as the GPUs of a process are taken to be alike
+    static std::atomic<int> kept[kKernelKinds][512 / 32 + 1];
+    std::atomic<int>& known = kept[shape.kernel][shape.threads / 32];
+    if ((*out = known.load(std::memory_order_relaxed)) > 0) return NU_OK;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kernel_of(shape.kernel), shape.threads,
                                                       ring_bytes(shape)) != cudaSuccess)
         return NU_ECUDA;
     if (shape.kernel == kFp64)
         *out = std::min(*out, std::max(1, kFp64WarpsPerSm * 32 / shape.threads));
+    known.store(*out, std::memory_order_relaxed);
     return NU_OK;
 }
 

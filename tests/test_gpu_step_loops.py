@@ -95,3 +95,38 @@ def test_results_do_not_depend_on_what_shares_the_launch(block, tpt):
                           masses=(0.05, 0.1, 0.2))
     for a, b in zip(results([small])[0], results([LARGE, small])[1]):
         assert np.array_equal(a, b)
+
+
+def test_interleaved_scans_give_the_results_of_fresh_tables():
+    """More halos and cosmologies in turn than tables and backgrounds are kept: every
+    result is that of the same request alone, and a handle's results outlive others'."""
+    probs = [PLAIN.replace(M_h=m, Om=om, n_steps=n, radii=np.array([4.0, 60.0]), n_q=16, n_mu=8)
+             for m in (1e12, 2e12, 4e12) for om in (0.29, 0.31, 0.33) for n in (50, 51)]
+    first = [nu.profile(pb) for pb in probs]
+    hs = [nu.create(pb) for pb in reversed(probs)]
+    try:
+        for h in hs:
+            nu.nu_profile_run(h)
+        again = [nu.nu_profile_result(h, 2) for h in hs][::-1]
+    finally:
+        for h in hs:
+            nu.nu_profile_destroy(h)
+    for a, b in zip(first, again):
+        assert np.array_equal(a, b)
+    assert len({r[0][0] for r in first}) == len(probs)
+
+
+def test_results_beyond_the_host_block_are_copied():
+    """Results of more values than the mapped host block holds, beside small ones."""
+    big = PLAIN.replace(radii=np.geomspace(2000.0, 1e5, 70000), n_q=2, n_mu=1, n_steps=1)
+    small = PLAIN.replace(n_steps=5)
+    want = nu.profile(small)
+    h = nu.create(big)
+    try:
+        nu.nu_profile_run(h)
+        out, err = nu.nu_profile_result(h, big.n_out)
+        assert np.array_equal(nu.profile(small), want)
+        # beyond R every trajectory keeps its momentum
+        assert np.allclose(out, 1.0, rtol=1e-6) and np.all(np.isfinite(err))
+    finally:
+        nu.nu_profile_destroy(h)
