@@ -194,37 +194,56 @@ __device__ __forceinline__ double series4(double p, double t)   // terms K + 3 .
     return fma(p, t, 1.0 / (K + 2));
 }
 
-// sum_{k=0}^{50} t^k/(k+2) for 0 < t <= t_max < 1/2.
-__device__ __forceinline__ double nfw_series(double t, float t_max)
+// FP64 steps that t_max < 1/2 needs: a multiple of 4 up to kSeriesMaxJ, or more
+// (the whole recurrence).
+__device__ __forceinline__ int series_steps(float t_max)
 {
     const int need = (int)(kSeriesBits * rcp_approx(-lg2_approx(t_max))) + 1;
-    const int J = max(8, (need + 3) & ~3);
-    double p;
-    if (J > kSeriesMaxJ) {
-        p = 1.0 / 52.0;
-        p = fma(p, t, 1.0 / 51.0);
-        p = fma(p, t, 1.0 / 50.0);
-    } else {
-        const float tf = trunc_f32(t);
-        float s = c_series[J + kSeriesTail - 1];
+    return max(8, (need + 3) & ~3);
+}
+
+// Horner's value before the last J (kSeriesMaxJ at most) steps.
+__device__ __forceinline__ double series_start(double t, int J)
+{
+    if (J > kSeriesMaxJ) return fma(fma(1.0 / 52.0, t, 1.0 / 51.0), t, 1.0 / 50.0);
+    const float tf = trunc_f32(t);
+    float s = c_series[J + kSeriesTail - 1];
 #pragma unroll
-        for (int i = kSeriesTail - 2; i >= 0; --i) s = fmaf(s, tf, c_series[J + i]);
-        p = widen_f32(s);
-    }
+    for (int i = kSeriesTail - 2; i >= 0; --i) s = fmaf(s, tf, c_series[J + i]);
+    return widen_f32(s);
+}
+
+// sums_{k=0}^{50} t^k/(k+2) of N values 0 < t <= t_max < 1/2, their chains side by side.
+template <int N>
+__device__ __forceinline__ void nfw_series_n(const double (&t)[N], float t_max, double (&p)[N])
+{
+    const int J = series_steps(t_max);
+#pragma unroll
+    for (int i = 0; i < N; ++i) p[i] = series_start(t[i], J);
+#define NU_TERMS(K)                                                                      \
+    case (K) + 4:                                                                        \
+        _Pragma("unroll") for (int i = 0; i < N; ++i) p[i] = series4<K>(p[i], t[i])
     switch (min(J, kSeriesMaxJ)) {
-    case 48: p = series4<44>(p, t);   // fallthrough, as all below
-    case 44: p = series4<40>(p, t);
-    case 40: p = series4<36>(p, t);
-    case 36: p = series4<32>(p, t);
-    case 32: p = series4<28>(p, t);
-    case 28: p = series4<24>(p, t);
-    case 24: p = series4<20>(p, t);
-    case 20: p = series4<16>(p, t);
-    case 16: p = series4<12>(p, t);
-    case 12: p = series4<8>(p, t);
-    default: p = series4<4>(p, t);
+        NU_TERMS(44); NU_TERMS(40); NU_TERMS(36); NU_TERMS(32); NU_TERMS(28); NU_TERMS(24);
+        NU_TERMS(20); NU_TERMS(16); NU_TERMS(12); NU_TERMS(8);
+    default:;                                        // every case goes on with the next
     }
-    return series4<0>(p, t);
+#undef NU_TERMS
+#pragma unroll
+    for (int i = 0; i < N; ++i) p[i] = series4<0>(series4<4>(p[i], t[i]), t[i]);
+}
+__device__ __forceinline__ double nfw_series(double t, float t_max)
+{
+    double p[1];
+    nfw_series_n<1>({t}, t_max, p);
+    return p[0];
+}
+__device__ __forceinline__ void nfw_series2(double ta, double tb, float t_max, double& pa, double& pb)
+{
+    double p[2];
+    nfw_series_n<2>({ta, tb}, t_max, p);
+    pa = p[0];
+    pb = p[1];
 }
 
 // Steps between two tests of the early exit (a power of two).
@@ -764,13 +783,13 @@ struct OneTrajectory {
     }
 };
 
-// A warp's window on the coefficient table: two buffers of kRingSteps rows in
-// shared memory, one filled by asynchronous copies while the steps of the other
-// run.  Read in place, a table row costs its first reader on an SM a wait for L2,
-// with all of a step behind it.
-constexpr int kRingSteps = 32;
-constexpr int kRow16 = C_COUNT / 4;                  // 16-byte words of a step's coefficients
-constexpr int kRing16 = 2 * kRingSteps * kRow16;     // and of a warp's two buffers
+// A warp's window on the coefficient table: two buffers of rows in shared memory,
+// one filled by asynchronous copies while the steps of the other run.  Read in
+// place, a table row costs its first reader on an SM a wait for L2, with all of a
+// step behind it.
+constexpr int kRow16 = C_COUNT / 4;                  // 16-byte words of an FP32 row; FP64 twice
+constexpr int kRingSteps = 32;                       // FP32 rows of a buffer; FP64 half
+constexpr int kRing16 = 2 * kRingSteps * kRow16;     // 16-byte words of a warp's two buffers
 
 __device__ __forceinline__ void copy16_async(float4* dst, const float4* src)
 {
@@ -784,31 +803,33 @@ __device__ __forceinline__ void copies_wait()
     asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
 }
 
-// Copy rows [first, first + kRingSteps), none past s_end, into one of the buffers.
+// Copy the rows of ROW words from `first` on, none past s_end, into a buffer.
+template <int ROW>
 __device__ __forceinline__ void ring_fill(float4* half, const float4* tab, int first, int s_end,
                                           int lane)
 {
-    const int n16 = min(kRingSteps, s_end - first) * kRow16;
-    for (int i = lane; i < n16; i += 32) copy16_async(half + i, tab + (size_t)first * kRow16 + i);
+    const int n16 = min(kRing16 / 2 / ROW, s_end - first) * ROW;
+    for (int i = lane; i < n16; i += 32) copy16_async(half + i, tab + (size_t)first * ROW + i);
     copies_commit();
 }
 
-// Run body(rows, count) over steps [s_begin, s_end) in windows of kRingSteps
+// Run body(rows, count) over steps [s_begin, s_end) in windows of a buffer's
 // rows until it returns false.  Warp-uniform; all copies are done on return, so
 // the buffers can be filled again.
-template <class Body>
+template <int ROW, class Body>
 __device__ __forceinline__ void over_ring(float4* ring, const float4* tab, int s_begin, int s_end,
                                           int lane, Body body)
 {
-    ring_fill(ring, tab, s_begin, s_end, lane);
-    ring_fill(ring + kRing16 / 2, tab, s_begin + kRingSteps, s_end, lane);
+    constexpr int kSteps = kRing16 / 2 / ROW;
+    ring_fill<ROW>(ring, tab, s_begin, s_end, lane);
+    ring_fill<ROW>(ring + kRing16 / 2, tab, s_begin + kSteps, s_end, lane);
     float4* half = ring;
-    for (int first = s_begin; first < s_end; first += kRingSteps) {
+    for (int first = s_begin; first < s_end; first += kSteps) {
         copies_wait<1>();                            // this half has arrived
         __syncwarp();
-        if (!body(half, min(kRingSteps, s_end - first))) break;
+        if (!body(half, min(kSteps, s_end - first))) break;
         __syncwarp();                                // every lane has read it
-        ring_fill(half, tab, first + 2 * kRingSteps, s_end, lane);
+        ring_fill<ROW>(half, tab, first + 2 * kSteps, s_end, lane);
         half = half == ring ? ring + kRing16 / 2 : ring;
     }
     copies_wait<0>();
@@ -844,7 +865,7 @@ __device__ __forceinline__ void step_loop(State& s, const float4* tab, int s_beg
     bool rational = true;
     bool select = false;             // the warp runs steps that select
     int k_select = 0;
-    over_ring(ring, tab, s_begin, s_end, lane, [&](const float4* rows, int count) {
+    over_ring<kRow16>(ring, tab, s_begin, s_end, lane, [&](const float4* rows, int count) {
         const float4* const end = rows + count * kRow16;
         // a bound below c, which comes last in the window first: c > 16, or an NFW
         // edge that lies beyond R
@@ -869,6 +890,143 @@ __device__ __forceinline__ void step_loop(State& s, const float4* tab, int s_beg
             else
                 s.template step<NARROW, kSelect>(rows, hc, rational);
             rows += kRow16;
+        }
+        return true;
+    });
+}
+
+// ---------------------------------------------------------------------------
+// FP64 step loop: rk4_step with its force evaluations in two independent pairs.  The
+// values are those of accel_m; what differs is which lanes compute them.  With one
+// warp on a scheduler the pair's chains fill each other's waits, and where the lanes
+// of a warp lie on both sides of y = 1, which most warps' do at some steps, the
+// evaluations of the pair that need the series are gathered into one pass over the
+// warp if they are 32 or fewer, and those that need the logarithm likewise.
+// ---------------------------------------------------------------------------
+struct Compact {                                     // a pair's evaluations that need a pass
+    unsigned a, b, below;                            // their lanes; the lanes below this one
+    __device__ __forceinline__ Compact(bool need_a, bool need_b, int lane)
+        : a(__ballot_sync(0xffffffffu, need_a)), b(__ballot_sync(0xffffffffu, need_b)),
+          below((1u << lane) - 1u)
+    {
+    }
+    __device__ __forceinline__ int count() const { return __popc(a) + __popc(b); }
+    __device__ __forceinline__ bool one_pass() const { return a && b && count() <= 32; }
+    __device__ __forceinline__ int slot_a() const { return __popc(a & below); }
+    __device__ __forceinline__ int slot_b() const { return __popc(a) + __popc(b & below); }
+    // f of va where need_a and of vb where need_b, in one pass (one_pass())
+    template <class F>
+    __device__ __forceinline__ void pass(bool need_a, bool need_b, double& va, double& vb, double* buf,
+                                         int lane, F f) const
+    {
+        if (need_a) buf[slot_a()] = va;
+        if (need_b) buf[slot_b()] = vb;
+        __syncwarp();
+        const double r = f(buf[lane < count() ? lane : 0]);
+        __syncwarp();
+        buf[lane] = r;
+        __syncwarp();
+        if (need_a) va = buf[slot_a()];
+        if (need_b) vb = buf[slot_b()];
+        __syncwarp();
+    }
+};
+
+__device__ __forceinline__ void accel_pair(double xa, double ya, double Sa, double Qa, double xb,
+                                           double yb, double Sb, double Qb, const HaloF64& hc,
+                                           double* buf, int lane, double& ma, double& mb)
+{
+    const unsigned full = 0xffffffffu;
+    const double r2a = fma(xa, xa, ya * ya), r2b = fma(xb, xb, yb * yb);
+    const bool in_a = less_nonneg(r2a, hc.R2), in_b = less_nonneg(r2b, hc.R2);
+    ma = mb = 0.0;
+    if (!__any_sync(full, in_a || in_b)) return;
+    const double rinva = rsqrt(less_nonneg(r2a, 1e-200) ? 1e-200 : r2a);
+    const double rinvb = rsqrt(less_nonneg(r2b, 1e-200) ? 1e-200 : r2b);
+    const bool nfw_a = in_a && less_nonneg(r2a, Qa), nfw_b = in_b && less_nonneg(r2b, Qb);
+    double sela = 1.0, selb = 1.0;
+    if (__any_sync(full, nfw_a || nfw_b)) {
+        const double ysa = (r2a * rinva) * Sa, ysb = (r2b * rinvb) * Sb;
+        const double ta = quotient(ysa, 1.0 + ysa), tb = quotient(ysb, 1.0 + ysb);
+        const bool sa = nfw_a && less_nonneg(ta, 0.5), sb = nfw_b && less_nonneg(tb, 0.5);
+        const bool la = nfw_a && !sa, lb = nfw_b && !sb;
+        double Ia = ta, Ib = tb;
+        const Compact cs(sa, sb, lane);
+        if (cs.a | cs.b) {
+            const float t_max = __uint_as_float(1u + __reduce_max_sync(
+                full, max(sa ? __float_as_uint(trunc_f32(ta)) : 0u,
+                          sb ? __float_as_uint(trunc_f32(tb)) : 0u)));
+            if (cs.one_pass()) {
+                cs.pass(sa, sb, Ia, Ib, buf, lane,
+                        [&](double t) { return (t * t) * nfw_series(t, t_max); });
+            } else if (cs.a && cs.b) {
+                double pa, pb;
+                nfw_series2(ta, tb, t_max, pa, pb);
+                Ia = (ta * ta) * pa;
+                Ib = (tb * tb) * pb;
+            } else if (cs.a) {
+                Ia = (ta * ta) * nfw_series(ta, t_max);
+            } else {
+                Ib = (tb * tb) * nfw_series(tb, t_max);
+            }
+        }
+        const Compact cl(la, lb, lane);
+        if (cl.a | cl.b) {
+            double ga = ysa, gb = ysb;
+            if (cl.one_pass()) {
+                cl.pass(la, lb, ga, gb, buf, lane, [](double v) { return log1p(v); });
+            } else {
+                if (cl.a) ga = log1p(ysa);
+                if (cl.b) gb = log1p(ysb);
+            }
+            if (la) Ia = ga - ta;
+            if (lb) Ib = gb - tb;
+        }
+        if (nfw_a) sela = Ia * hc.invIc;
+        if (nfw_b) selb = Ib * hc.invIc;
+    }
+    if (in_a) ma = fma(sela, rinva * rinva * rinva, -hc.invR3);
+    if (in_b) mb = fma(selb, rinvb * rinvb * rinvb, -hc.invR3);
+}
+
+__device__ __forceinline__ void fp64_loop(double& x, double& y, double& vx, double& vy,
+                                          const float4* tab, int s_begin, int s_end, bool done,
+                                          const HaloF64& hc, float4* ring, double* buf, int lane)
+{
+    if (__all_sync(0xffffffffu, done)) return;
+    int k = 0;
+    over_ring<2 * kRow16>(ring, tab, s_begin, s_end, lane, [&](const float4* rows, int count) {
+        for (int i = 0; i < count; ++i) {
+            const double* c = reinterpret_cast<const double*>(rows + i * 2 * kRow16);
+            if ((k++ & (kSelectEvery - 1)) == 0) {
+                done |= escapes(fma(x, x, y * y), fma(x, vx, y * vy), fma(vx, vx, vy * vy), hc.R2, hc.R,
+                                c[C_IREM]);
+                if (__all_sync(0xffffffffu, done)) return false;
+            }
+            const double X2 = fma(c[C_MA1], vx, x), Y2 = fma(c[C_MA1], vy, y);
+            double m1, m2;
+            accel_pair(x, y, c[C_S0], c[C_Q0], X2, Y2, c[C_S1], c[C_Q1], hc, buf, lane, m1, m2);
+            const double p1 = c[C_B1] * m1;
+            const double VX2 = fma(p1, x, vx), VY2 = fma(p1, y, vy);
+            const double p2 = c[C_B2] * m2;
+            const double VX3 = fma(p2, X2, vx), VY3 = fma(p2, Y2, vy);
+            const double X3 = fma(c[C_MA2], VX2, x), Y3 = fma(c[C_MA2], VY2, y);
+            const double X4 = fma(c[C_MA3], VX3, x), Y4 = fma(c[C_MA3], VY3, y);
+            double m3, m4;
+            accel_pair(X3, Y3, c[C_S1], c[C_Q1], X4, Y4, c[C_S2], c[C_Q2], hc, buf, lane, m3, m4);
+            const double p3 = c[C_B3] * m3;
+            const double VX4 = fma(p3, X3, vx), VY4 = fma(p3, Y3, vy);
+            const double p4 = c[C_B4] * m4;
+            const double nx = fma(c[C_W2], VX4, fma(c[C_W1], VX2 + VX3, fma(c[C_W0], vx, x)));
+            const double ny = fma(c[C_W2], VY4, fma(c[C_W1], VY2 + VY3, fma(c[C_W0], vy, y)));
+            const double p2x2 = p2 * 2.0;            // exact doubling
+            const double third = 1.0 / 3.0;
+            const double tx = fma(p3, X3, fma(p2x2, X2, p1 * x));
+            const double ty = fma(p3, Y3, fma(p2x2, Y2, p1 * y));
+            vx = fma(p4, X4, fma(tx, third, vx));
+            vy = fma(p4, Y4, fma(ty, third, vy));
+            x = nx;
+            y = ny;
         }
         return true;
     });
@@ -949,15 +1107,16 @@ __device__ __forceinline__ double sum_of_four(int n, int have, Load load)
 //                the precision sweep of four masses; 96 and 20 warps, 5.74 ms, but
 //                the uneven batch 27.5 against 27.0 ms);
 //   kLoopRing    one trajectory per thread, for small launches (plan_shape);
-//   kLoopGeneral one trajectory after another with the general force: the FP64
-//                mode, and with COUNT the counting variant of either mode.
-enum StepLoop { kLoopGeneral, kLoopPacked, kLoopRing };
+//   kLoopFp64    one trajectory per thread;
+//   kLoopGeneral one trajectory after another with the general force: with COUNT
+//                the counting variant of either mode.
+enum StepLoop { kLoopGeneral, kLoopPacked, kLoopRing, kLoopFp64 };
 constexpr int kRingThreads = 128;
 
 __device__ __forceinline__ int warp_id() { return threadIdx.x >> 5; }
 
 template <typename T, int TPT, bool COUNT, StepLoop LOOP>
-__global__ void __launch_bounds__(LOOP == kLoopGeneral ? (COUNT || TPT == 2 ? 512 : 256) : LOOP == kLoopPacked ? 256 : kRingThreads,
+__global__ void __launch_bounds__(LOOP == kLoopGeneral ? 512 : LOOP == kLoopRing ? kRingThreads : 256,
                                   LOOP == kLoopPacked ? 3 : 1)
 traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_prefix,
             int n_probs, int n_tiles, unsigned* __restrict__ ctrl,
@@ -975,6 +1134,7 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
     // the second hands its lanes' values to the first
     __shared__ double s_red[16][2];
     __shared__ double s_half[TPT == 1 ? 8 : 1][2][32];
+    __shared__ double s_pass[LOOP == kLoopFp64 ? 8 : 1][32];
     extern __shared__ __align__(16) float4 s_ring[];   // kRing16 words a warp (not kLoopGeneral)
     float4* ring = s_ring + warp_id() * kRing16;
 
@@ -1036,7 +1196,8 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
         double* part = P.partials + ((size_t)seg * tps + tis) * 2 * nm;
 
         // one pass, but for a tile of more trajectories than the CTA holds
-        for (int base = 0; base < (LOOP == kLoopGeneral ? P.tile : 1); base += blockDim.x * TPT) {
+        constexpr bool kPasses = LOOP == kLoopGeneral || LOOP == kLoopFp64;
+        for (int base = 0; base < (kPasses ? P.tile : 1); base += blockDim.x * TPT) {
         T x[TPT], y[TPT], vx[TPT], vy[TPT];
         bool act[TPT];
         bool done = true;            // every trajectory of this lane is finished
@@ -1069,7 +1230,10 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
         // that keeps stepping with its warp stays beyond R with its velocity
         // unchanged.  All lanes of the warp reach the votes, so the full mask is
         // valid.
-        if constexpr (LOOP != kLoopGeneral) {
+        if constexpr (LOOP == kLoopFp64) {
+            fp64_loop(x[0], y[0], vx[0], vy[0], reinterpret_cast<const float4*>(tab), s_begin, s_end,
+                      done, hc, ring, s_pass[warp], lane);
+        } else if constexpr (LOOP != kLoopGeneral) {
             using State = typename std::conditional<LOOP == kLoopPacked, TwoTrajectories, OneTrajectory>::type;
             static_assert(TPT == (LOOP == kLoopPacked ? 2 : 1), "trajectories of a lane");
             const HaloX2 h2{dup(hc.invIc), dup(-hc.invR3), hc.R2, hc.R, hc.c};
@@ -1374,7 +1538,7 @@ static TrajKernel kernel_of(int kernel)
     switch (kernel) {
     case kPacked: return traj_kernel<float, 2, false, kLoopPacked>;
     case kRing: return traj_kernel<float, 1, false, kLoopRing>;
-    case kFp64: return traj_kernel<double, 1, false, kLoopGeneral>;
+    case kFp64: return traj_kernel<double, 1, false, kLoopFp64>;
     case kGeneralF32: return traj_kernel<float, 2, false, kLoopGeneral>;
     case kCountF32: return traj_kernel<float, 2, true, kLoopGeneral>;
     default: return traj_kernel<double, 2, true, kLoopGeneral>;
@@ -1384,7 +1548,7 @@ static TrajKernel kernel_of(int kernel)
 // Shared memory of a CTA: its warps' windows on the table.
 static size_t ring_bytes(const LaunchShape& shape)
 {
-    return shape.kernel == kPacked || shape.kernel == kRing
+    return shape.kernel == kPacked || shape.kernel == kRing || shape.kernel == kFp64
                ? (size_t)(shape.threads / 32) * kRing16 * sizeof(float4) : 0;
 }
 
