@@ -657,6 +657,7 @@ __device__ __forceinline__ f2 m_form(f2 r2, f2 S, float Yq0, float Yq1, f2 T, co
 // Two trajectories of a lane: the halves of every pair are theirs.
 struct TwoTrajectories {
     f2 x, y, vx, vy;
+    __device__ __forceinline__ void begin(const float4*) {}
     __device__ __forceinline__ TwoTrajectories(const float* x_, const float* y_, const float* vx_,
                                                const float* vy_)
         : x(pk(x_[0], x_[1])), y(pk(y_[0], y_[1])), vx(pk(vx_[0], vx_[1])), vy(pk(vy_[0], vy_[1]))
@@ -679,7 +680,7 @@ struct TwoTrajectories {
                (!act[1] || escapes(f2hi(r2), f2hi(dot), f2hi(v2), hc.R2, hc.R, irem));
     }
     template <bool NARROW, StepForm FORM>
-    __device__ __forceinline__ bool step(const float4* row, const HaloX2& hc, bool& rational)
+    __device__ __forceinline__ bool step(const float4* row, const float4*, const HaloX2& hc, bool& rational)
     {
         auto r2 = [](f2 a, f2 b) { return fma2(a, a, fma2(b, b, dup(kR2Guard))); };
         const float4 q0 = row[0];                    // MA1 MA2 MA3 W0
@@ -735,6 +736,8 @@ struct TwoTrajectories {
 // is what a scheduler with few warps is bound by.
 struct OneTrajectory {
     f2 r, v;
+    float ma1;                                       // the next step's C_MA1, read a step ahead
+    __device__ __forceinline__ void begin(const float4* row) { ma1 = row[0].x; }
     __device__ __forceinline__ OneTrajectory(const float* x, const float* y, const float* vx,
                                              const float* vy)
         : r(pk(x[0], y[0])), v(pk(vx[0], vy[0]))
@@ -752,11 +755,13 @@ struct OneTrajectory {
                                   hc.R, irem);
     }
     template <bool NARROW, StepForm FORM>
-    __device__ __forceinline__ bool step(const float4* row, const HaloX2& hc, bool& rational)
+    __device__ __forceinline__ bool step(const float4* row, const float4* next, const HaloX2& hc,
+                                         bool& rational)
     {
+        const f2 R2 = fma2(dup(ma1), v, r);
+        const float ma1_next = next[0].x;
         auto r2 = [](f2 a, f2 b) { return pk(guarded_r2(f2lo(a), f2hi(a)), guarded_r2(f2lo(b), f2hi(b))); };
         const float4 q0 = row[0], q1 = row[1], q2 = row[2], q3 = row[3], q4 = row[4];
-        const f2 R2 = fma2(dup(q0.x), v, r);
         f2 y12, y43;
         const f2 m12 = m_form<NARROW, FORM>(r2(r, R2), pk(q2.z, q2.w), q3.y, q3.z, pk(q4.x, q4.y), hc, y12);
         const f2 p12 = mul2(pk(q1.x, q1.y), m12);
@@ -779,6 +784,7 @@ struct OneTrajectory {
         const f2 t = fma2(p3, R3, fma2(dup(f2hi(p12) * 2.0f), R2, mul2(p1, r)));
         v = fma2(p4, R4, fma2(t, dup(1.0f / 3.0f), v));
         r = nr;
+        ma1 = ma1_next;
         return true;
     }
 };
@@ -870,10 +876,12 @@ __device__ __forceinline__ void step_loop(State& s, const float4* tab, int s_beg
         // a bound below c, which comes last in the window first: c > 16, or an NFW
         // edge that lies beyond R
         const bool logarithm = end[3 - kRow16].w < hc.c;
+        auto next = [&] { return rows + kRow16 < end ? rows + kRow16 : rows; };
+        s.begin(rows);
         while (rows < end) {
             if (!select) {
                 for (; rows < end; rows += kRow16)
-                    if (!s.template step<NARROW, kRational>(rows, hc, rational)) break;
+                    if (!s.template step<NARROW, kRational>(rows, next(), hc, rational)) break;
                 if (rows >= end) break;
                 select = true;
                 k_select = 0;
@@ -886,9 +894,9 @@ __device__ __forceinline__ void step_loop(State& s, const float4* tab, int s_beg
                 rational = true;
             }
             if (logarithm)
-                s.template step<NARROW, kSelectLog>(rows, hc, rational);
+                s.template step<NARROW, kSelectLog>(rows, next(), hc, rational);
             else
-                s.template step<NARROW, kSelect>(rows, hc, rational);
+                s.template step<NARROW, kSelect>(rows, next(), hc, rational);
             rows += kRow16;
         }
         return true;
