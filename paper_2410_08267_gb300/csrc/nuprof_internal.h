@@ -185,7 +185,7 @@ int profile_twin_query(const nu_profile* h);
 // Kernel launch helpers (traj_kernel.cu).  A request's or batch's shape
 // (nu_opts.block x tpt) fixes its tile, whose sums are added in order, and so the
 // rounding of its results; how a launch runs such tiles is chosen by plan_shape.
-enum TrajKernelKind { kPacked, kRing, kFp64, kGeneralF32, kCountF32, kCountF64, kKernelKinds };
+enum TrajKernelKind { kPacked, kRing, kFp64, kFp64Split, kGeneralF32, kCountF32, kCountF64, kKernelKinds };
 struct LaunchShape {
     int kernel;      // TrajKernelKind
     int threads;     // of a CTA
@@ -193,10 +193,11 @@ struct LaunchShape {
     int group;       // such tiles in one tile of the asked shape
 };
 struct LaunchSize {
-    long long n_traj = 0, tiles128 = 0, tiles256 = 0;   // and tiles of 128 and of 256
+    long long n_traj = 0, tiles64 = 0, tiles128 = 0, tiles256 = 0;   // and tiles of 64 ...
     void add(long long n_radii, long long n_seg)        // a request's radii, trajectories of one
     {
         n_traj += n_radii * n_seg;
+        tiles64 += n_radii * ((n_seg + 63) / 64);
         tiles128 += n_radii * ((n_seg + 127) / 128);
         tiles256 += n_radii * ((n_seg + 255) / 256);
     }

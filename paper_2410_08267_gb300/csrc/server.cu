@@ -401,7 +401,7 @@ void nu_server::run()
             size.add(d.n_radii, (long long)d.n_q * d.n_mu);
         }
         // (requests may join a resident launch later: it is taken to fill the chip)
-        if (o.resident) size.tiles256 = std::max(size.tiles256, 1LL << 20);
+        if (o.resident) size.tiles64 = size.tiles256 = 1LL << 40;
         const LaunchShape shape = plan_shape(o.precision, tile, size);
         if (chunk > 0 && traj_active * chunk > o.step_budget)
             chunk = std::max(1, (int)(o.step_budget / traj_active));

@@ -997,9 +997,12 @@ __device__ __forceinline__ void accel_pair(double xa, double ya, double Sa, doub
     if (in_b) mb = fma(selb, rinvb * rinvb * rinvb, -hc.invR3);
 }
 
+// The loop of one warp.  pair(x, y, S, Q, X, Y, S', Q', m, m') evaluates the forces of
+// two points.
+template <class Pair>
 __device__ __forceinline__ void fp64_loop(double& x, double& y, double& vx, double& vy,
                                           const float4* tab, int s_begin, int s_end, bool done,
-                                          const HaloF64& hc, float4* ring, double* buf, int lane)
+                                          const HaloF64& hc, float4* ring, int lane, Pair pair)
 {
     if (__all_sync(0xffffffffu, done)) return;
     int k = 0;
@@ -1013,7 +1016,7 @@ __device__ __forceinline__ void fp64_loop(double& x, double& y, double& vx, doub
             }
             const double X2 = fma(c[C_MA1], vx, x), Y2 = fma(c[C_MA1], vy, y);
             double m1, m2;
-            accel_pair(x, y, c[C_S0], c[C_Q0], X2, Y2, c[C_S1], c[C_Q1], hc, buf, lane, m1, m2);
+            pair(x, y, c[C_S0], c[C_Q0], X2, Y2, c[C_S1], c[C_Q1], m1, m2);
             const double p1 = c[C_B1] * m1;
             const double VX2 = fma(p1, x, vx), VY2 = fma(p1, y, vy);
             const double p2 = c[C_B2] * m2;
@@ -1021,7 +1024,7 @@ __device__ __forceinline__ void fp64_loop(double& x, double& y, double& vx, doub
             const double X3 = fma(c[C_MA2], VX2, x), Y3 = fma(c[C_MA2], VY2, y);
             const double X4 = fma(c[C_MA3], VX3, x), Y4 = fma(c[C_MA3], VY3, y);
             double m3, m4;
-            accel_pair(X3, Y3, c[C_S1], c[C_Q1], X4, Y4, c[C_S2], c[C_Q2], hc, buf, lane, m3, m4);
+            pair(X3, Y3, c[C_S1], c[C_Q1], X4, Y4, c[C_S2], c[C_Q2], m3, m4);
             const double p3 = c[C_B3] * m3;
             const double VX4 = fma(p3, X3, vx), VY4 = fma(p3, Y3, vy);
             const double p4 = c[C_B4] * m4;
@@ -1039,6 +1042,27 @@ __device__ __forceinline__ void fp64_loop(double& x, double& y, double& vx, doub
         return true;
     });
 }
+
+// The pairs of a small launch, whose warps leave half of the schedulers without one:
+// two warps integrate the same trajectories, each evaluates one point of a pair and
+// hands it to the other.  They hold the same state, so they meet at every barrier.
+struct SplitPair {
+    const HaloF64& hc;
+    double* shared;                                  // [2][2][32]: pairs in turn, points
+    int barrier, role, lane, turn;
+    __device__ __forceinline__ void operator()(double xa, double ya, double Sa, double Qa, double xb,
+                                               double yb, double Sb, double Qb, double& ma, double& mb)
+    {
+        NoTally none;
+        const double m = role ? accel_m(xb, yb, Sb, Qb, 0.0, hc, none) : accel_m(xa, ya, Sa, Qa, 0.0, hc, none);
+        double* at = shared + turn * 64;
+        at[role * 32 + lane] = m;
+        asm volatile("bar.sync %0, 64;" ::"r"(barrier) : "memory");
+        ma = at[lane];
+        mb = at[32 + lane];
+        turn ^= 1;       // written again only after the next pair's barrier, past these reads
+    }
+};
 
 // ---------------------------------------------------------------------------
 // Work queue of a resident launch (see QueueCtl).  Thread 0 of a CTA has
@@ -1116,9 +1140,11 @@ __device__ __forceinline__ double sum_of_four(int n, int have, Load load)
 //                the uneven batch 27.5 against 27.0 ms);
 //   kLoopRing    one trajectory per thread, for small launches (plan_shape);
 //   kLoopFp64    one trajectory per thread;
+//   kLoopFp64Split  one trajectory in a lane of two warps (SplitPair): CTAs of four
+//                warps and 64 trajectories;
 //   kLoopGeneral one trajectory after another with the general force: with COUNT
 //                the counting variant of either mode.
-enum StepLoop { kLoopGeneral, kLoopPacked, kLoopRing, kLoopFp64 };
+enum StepLoop { kLoopGeneral, kLoopPacked, kLoopRing, kLoopFp64, kLoopFp64Split };
 constexpr int kRingThreads = 128;
 
 __device__ __forceinline__ int warp_id() { return threadIdx.x >> 5; }
@@ -1142,15 +1168,17 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
     // the second hands its lanes' values to the first
     __shared__ double s_red[16][2];
     __shared__ double s_half[TPT == 1 ? 8 : 1][2][32];
-    __shared__ double s_pass[LOOP == kLoopFp64 ? 8 : 1][32];
+    __shared__ double s_pass[LOOP == kLoopFp64 ? 8 : LOOP == kLoopFp64Split ? 8 : 1][32];
     extern __shared__ __align__(16) float4 s_ring[];   // kRing16 words a warp (not kLoopGeneral)
     float4* ring = s_ring + warp_id() * kRing16;
 
     const int lane = threadIdx.x & 31;
     const int warp = warp_id();
     const int n_warps = blockDim.x >> 5;
+    constexpr bool kSplit = LOOP == kLoopFp64Split;
+    const int group = kSplit ? warp & 1 : warp;      // of 32 trajectories of a thread's slot
     // trajectory of slot i of this thread within a pass
-    auto slot = [&](int i) { return (warp * TPT + i) * 32 + lane; };
+    auto slot = [&](int i) { return (group * TPT + i) * 32 + lane; };
 
     for (;;) {
         if (threadIdx.x == 0) {
@@ -1240,7 +1268,16 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
         // valid.
         if constexpr (LOOP == kLoopFp64) {
             fp64_loop(x[0], y[0], vx[0], vy[0], reinterpret_cast<const float4*>(tab), s_begin, s_end,
-                      done, hc, ring, s_pass[warp], lane);
+                      done, hc, ring, lane,
+                      [&](double xa, double ya, double Sa, double Qa, double xb, double yb, double Sb,
+                          double Qb, double& ma, double& mb) {
+                          accel_pair(xa, ya, Sa, Qa, xb, yb, Sb, Qb, hc, s_pass[warp], lane, ma, mb);
+                      });
+        } else if constexpr (kSplit) {
+            SplitPair pair{hc, s_pass[group * 4], 1 + group, warp >> 1, lane, 0};
+            fp64_loop(x[0], y[0], vx[0], vy[0], reinterpret_cast<const float4*>(tab), s_begin, s_end,
+                      done, hc, ring, lane, pair);
+            if (warp >> 1) act[0] = false;               // counted once
         } else if constexpr (LOOP != kLoopGeneral) {
             using State = typename std::conditional<LOOP == kLoopPacked, TwoTrajectories, OneTrajectory>::type;
             static_assert(TPT == (LOOP == kLoopPacked ? 2 : 1), "trajectories of a lane");
@@ -1487,7 +1524,10 @@ int launch_force_probe(int precision, const DevProblem* d_prob, int stage, const
 // those only as many on an SM as give each scheduler a warp: one keeps its FP64
 // unit busy, and work not yet started can go to an SM that is done early.  Six radii of
 // the precision sweep take 26.7 ms with 4 warps on an SM, 27.5 with 6, 31.6 with 8 and
-// 33.8 with 20; 27.2 in CTAs of 4 warps and 33.2 of 8.
+// 33.8 with 20; 27.2 in CTAs of 4 warps and 33.2 of 8.  Up to 5/3 such tiles for
+// an SM a second pair of warps takes half of the force evaluations, one CTA on an SM: 16 to
+// 224 tiles of the plain workload 3.75-3.79 ms instead of 5.7-6.4, 256 tiles 4.3 instead of 6.5,
+// 304 tiles 6.6 against 6.5.
 constexpr int kFp64WarpsPerSm = 4;
 constexpr int kSms = 152;
 constexpr int kPackedTile = 256;
@@ -1499,9 +1539,10 @@ LaunchShape plan_shape(int precision, int tile, const LaunchSize& size)
     LaunchShape s;
     s.tile = tile;
     if (precision == NU_FP64) {
-        s.kernel = kFp64;
+        const bool split = tile % kUnit == 0 && size.tiles64 * 3 <= kSms * 5;
+        s.kernel = split ? kFp64Split : kFp64;
         s.tile = tile % kUnit == 0 ? kUnit : tile;
-        s.threads = std::min(s.tile, 256);
+        s.threads = split ? 2 * kUnit : std::min(s.tile, 256);
     } else {
         const long long w1 = (size.tiles128 + kSms - 1) / kSms, w2 = (size.tiles256 + kSms - 1) / kSms;
         const bool one = tile % kRingThreads == 0 && w2 <= kPackedCtas &&
@@ -1547,6 +1588,7 @@ static TrajKernel kernel_of(int kernel)
     case kPacked: return traj_kernel<float, 2, false, kLoopPacked>;
     case kRing: return traj_kernel<float, 1, false, kLoopRing>;
     case kFp64: return traj_kernel<double, 1, false, kLoopFp64>;
+    case kFp64Split: return traj_kernel<double, 1, false, kLoopFp64Split>;
     case kGeneralF32: return traj_kernel<float, 2, false, kLoopGeneral>;
     case kCountF32: return traj_kernel<float, 2, true, kLoopGeneral>;
     default: return traj_kernel<double, 2, true, kLoopGeneral>;
@@ -1556,7 +1598,8 @@ static TrajKernel kernel_of(int kernel)
 // Shared memory of a CTA: its warps' windows on the table.
 static size_t ring_bytes(const LaunchShape& shape)
 {
-    return shape.kernel == kPacked || shape.kernel == kRing || shape.kernel == kFp64
+    return shape.kernel == kPacked || shape.kernel == kRing || shape.kernel == kFp64 ||
+                   shape.kernel == kFp64Split
                ? (size_t)(shape.threads / 32) * kRing16 * sizeof(float4) : 0;
 }
 
@@ -1596,7 +1639,7 @@ int max_ctas_per_sm(const LaunchShape& shape, int* out)
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kernel_of(shape.kernel), shape.threads,
                                                       ring_bytes(shape)) != cudaSuccess)
         return NU_ECUDA;
-    if (shape.kernel == kFp64)
+    if (shape.kernel == kFp64 || shape.kernel == kFp64Split)
         *out = std::min(*out, std::max(1, kFp64WarpsPerSm * 32 / shape.threads));
     known.store(*out, std::memory_order_relaxed);
     return NU_OK;

@@ -70,9 +70,12 @@ def test_large_launch_is_bitwise_the_counting_loop(change, block, tpt):
         assert np.array_equal(a, b, equal_nan=True)
 
 
-@pytest.mark.parametrize("block,tpt", [(96, 1), (480, 1), (512, 2)])
-def test_fp64_is_bitwise_the_counting_loop(block, tpt):
-    pb = PLAIN.replace(precision=W.FP64, n_steps=20)
+# 3, 160 (one for an SM) and 480 tiles of 64 trajectories; odd shapes run whole tiles
+@pytest.mark.parametrize("block,tpt", [(256, 1), (96, 1), (480, 1), (512, 2)])
+@pytest.mark.parametrize("change", [{"n_q": 11, "n_mu": 5, "radii": np.array([2.0, 40.0, 900.0])}, {},
+                                    {"radii": np.geomspace(1.0, 3000.0, 30)}, {"c": 25.0}])
+def test_fp64_is_bitwise_the_counting_loop(change, block, tpt):
+    pb = PLAIN.replace(precision=W.FP64, n_steps=20).replace(**change)
     for a, b in zip(*_both(pb, block, tpt)):
         assert np.array_equal(a, b)
 
