@@ -57,15 +57,15 @@ FLOPS_COMBINE = 61
 FLOPS_FULL = 121
 SMS, FP32_LANES_PER_SM = 152, 128
 # DRAM bytes (read + write) per launch of the trajectory kernel at the tuned
-# shape 128x3xg on this workload: mean of two launches of one ncu capture
+# this workload (every shape runs the same kernel): mean of two launches of one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum), recorded in
 # profiles/traj_kernel_precision_sweep_mixed.md.  Must be reset to None
 # whenever the kernel changes, until it is captured again.
-NCU_TRAFFIC_BYTES = {"128x3xg": 1229568.0}
-# Pipe utilisation of the same kernel and shape on this workload, from one-pass
+NCU_TRAFFIC_BYTES = 360320.0
+# Pipe utilisation of the same kernel on this workload, from one-pass
 # ncu captures (sm__pipe_fma_cycles_active, smsp__issue_active), also recorded
 # in that profile summary; reset together with the traffic when the kernel changes.
-NCU_PIPES = {"128x3xg": {"fma_pipe_cycles_active": 0.668, "issue_slots_active": 0.630}}
+NCU_PIPES = {"fma_pipe_cycles_active": 0.776, "issue_slots_active": 0.569}
 SAMPLE_RADII = (0, 9, 18, 27, 36, 45, 54, 63)   # oracle sample: ~1 s on 16 cores
 SAMPLE_MASS_INDEX = 2          # 0.1 eV
 
@@ -587,12 +587,10 @@ def bench_ours(args):
         peak_basis = f"152 SMs x 128 FP32 lanes x 2 flop/FMA x {peak_mhz:.0f} MHz"
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak,
-                "traffic": (NCU_TRAFFIC_BYTES.get(f"{block}x{tpt}{'xg' if tflags else ''}")
-                            if args.case == "full" and prec == W.MIXED else None),
-                "ncu_pipes": (NCU_PIPES.get(f"{block}x{tpt}{'xg' if tflags else ''}")
-                              if args.case == "full" and prec == W.MIXED else None),
-                "kernel": (f"traj_kernel<{'double' if prec == W.FP64 else 'float'},{min(tpt, 2)},"
-                           f"packed={tpt == 3},l1_table={bool(tflags)}>"),
+                "traffic": NCU_TRAFFIC_BYTES if args.case == "full" and prec == W.MIXED else None,
+                "ncu_pipes": NCU_PIPES if args.case == "full" and prec == W.MIXED else None,
+                "kernel": ("traj_kernel<double, one trajectory a lane>" if prec == W.FP64 else
+                           "traj_kernel<float, two trajectories a lane in packed FP32x2>"),
                 "kernel_ms": kms,
                 "flops_per_launch": flops, "flops_per_executed_traj_step": flops / live_steps,
                 "executed_traj_steps": live_steps,
@@ -670,9 +668,9 @@ def bench_ours(args):
                        "precision": ("FP64 state, force, f and sums" if prec == W.FP64 else
                                      "mixed: FP32 state/force, FP64 tables and sums"),
                        "l2": "flushed (256 MiB write) between timed steps",
-                       "launch": f"one persistent batched launch per step: grid {grid} CTAs x {block} "
-                                 f"threads, shape {block}x{tpt}{'xg' if tflags else ''} "
-                                 "(tpt 3 = two trajectories/thread in packed FP32x2; g = table via L1)",
+                       "launch": f"one persistent batched launch per step: grid {grid} CTAs, tile shape "
+                                 f"{block}x{tpt}{'xg' if tflags else ''} (block x trajectories; it fixes "
+                                 "the order of the sums, the library chooses kernel and threads)",
                        "autotune": (None if tune is None else
                                     {f"{b_}x{t_}{'xg' if f_ else ''}": round(ms, 4)
                                      for b_, t_, f_, ms in tune["candidates"]}),
