@@ -1,10 +1,9 @@
 // Launch-shape autotuner for batched trajectory launches.
 //
-// The tile shape (threads per CTA x trajectories per thread) trades
-// occupancy against instruction-level parallelism and tile padding; the best
-// one depends on the GPU, the precision mode, the step count (which sets the
-// shared-memory table size and hence how many CTAs fit on an SM) and the
-// amount of work.  nu_autotune times each candidate shape on the caller's own
+// The shape (block x trajectories) fixes the tiles whose sums are added in order;
+// the kernel and its threads the library chooses from the precision and the
+// launch's size (plan_shape), so shapes differ in tile padding and in the split of
+// odd tiles.  nu_autotune times each candidate shape on the caller's own
 // batch of requests (one warm-up run, then the median of three timed runs of
 // the trajectory kernel) and returns the fastest.  Results are cached in a
 // JSON-lines file keyed by GPU name, precision, step-count bucket and
@@ -26,7 +25,7 @@ namespace {
 struct Shape {
     int block, tpt, flags;
 };
-// threads per CTA, trajectories per thread (3: two, packed FP32x2), table source
+// block, trajectories (3: as 2), flags (NU_FLAG_GTAB: without effect)
 const Shape kShapes[] = {{256, 1, 0}, {512, 1, 0}, {256, 2, 0}, {256, 1, NU_FLAG_GTAB},
                          {384, 1, NU_FLAG_GTAB}, {256, 3, NU_FLAG_GTAB}, {128, 3, NU_FLAG_GTAB},
                          {256, 3, 0}};

@@ -5,14 +5,15 @@
 // (Eq. eoms), the force being the closed-form gradient of the compensated,
 // growing NFW halo (App. A).  The state (x, y, vx, vy) stays in registers for
 // the whole integration; the per-step coefficients (background, growth,
-// coupling at the three RK stage times, built in FP64 on the host) are read as
-// warp-uniform vector loads through the L1 cache.  At the end the Liouville map
-// f0 = f_init(P_i) (Sec. II.C) and the weight of the trajectory in
+// coupling at the three RK stage times, built in FP64 on the host) come to each
+// warp through a window of its own in shared memory.  At the end the Liouville
+// map f0 = f_init(P_i) (Sec. II.C) and the weight of the trajectory in
 // Eq. localdensity are applied, once per relic mass read from the trajectory
-// (Sec. III), and each tile's sum is formed by a warp-shuffle + shared-memory tree.  Tile sums land in a per-request
-// array; the CTA that completes the last tile of a radius adds them in tile
-// order (so every result is bitwise independent of scheduling and of what
-// else shares the launch) and writes n/nbar.
+// (Sec. III), and each tile's sum is formed by a warp-shuffle + shared-memory tree.
+// Tile sums land in a per-request array; the CTA that completes the last tile of a
+// radius adds them in an order that the trajectories alone fix (so every result is
+// bitwise independent of the kernel, of scheduling and of what else shares the
+// launch) and writes n/nbar.  plan_shape chooses the kernel of a launch.
 //
 // Work distribution: CTAs of a persistent grid pull tile indices from one
 // atomic counter; a tile is `tile` consecutive trajectories of one radius of
@@ -1211,7 +1212,7 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
         __syncthreads();
         const DevProblem& P = s_prob;
         const int n_steps = P.n_steps;
-        // coefficient table, read in place through the L1 cache with warp-uniform loads
+        // coefficient table: read through the warp's window, by kLoopGeneral in place
         const T* tab = reinterpret_cast<const T*>(P.coef);
 
         const int tps = P.tiles_per_seg;
