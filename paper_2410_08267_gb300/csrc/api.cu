@@ -497,7 +497,7 @@ int nuprof::profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_
     h->info = info;
     h->n_radii = n_radii;
     LaunchSize size;
-    size.add(n_radii, (long long)p_grid->n_q * p_grid->n_mu);
+    size.add(n_radii, (long long)p_grid->n_q * p_grid->n_mu, relic_n_mass(*relic));
     h->shape = plan_shape(o.precision, info.tile, size);
     h->n_tiles = tiles_of(h->shape, (long long)p_grid->n_q * p_grid->n_mu) * n_radii;
 
@@ -829,7 +829,7 @@ int nu_batch_create(nu_profile* const* hs, int n, const nu_opts* opts, nu_batch*
     const int tile = b->block * traj_per_thread(b->tpt);
     LaunchSize size;
     for (int i = 0; i < n; ++i)
-        size.add(hs[i]->n_radii, (long long)hs[i]->grid.n_q * hs[i]->grid.n_mu);
+        size.add(hs[i]->n_radii, (long long)hs[i]->grid.n_q * hs[i]->grid.n_mu, hs[i]->hdp.n_mass);
     b->shape = plan_shape(b->precision, tile, size);
     std::vector<DevProblem> descs(n);
     std::vector<int> prefix(n + 1, 0);

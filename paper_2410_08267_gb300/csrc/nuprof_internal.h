@@ -185,7 +185,7 @@ int profile_twin_query(const nu_profile* h);
 // Kernel launch helpers (traj_kernel.cu).  A request's or batch's shape
 // (nu_opts.block x tpt) fixes its tile, whose sums are added in order, and so the
 // rounding of its results; how a launch runs such tiles is chosen by plan_shape.
-enum TrajKernelKind { kPacked, kRing, kFp64, kFp64Split, kGeneralF32, kCountF32, kCountF64, kKernelKinds };
+enum TrajKernelKind { kPacked, kRing, kRingMasses, kFp64, kFp64Split, kGeneralF32, kCountF32, kCountF64, kKernelKinds };
 struct LaunchShape {
     int kernel;      // TrajKernelKind
     int threads;     // of a CTA
@@ -194,8 +194,10 @@ struct LaunchShape {
 };
 struct LaunchSize {
     long long n_traj = 0, tiles64 = 0, tiles128 = 0, tiles256 = 0;   // and tiles of 64 ...
-    void add(long long n_radii, long long n_seg)        // a request's radii, trajectories of one
+    int most_masses = 1;                                // read by one request
+    void add(long long n_radii, long long n_seg, int n_mass)   // a request's radii, trajectories of one
     {
+        if (n_mass > most_masses) most_masses = n_mass;
         n_traj += n_radii * n_seg;
         tiles64 += n_radii * ((n_seg + 63) / 64);
         tiles128 += n_radii * ((n_seg + 127) / 128);

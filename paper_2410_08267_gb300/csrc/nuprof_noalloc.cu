@@ -130,7 +130,7 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
     const size_t o_err = carve((size_t)n_radii * sizeof(double));
     const size_t o_part = off;
     LaunchSize size;
-    size.add(n_radii, seg);
+    size.add(n_radii, seg, 1);
     for (bool whole : {false, true}) {
         shape = whole ? whole_tiles(o.precision, o.block * o.tpt)
                       : plan_shape(o.precision, o.block * o.tpt, size);

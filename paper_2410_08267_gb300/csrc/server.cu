@@ -398,7 +398,7 @@ void nu_server::run()
         LaunchSize size;
         for (const Active& a : active) {
             const DevProblem& d = profile_desc(a.h);
-            size.add(d.n_radii, (long long)d.n_q * d.n_mu);
+            size.add(d.n_radii, (long long)d.n_q * d.n_mu, d.n_mass);
         }
         // (requests may join a resident launch later: it is taken to fill the chip)
         if (o.resident) size.tiles64 = size.tiles256 = 1LL << 40;

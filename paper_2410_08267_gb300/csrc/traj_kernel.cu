@@ -849,18 +849,18 @@ __device__ __forceinline__ void over_ring(float4* ring, const float4* tab, int s
 // With many warps it is bound by register operands and issue: a packed fused
 // multiply-add with three different register pairs takes 3 cycles of a scheduler,
 // one with a constant operand 2, each other instruction about one more (measured
-// with independent chains), and 102 of a packed step's 156 instructions are such
+// with independent chains), and 97 of a packed step's 145 instructions are such
 // operations.  With one warp on a scheduler it is bound by that warp's own issue
 // (a scalar fused multiply-add every 2 cycles) and the chain of a step.  So the
-// instructions of a step count, and no step has more than two votes, both off the
-// chain, and no branch but theirs.
+// instructions of a step count, and no step has more than one vote, off the chain,
+// and no branch but its.
 // A warp whose lanes all stay on the rational branch runs kRational steps, without
 // selects and without the exit test (no lane of it is beyond R).  Where one fails
 // it is done again in a form that lets each lane select its branch, and so are the
 // following steps: every kSelectEvery of them the warp stops if its lanes are all
 // finished, and goes back to kRational steps if they were all on that branch.
 // Evaluating the branches of such a warp by votes and warp-uniform paths took 1900
-// cycles a step on one scheduler, selecting takes 626 (431 one trajectory a lane).
+// cycles a step on one scheduler, selecting takes 479 (412 one trajectory a lane).
 constexpr int kSelectEvery = 8;
 
 template <bool NARROW, class State>
@@ -1124,6 +1124,29 @@ __device__ int queue_wait(QueueCtl* q, unsigned g, int* n_probs)
 // into ones of a unit, two or four gives the same bits.
 constexpr int kUnit = 64;
 
+// Sums over the warp of N (2 or 8) values a lane, each by warp_sum's tree: at every
+// level the lanes of one half hand over the values that the other half goes on with,
+// so 8 sums take 9 FP64 additions a lane where one after another they take 40.
+// Lane l returns the sum of value l N / 32.
+template <int N>
+__device__ __forceinline__ double warp_sums(double (&v)[N], int lane)
+{
+    int step = 16;
+#pragma unroll
+    for (int n = N / 2; n >= 1; n /= 2, step /= 2) {
+        const bool upper = (lane & step) != 0;
+#pragma unroll
+        for (int j = 0; j < n; ++j) {
+            const double give = upper ? v[j] : v[j + n], keep = upper ? v[j + n] : v[j];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, step);
+        }
+    }
+    double sum = v[0];
+#pragma unroll
+    for (; step >= 1; step /= 2) sum += __shfl_xor_sync(0xffffffffu, sum, step);
+    return sum;
+}
+
 // Sum of n (1, 2 or 4) values of a four, those from `have` on being absent.
 template <class Load>
 __device__ __forceinline__ double sum_of_four(int n, int have, Load load)
@@ -1136,22 +1159,34 @@ __device__ __forceinline__ double sum_of_four(int n, int have, Load load)
 // consecutive trajectories of one radius and integrate them in passes of
 // blockDim.x * TPT.  The step loop:
 //   kLoopPacked  two trajectories per thread in packed FP32x2, 24 warps per SM (80
-//                registers: 64 spill in the step forms, 5.95 ms against 5.75 ms on
-//                the precision sweep of four masses; 96 and 20 warps, 5.74 ms, but
-//                the uneven batch 27.5 against 27.0 ms);
+//                registers, 5.61 ms on the precision sweep of four masses; before the
+//                coefficients were read ahead 5.75 ms, 5.95 with 64 registers, which
+//                spill, and 5.74 with 96 and 20 warps, but the uneven batch 27.5
+//                against 27.0 ms);
 //   kLoopRing    one trajectory per thread, for small launches (plan_shape);
+//   kLoopRingMasses  the same with an epilogue that takes kMassGroup masses at a time,
+//                for launches in which a request reads several: f and its sums in FP64
+//                were a fifth of the kernel at 15 masses.  20 radii x 6400 trajectories
+//                x 300 steps: 301 -> 261 us with 15 masses, 220 -> 204 with 8, 185 ->
+//                177 with 4, the same with 2; the paper's production grid 281 -> 272.
+//                For one mass kLoopRing stays (relic-table profile 237 against 243 us);
+//                groups of 8 take 263 us on the paper's grid but 102 against 97 us for
+//                4 masses of 128,000 short trajectories; two trajectories a lane would
+//                spill (precision sweep 5.61 -> 5.79 ms);
 //   kLoopFp64    one trajectory per thread;
 //   kLoopFp64Split  one trajectory in a lane of two warps (SplitPair): CTAs of four
 //                warps and 64 trajectories;
 //   kLoopGeneral one trajectory after another with the general force: with COUNT
 //                the counting variant of either mode.
-enum StepLoop { kLoopGeneral, kLoopPacked, kLoopRing, kLoopFp64, kLoopFp64Split };
+enum StepLoop { kLoopGeneral, kLoopPacked, kLoopRing, kLoopRingMasses, kLoopFp64, kLoopFp64Split };
 constexpr int kRingThreads = 128;
+constexpr int kMassGroup = 4;
 
 __device__ __forceinline__ int warp_id() { return threadIdx.x >> 5; }
 
 template <typename T, int TPT, bool COUNT, StepLoop LOOP>
-__global__ void __launch_bounds__(LOOP == kLoopGeneral ? 512 : LOOP == kLoopRing ? kRingThreads : 256,
+__global__ void __launch_bounds__(LOOP == kLoopGeneral ? 512
+                                  : LOOP == kLoopRing || LOOP == kLoopRingMasses ? kRingThreads : 256,
                                   LOOP == kLoopPacked ? 3 : 1)
 traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_prefix,
             int n_probs, int n_tiles, unsigned* __restrict__ ctrl,
@@ -1167,8 +1202,9 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
     __shared__ __align__(16) DevProblem s_prob;
     // unit sums of a pass; with one trajectory per thread a unit is two warps, and
     // the second hands its lanes' values to the first
-    __shared__ double s_red[16][2];
-    __shared__ double s_half[TPT == 1 ? 8 : 1][2][32];
+    constexpr int kMasses = LOOP == kLoopRingMasses ? kMassGroup : 1;   // of an epilogue's pass
+    __shared__ double s_red[16][2 * kMasses];
+    __shared__ double s_half[TPT == 1 ? (kMasses > 1 ? 2 : 8) : 1][2 * kMasses][32];
     __shared__ double s_pass[LOOP == kLoopFp64 ? 8 : LOOP == kLoopFp64Split ? 8 : 1][32];
     extern __shared__ __align__(16) float4 s_ring[];   // kRing16 words a warp (not kLoopGeneral)
     float4* ring = s_ring + warp_id() * kRing16;
@@ -1356,7 +1392,38 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
             tj[i] = t / n_mu;
             tk[i] = t - tj[i] * n_mu;
         }
-        for (int a = 0; a < nm; ++a) {
+        int a = 0;
+        if constexpr (kMasses > 1) {
+            const double wm = P.wmu[tk[0]], w = P.wq[tj[0]] * wm, wc = P.wqc[tj[0]] * wm;
+            for (; a < nm; a += kMasses) {           // a last group may be short
+                double v[2 * kMasses];
+#pragma unroll
+                for (int m = 0; m < kMasses; ++m) {
+                    const bool read = act[0] && a + m < nm;
+                    const double f = read ? relic_f_dev(P, qf[0] * P.mass_s[a + m]) : 0.0;
+                    v[2 * m] = read ? __dadd_rn(0.0, __dmul_rn(w, f)) : 0.0;
+                    v[2 * m + 1] = read ? __dadd_rn(0.0, __dmul_rn(wc, f)) : 0.0;
+                }
+                if (warp & 1) {
+#pragma unroll
+                    for (int j = 0; j < 2 * kMasses; ++j) s_half[warp >> 1][j][lane] = v[j];
+                }
+                __syncthreads();
+                if (!(warp & 1)) {
+#pragma unroll
+                    for (int j = 0; j < 2 * kMasses; ++j) v[j] += s_half[warp >> 1][j][lane];
+                    const double sum = warp_sums(v, lane);
+                    constexpr int kLanes = 16 / kMasses;         // that return one sum
+                    if (lane % kLanes == 0) s_red[warp >> 1][lane / kLanes] = sum;
+                }
+                __syncthreads();
+                if (threadIdx.x < 2 * min(kMasses, nm - a))
+                    part[2 * a + threadIdx.x] =
+                        sum_of_four(4, kRingThreads / kUnit, [&](int i) { return s_red[i][threadIdx.x]; });
+                __syncthreads();
+            }
+        }
+        for (; kMasses == 1 && a < nm; ++a) {
             const double sa = P.mass_s[a];
             double acc = 0.0, accc = 0.0;
 #pragma unroll
@@ -1524,8 +1591,8 @@ int launch_force_probe(int precision, const DevProblem* d_prob, int stage, const
 //   FP64: one trajectory a lane, in the smallest CTAs there are sums for, and of
 // those only as many on an SM as give each scheduler a warp: one keeps its FP64
 // unit busy, and work not yet started can go to an SM that is done early.  Six radii of
-// the precision sweep take 26.7 ms with 4 warps on an SM, 27.5 with 6, 31.6 with 8 and
-// 33.8 with 20; 27.2 in CTAs of 4 warps and 33.2 of 8.  Up to 5/3 such tiles for
+// the precision sweep take 25.5 ms with 4 warps on an SM, 26.0 with 6 and 30.5 with 8;
+// 26.1 in CTAs of 4 warps.  Up to 5/3 such tiles for
 // an SM a second pair of warps takes half of the force evaluations, one CTA on an SM: 16 to
 // 224 tiles of the plain workload 3.75-3.79 ms instead of 5.7-6.4, 256 tiles 4.3 instead of 6.5,
 // 304 tiles 6.6 against 6.5.
@@ -1548,7 +1615,7 @@ LaunchShape plan_shape(int precision, int tile, const LaunchSize& size)
         const long long w1 = (size.tiles128 + kSms - 1) / kSms, w2 = (size.tiles256 + kSms - 1) / kSms;
         const bool one = tile % kRingThreads == 0 && w2 <= kPackedCtas &&
                          std::max(440LL, 270 + 125 * w1) < std::max(500LL, 90 + 300 * w2);
-        s.kernel = one ? kRing : kPacked;
+        s.kernel = !one ? kPacked : size.most_masses > 1 ? kRingMasses : kRing;
         for (int t : {one ? kRingThreads : kPackedTile, 128, 64})
             if (tile % t == 0) {
                 s.tile = t;
@@ -1588,6 +1655,7 @@ static TrajKernel kernel_of(int kernel)
     switch (kernel) {
     case kPacked: return traj_kernel<float, 2, false, kLoopPacked>;
     case kRing: return traj_kernel<float, 1, false, kLoopRing>;
+    case kRingMasses: return traj_kernel<float, 1, false, kLoopRingMasses>;
     case kFp64: return traj_kernel<double, 1, false, kLoopFp64>;
     case kFp64Split: return traj_kernel<double, 1, false, kLoopFp64Split>;
     case kGeneralF32: return traj_kernel<float, 2, false, kLoopGeneral>;
@@ -1599,7 +1667,8 @@ static TrajKernel kernel_of(int kernel)
 // Shared memory of a CTA: its warps' windows on the table.
 static size_t ring_bytes(const LaunchShape& shape)
 {
-    return shape.kernel == kPacked || shape.kernel == kRing || shape.kernel == kFp64 ||
+    return shape.kernel == kPacked || shape.kernel == kRing ||
+                   shape.kernel == kRingMasses || shape.kernel == kFp64 ||
                    shape.kernel == kFp64Split
                ? (size_t)(shape.threads / 32) * kRing16 * sizeof(float4) : 0;
 }

@@ -51,6 +51,17 @@ CASES = {
 }
 
 
+# masses below, at and between multiples of the group that an epilogue takes at a time
+@pytest.mark.parametrize("n_mass", [3, 4, 5, 15])
+@pytest.mark.parametrize("change", [{}, {"n_q": 257, "n_mu": 1}, {"n_q": 3, "n_mu": 11}])
+def test_masses_of_a_small_launch_are_bitwise_the_counting_loop(n_mass, change):
+    pb = PLAIN.replace(radii=np.geomspace(1.0, 3000.0, 5), n_steps=60,
+                       masses=tuple(np.geomspace(0.01, 0.3, n_mass))).replace(**change)
+    assert pb.n_out == 5 * n_mass
+    for x, y in zip(*_both(pb, 256, 1)):
+        assert np.array_equal(x, y)
+
+
 # many radii of short runs: the launch is large enough for two trajectories a lane
 LARGE = PLAIN.replace(radii=np.geomspace(1.0, 3000.0, 300), n_steps=40)
 
