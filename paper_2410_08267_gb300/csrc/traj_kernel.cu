@@ -176,14 +176,16 @@ __device__ __forceinline__ double widen_f32(float v)
     return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
 }
 
-// y / u for 0 <= y < u and 1 <= u (6 FP64 operations).
+// y / u for y >= 0 and u = 1 + y as rounded (6 FP64 operations).
 __device__ __forceinline__ double quotient(double y, double u)
 {
     const double r0 = widen_f32(rcp_approx(trunc_f32(u)));   // 1/u to 2^-22
     const double e = fma(-u, r0, 1.0);
     const double r = fma(r0, fma(e, e, e), r0);               // to an ulp
     const double q = y * r;
-    return fma(fma(-q, u, y), r, q);                          // the remainder is exact
+    const double t = fma(fma(-q, u, y), r, q);                // the remainder is exact
+    // from u = 2^54 on the quotient rounds to 1; the seed ends with the float range
+    return less_nonneg(0x1p60, u) ? 1.0 : t;
 }
 
 template <int K>
