@@ -1165,6 +1165,8 @@ __device__ __forceinline__ double sum_of_four(int n, int have, Load load)
 //                coefficients were read ahead 5.75 ms, 5.95 with 64 registers, which
 //                spill, and 5.74 with 96 and 20 warps, but the uneven batch 27.5
 //                against 27.0 ms);
+//   kLoopPackedPasses  the same for tiles of more trajectories than a CTA holds
+//                (whole_tiles);
 //   kLoopRing    one trajectory per thread, for small launches (plan_shape);
 //   kLoopRingMasses  the same with an epilogue that takes kMassGroup masses at a time,
 //                for launches in which a request reads several: f and its sums in FP64
@@ -1178,18 +1180,20 @@ __device__ __forceinline__ double sum_of_four(int n, int have, Load load)
 //   kLoopFp64    one trajectory per thread;
 //   kLoopFp64Split  one trajectory in a lane of two warps (SplitPair): CTAs of four
 //                warps and 64 trajectories;
-//   kLoopGeneral one trajectory after another with the general force: with COUNT
-//                the counting variant of either mode.
-enum StepLoop { kLoopGeneral, kLoopPacked, kLoopRing, kLoopRingMasses, kLoopFp64, kLoopFp64Split };
+//   kLoopGeneral one trajectory after another with the general force: the counting
+//                variant of either mode.
+enum StepLoop { kLoopGeneral, kLoopPacked, kLoopPackedPasses, kLoopRing, kLoopRingMasses, kLoopFp64,
+                kLoopFp64Split };
 constexpr int kRingThreads = 128;
 constexpr int kMassGroup = 4;
+template <StepLoop LOOP> constexpr bool kTwo = LOOP == kLoopPacked || LOOP == kLoopPackedPasses;
 
 __device__ __forceinline__ int warp_id() { return threadIdx.x >> 5; }
 
 template <typename T, int TPT, bool COUNT, StepLoop LOOP>
 __global__ void __launch_bounds__(LOOP == kLoopGeneral ? 512
                                   : LOOP == kLoopRing || LOOP == kLoopRingMasses ? kRingThreads : 256,
-                                  LOOP == kLoopPacked ? 3 : 1)
+                                  kTwo<LOOP> ? 3 : 1)
 traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_prefix,
             int n_probs, int n_tiles, unsigned* __restrict__ ctrl,
             unsigned long long* __restrict__ tallies, QueueCtl* queue)
@@ -1271,7 +1275,7 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
         double* part = P.partials + ((size_t)seg * tps + tis) * 2 * nm;
 
         // one pass, but for a tile of more trajectories than the CTA holds
-        constexpr bool kPasses = LOOP == kLoopGeneral || LOOP == kLoopFp64;
+        constexpr bool kPasses = LOOP == kLoopGeneral || LOOP == kLoopFp64 || LOOP == kLoopPackedPasses;
         for (int base = 0; base < (kPasses ? P.tile : 1); base += blockDim.x * TPT) {
         T x[TPT], y[TPT], vx[TPT], vy[TPT];
         bool act[TPT];
@@ -1318,8 +1322,8 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
                       done, hc, ring, lane, pair);
             if (warp >> 1) act[0] = false;               // counted once
         } else if constexpr (LOOP != kLoopGeneral) {
-            using State = typename std::conditional<LOOP == kLoopPacked, TwoTrajectories, OneTrajectory>::type;
-            static_assert(TPT == (LOOP == kLoopPacked ? 2 : 1), "trajectories of a lane");
+            using State = typename std::conditional<kTwo<LOOP>, TwoTrajectories, OneTrajectory>::type;
+            static_assert(TPT == (kTwo<LOOP> ? 2 : 1), "trajectories of a lane");
             const HaloX2 h2{dup(hc.invIc), dup(-hc.invR3), hc.R2, hc.R, hc.c};
             const float4* tab4 = reinterpret_cast<const float4*>(tab);
             State st(x, y, vx, vy);
@@ -1630,7 +1634,10 @@ LaunchShape plan_shape(int precision, int tile, const LaunchSize& size)
 }
 
 // The same with CTAs that claim whole tiles, for callers without room for the sums
-// of smaller ones.
+// of smaller ones.  A mixed tile of more than 512 trajectories is integrated in passes
+// of four units, which leaves 24 warps on an SM: 300 radii x 262144 trajectories x 20
+// steps take 10.8 ms in tiles of 576 and 9.3 in tiles of 1024; one trajectory after
+// another with the branching force took 24.0 and 17.4.
 LaunchShape whole_tiles(int precision, int tile)
 {
     LaunchShape s;
@@ -1643,8 +1650,8 @@ LaunchShape whole_tiles(int precision, int tile)
         s.kernel = kPacked;
         s.threads = (tile + kUnit - 1) / kUnit * 32;
     } else {
-        s.kernel = kGeneralF32;
-        s.threads = 512;
+        s.kernel = kPackedPasses;
+        s.threads = kPackedTile / 2;
     }
     return s;
 }
@@ -1660,7 +1667,7 @@ static TrajKernel kernel_of(int kernel)
     case kRingMasses: return traj_kernel<float, 1, false, kLoopRingMasses>;
     case kFp64: return traj_kernel<double, 1, false, kLoopFp64>;
     case kFp64Split: return traj_kernel<double, 1, false, kLoopFp64Split>;
-    case kGeneralF32: return traj_kernel<float, 2, false, kLoopGeneral>;
+    case kPackedPasses: return traj_kernel<float, 2, false, kLoopPackedPasses>;
     case kCountF32: return traj_kernel<float, 2, true, kLoopGeneral>;
     default: return traj_kernel<double, 2, true, kLoopGeneral>;
     }
@@ -1669,10 +1676,7 @@ static TrajKernel kernel_of(int kernel)
 // Shared memory of a CTA: its warps' windows on the table.
 static size_t ring_bytes(const LaunchShape& shape)
 {
-    return shape.kernel == kPacked || shape.kernel == kRing ||
-                   shape.kernel == kRingMasses || shape.kernel == kFp64 ||
-                   shape.kernel == kFp64Split
-               ? (size_t)(shape.threads / 32) * kRing16 * sizeof(float4) : 0;
+    return (size_t)(shape.threads / 32) * kRing16 * sizeof(float4);   // (not the counting kernels)
 }
 
 int launch_traj(const LaunchShape& shape, int grid, const DevProblem* d_probs, const int* d_prefix,

@@ -1,0 +1,29 @@
+"""The kernels and tiles that plan_shape and whole_tiles choose give the bits of the
+other paths at the sizes where a rule changes over."""
+import numpy as np
+import pytest
+
+from paper_2410_08267_gb300 import nuprof as nu
+from paper_2410_08267_gb300 import workloads as W
+
+from gpu_common import require_gpu
+
+pytestmark = pytest.mark.gpu
+PLAIN = W.plain_small(precision=W.MIXED)[0]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def gpu():
+    return require_gpu()
+
+
+# the sums of 256-trajectory tiles of 260 radii exceed the static array; tiles of 576
+# and 960 trajectories end in a short pass, and 2^18 trajectories in a short tile
+@pytest.mark.parametrize("block", [288, 480, 512])
+def test_noalloc_wide_tiles_are_bitwise_the_handle_path(block):
+    pb = PLAIN.replace(radii=np.geomspace(1.0, 3000.0, 260), n_q=1024, n_mu=256, n_steps=2)
+    cosmo, halo, relic, radii, grid, opts = nu.structs(pb, torch_alloc=False, block=block, tpt=2)
+    got = nu.nu_profile_compute_noalloc(cosmo, halo, relic, radii, grid, opts)
+    want = nu.profile(pb, block=block, tpt=2)
+    for a, b in zip(got, want):
+        assert np.array_equal(a, b)
