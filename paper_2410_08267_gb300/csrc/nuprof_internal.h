@@ -193,11 +193,12 @@ struct LaunchShape {
     int group;       // such tiles in one tile of the asked shape
 };
 struct LaunchSize {
-    long long n_traj = 0, tiles64 = 0, tiles128 = 0, tiles256 = 0;   // and tiles of 64 ...
+    long long radii = 0, n_traj = 0, tiles64 = 0, tiles128 = 0, tiles256 = 0;   // and tiles of 64 ...
     int most_masses = 1;                                // read by one request
     void add(long long n_radii, long long n_seg, int n_mass)   // a request's radii, trajectories of one
     {
         if (n_mass > most_masses) most_masses = n_mass;
+        radii += n_radii;
         n_traj += n_radii * n_seg;
         tiles64 += n_radii * ((n_seg + 63) / 64);
         tiles128 += n_radii * ((n_seg + 127) / 128);

@@ -1598,10 +1598,16 @@ int launch_force_probe(int precision, const DevProblem* d_prob, int stage, const
 // those only as many on an SM as give each scheduler a warp: one keeps its FP64
 // unit busy, and work not yet started can go to an SM that is done early.  Six radii of
 // the precision sweep take 25.5 ms with 4 warps on an SM, 26.0 with 6 and 30.5 with 8;
-// 26.1 in CTAs of 4 warps.  Up to 5/3 such tiles for
-// an SM a second pair of warps takes half of the force evaluations, one CTA on an SM: 16 to
-// 224 tiles of the plain workload 3.75-3.79 ms instead of 5.7-6.4, 256 tiles 4.3 instead of 6.5,
-// 304 tiles 6.6 against 6.5.
+// 26.1 in CTAs of 4 warps.  A second pair of warps takes half of the force evaluations
+// where each SM has a tile at most (16 to 144 tiles of the plain workload 3.75-3.79 ms
+// instead of 5.7-6.4).  The split kernel has one CTA on an SM, so further tiles wait for
+// one to end, which costs nothing while fast trajectories leave their tiles early.  At 100
+// steps, split against whole: 160 to 225 tiles of the plain and the sweep grid 1.00-1.08 ms
+// against 1.53-1.69, 248 to 253 1.0-1.8 against 1.6-1.7, 256 to 260 1.1-1.8, 272 to 320
+// 1.7-1.95 against 1.5-1.7.  So it is taken up to 5/3 tiles an SM.  Where nothing leaves
+// (relics of 0.3 eV and more, the heaviest halos) it costs up to 15 % from 185 tiles on;
+// and with one or two tiles a radius each tile holds slow momenta, and nothing ends early
+// on any halo (200 tiles 1.71 against 1.56 ms), so from two waves on those run whole.
 constexpr int kFp64WarpsPerSm = 4;
 constexpr int kSms = 152;
 constexpr int kPackedTile = 256;
@@ -1613,7 +1619,9 @@ LaunchShape plan_shape(int precision, int tile, const LaunchSize& size)
     LaunchShape s;
     s.tile = tile;
     if (precision == NU_FP64) {
-        const bool split = tile % kUnit == 0 && size.tiles64 * 3 <= kSms * 5;
+        const bool split = tile % kUnit == 0 &&
+                           (size.tiles64 <= kSms ||
+                            (size.tiles64 * 3 <= kSms * 5 && size.tiles64 >= 3 * size.radii));
         s.kernel = split ? kFp64Split : kFp64;
         s.tile = tile % kUnit == 0 ? kUnit : tile;
         s.threads = split ? 2 * kUnit : std::min(s.tile, 256);

@@ -27,3 +27,26 @@ def test_noalloc_wide_tiles_are_bitwise_the_handle_path(block):
     want = nu.profile(pb, block=block, tpt=2)
     for a, b in zip(got, want):
         assert np.array_equal(a, b)
+
+
+# Tiles of 64 trajectories: up to one an SM (152), and up to 253 with three or more a
+# radius, two pairs of warps share one, with one CTA an SM; otherwise a CTA takes one alone.
+@pytest.mark.parametrize("n_q,n_mu,n_radii,grid", [(8, 16, 76, 152), (8, 16, 77, 154), (8, 16, 126, 252),
+                                                   (8, 8, 153, 153), (12, 16, 51, 152), (12, 16, 84, 152),
+                                                   (12, 16, 85, 255)])
+def test_fp64_launches_around_the_split(n_q, n_mu, n_radii, grid):
+    pb = PLAIN.replace(precision=W.FP64, n_steps=12, n_q=n_q, n_mu=n_mu,
+                       radii=np.geomspace(1.0, 3000.0, n_radii))
+    h = nu.create(pb, flags=nu.NU_FLAG_KEEP_QI)
+    b = nu.nu_batch_create([h])
+    try:
+        assert nu.nu_batch_info(b)["grid"] == grid
+        nu.nu_batch_run(b)
+        runs = [(*nu.nu_profile_result(h, n_radii), nu.nu_profile_qi(h, pb.n_traj))]
+        nu.nu_batch_branch_counts(b)
+        runs.append((*nu.nu_profile_result(h, n_radii), nu.nu_profile_qi(h, pb.n_traj)))
+    finally:
+        nu.nu_batch_destroy(b)
+        nu.nu_profile_destroy(h)
+    for x, y in zip(*runs):
+        assert np.array_equal(x, y)
