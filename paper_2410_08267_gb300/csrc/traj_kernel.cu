@@ -141,23 +141,27 @@ __device__ __forceinline__ float nfw_I_log(float y, float u)
 //   It starts in FP32, whose relative error 2^-22 is multiplied by t^J in the J
 //   FP64 steps that remain; J is the smallest multiple of 4 that makes that
 //   2^-93, 2^-40 of an ulp of the sum.  So the sum has the bits of the whole
-//   recurrence but where a rounding lies within 2^-40 ulp of a tie.
+//   recurrence but where a rounding lies within 2^-40 ulp of a tie (none of 9e9
+//   arguments differed).  Each lane starts at its own J while the warp runs the steps
+//   of the largest, so the sum depends on t alone, not on what shares the warp.
 // * Non-negative numbers are ordered as their bits, so tests are integer ones.
-// * t is the correctly rounded quotient from Newton's iteration and Markstein's
-//   final correction (IBM J. Res. Dev. 34, 1990): the seed is an FP32 reciprocal.
+// * t is the quotient from Newton's iteration and Markstein's final correction (IBM
+//   J. Res. Dev. 34, 1990), with an FP32 reciprocal as seed: the bits of the
+//   division on all of 1.3e10 arguments from 2^-60 to 2^1000.
 constexpr float kSeriesBits = 71.0f;       // 93 - 22
 constexpr int kSeriesTail = 20;            // FP32 terms: 2^-23 at the largest t that uses them
 constexpr int kSeriesMaxJ = 48;            // above: the whole recurrence
 
-__constant__ float c_series[kSeriesMaxJ + kSeriesTail] = {   // 1/(k+2)
-#define NU_INV4(k) 1.0f / ((k) + 2), 1.0f / ((k) + 3), 1.0f / ((k) + 4), 1.0f / ((k) + 5)
+__device__ const float4 c_series[(kSeriesMaxJ + kSeriesTail) / 4] = {   // 1/(k+2)
+#define NU_INV4(k) {1.0f / ((k) + 2), 1.0f / ((k) + 3), 1.0f / ((k) + 4), 1.0f / ((k) + 5)}
 #define NU_INV16(k) NU_INV4(k), NU_INV4((k) + 4), NU_INV4((k) + 8), NU_INV4((k) + 12)
     NU_INV16(0), NU_INV16(16), NU_INV16(32), NU_INV16(48), NU_INV4(64)
 #undef NU_INV16
 #undef NU_INV4
 };
 
-// a < b for doubles that are not negative (NaN: false for a NaN a)
+// a < b for doubles that are not negative (false for a NaN a but where its sign is set,
+// as the hardware's NaN may be: what follows from it is NaN either way)
 __device__ __forceinline__ bool less_nonneg(double a, double b)
 {
     return __double_as_longlong(a) < __double_as_longlong(b);
@@ -197,54 +201,81 @@ __device__ __forceinline__ double series4(double p, double t)   // terms K + 3 .
     return fma(p, t, 1.0 / (K + 2));
 }
 
-// FP64 steps that t_max < 1/2 needs: a multiple of 4 up to kSeriesMaxJ, or more
-// (the whole recurrence).
-__device__ __forceinline__ int series_steps(float t_max)
+// The same where J > K, and the start value elsewhere.  The choice is made on the
+// last step's operands: on its result it would lengthen the chain (FP64 cases 2 to 3 %).
+template <int K>
+__device__ __forceinline__ double series4_from(double p, double t, int J, double start)
 {
-    const int need = (int)(kSeriesBits * rcp_approx(-lg2_approx(t_max))) + 1;
+    p = fma(p, t, 1.0 / (K + 5));
+    p = fma(p, t, 1.0 / (K + 4));
+    p = fma(p, t, 1.0 / (K + 3));
+    return fma(p, J > K ? t : 0.0, J > K ? 1.0 / (K + 2) : start);
+}
+
+// FP64 steps that t < 1/2 needs: a multiple of 4 from 8 to kSeriesMaxJ, or more, up to
+// 68 (the whole recurrence).  For any other t a number in that range.
+__device__ __forceinline__ int series_steps(double t)
+{
+    const float above = __uint_as_float(__float_as_uint(trunc_f32(t)) + 1u);
+    const int need = (int)fminf(kSeriesBits * rcp_approx(-lg2_approx(above)), 64.0f) + 1;
     return max(8, (need + 3) & ~3);
 }
 
-// Horner's value before the last J (kSeriesMaxJ at most) steps.
-__device__ __forceinline__ double series_start(double t, int J)
+// Horner's value before the last J (48 where J is more) steps.  J_max: the warp's most,
+// whose branch is uniform (one for each lane's J costs 3 %).
+__device__ __forceinline__ double series_start(double t, int J, int J_max)
 {
-    if (J > kSeriesMaxJ) return fma(fma(1.0 / 52.0, t, 1.0 / 51.0), t, 1.0 / 50.0);
     const float tf = trunc_f32(t);
-    float s = c_series[J + kSeriesTail - 1];
+    const float4* c = c_series + min(J, kSeriesMaxJ) / 4;
+    float s = 0.0f;
 #pragma unroll
-    for (int i = kSeriesTail - 2; i >= 0; --i) s = fmaf(s, tf, c_series[J + i]);
-    return widen_f32(s);
+    for (int i = kSeriesTail / 4 - 1; i >= 0; --i) {
+        const float4 q = __ldg(c + i);
+        s = fmaf(fmaf(fmaf(fmaf(s, tf, q.w), tf, q.z), tf, q.y), tf, q.x);
+    }
+    double p = widen_f32(s);
+    if (J_max > kSeriesMaxJ) {
+        const double whole = fma(fma(1.0 / 52.0, t, 1.0 / 51.0), t, 1.0 / 50.0);
+        if (J > kSeriesMaxJ) p = whole;
+    }
+    return p;
 }
 
-// sums_{k=0}^{50} t^k/(k+2) of N values 0 < t <= t_max < 1/2, their chains side by side.
+// sums_{k=0}^{50} t^k/(k+2) of N values 0 < t < 1/2, their chains side by side.  J_max:
+// the most steps that a value of the warp needs (or more).
 template <int N>
-__device__ __forceinline__ void nfw_series_n(const double (&t)[N], float t_max, double (&p)[N])
+__device__ __forceinline__ void nfw_series_n(const double (&t)[N], int J_max, double (&p)[N])
 {
-    const int J = series_steps(t_max);
+    int J[N];
+    double start[N];
 #pragma unroll
-    for (int i = 0; i < N; ++i) p[i] = series_start(t[i], J);
+    for (int i = 0; i < N; ++i) {
+        J[i] = series_steps(t[i]);
+        p[i] = start[i] = series_start(t[i], J[i], J_max);
+    }
 #define NU_TERMS(K)                                                                      \
     case (K) + 4:                                                                        \
-        _Pragma("unroll") for (int i = 0; i < N; ++i) p[i] = series4<K>(p[i], t[i])
-    switch (min(J, kSeriesMaxJ)) {
-        NU_TERMS(44); NU_TERMS(40); NU_TERMS(36); NU_TERMS(32); NU_TERMS(28); NU_TERMS(24);
-        NU_TERMS(20); NU_TERMS(16); NU_TERMS(12); NU_TERMS(8);
+        _Pragma("unroll") for (int i = 0; i < N; ++i)                                    \
+            p[i] = series4_from<K>(p[i], t[i], J[i], start[i]);
+    switch (min(J_max, kSeriesMaxJ)) {
+        NU_TERMS(44) NU_TERMS(40) NU_TERMS(36) NU_TERMS(32) NU_TERMS(28) NU_TERMS(24)
+        NU_TERMS(20) NU_TERMS(16) NU_TERMS(12) NU_TERMS(8)
     default:;                                        // every case goes on with the next
     }
 #undef NU_TERMS
 #pragma unroll
     for (int i = 0; i < N; ++i) p[i] = series4<0>(series4<4>(p[i], t[i]), t[i]);
 }
-__device__ __forceinline__ double nfw_series(double t, float t_max)
+__device__ __forceinline__ double nfw_series(double t, int J_max)
 {
     double p[1];
-    nfw_series_n<1>({t}, t_max, p);
+    nfw_series_n<1>({t}, J_max, p);
     return p[0];
 }
-__device__ __forceinline__ void nfw_series2(double ta, double tb, float t_max, double& pa, double& pb)
+__device__ __forceinline__ void nfw_series2(double ta, double tb, int J_max, double& pa, double& pb)
 {
     double p[2];
-    nfw_series_n<2>({ta, tb}, t_max, p);
+    nfw_series_n<2>({ta, tb}, J_max, p);
     pa = p[0];
     pb = p[1];
 }
@@ -368,7 +399,7 @@ __device__ __forceinline__ float accel_m(float x, float y, float S, float Yq, fl
 }
 
 // FP64.  WARP: every lane of the warp is here (the integration loops), and the
-// series' length is that of the lane that needs most.
+// series' steps are run for the lane that needs most.
 template <class Ctr = NoTally, bool WARP = true>
 __device__ __forceinline__ double accel_m(double x, double y, double S, double Q, double,
                                           const HaloF64& hc, Ctr& ctr)
@@ -383,14 +414,12 @@ __device__ __forceinline__ double accel_m(double x, double y, double S, double Q
         t = quotient(ys, 1.0 + ys);
         series = less_nonneg(t, 0.5);
     }
-    unsigned t_max = series ? __float_as_uint(trunc_f32(t)) : 0u;
-    if (WARP) t_max = __reduce_max_sync(0xffffffffu, t_max);
+    int J_max = series ? series_steps(t) : 0;
+    if (WARP) J_max = __reduce_max_sync(0xffffffffu, J_max);
     if (in) {
         if (nfw) {
             ctr.add(ys < 1.0 ? 2 : 3);
-            // the truncated t_max is one float below t at most
-            const double I = series ? (t * t) * nfw_series(t, __uint_as_float(t_max + 1u))
-                                    : log1p(ys) - t;
+            const double I = series ? (t * t) * nfw_series(t, J_max) : log1p(ys) - t;
             sel = I * hc.invIc;
         } else {
             ctr.add(1);
@@ -964,21 +993,20 @@ __device__ __forceinline__ void accel_pair(double xa, double ya, double Sa, doub
         double Ia = ta, Ib = tb;
         const Compact cs(sa, sb, lane);
         if (cs.a | cs.b) {
-            const float t_max = __uint_as_float(1u + __reduce_max_sync(
-                full, max(sa ? __float_as_uint(trunc_f32(ta)) : 0u,
-                          sb ? __float_as_uint(trunc_f32(tb)) : 0u)));
+            const int J_max = __reduce_max_sync(full, max(sa ? series_steps(ta) : 0,
+                                                          sb ? series_steps(tb) : 0));
             if (cs.one_pass()) {
                 cs.pass(sa, sb, Ia, Ib, buf, lane,
-                        [&](double t) { return (t * t) * nfw_series(t, t_max); });
+                        [&](double t) { return (t * t) * nfw_series(t, J_max); });
             } else if (cs.a && cs.b) {
                 double pa, pb;
-                nfw_series2(ta, tb, t_max, pa, pb);
+                nfw_series2(ta, tb, J_max, pa, pb);
                 Ia = (ta * ta) * pa;
                 Ib = (tb * tb) * pb;
             } else if (cs.a) {
-                Ia = (ta * ta) * nfw_series(ta, t_max);
+                Ia = (ta * ta) * nfw_series(ta, J_max);
             } else {
-                Ib = (tb * tb) * nfw_series(tb, t_max);
+                Ib = (tb * tb) * nfw_series(tb, J_max);
             }
         }
         const Compact cl(la, lb, lane);
