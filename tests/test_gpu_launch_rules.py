@@ -29,6 +29,22 @@ def test_noalloc_wide_tiles_are_bitwise_the_handle_path(block):
         assert np.array_equal(a, b)
 
 
+def _normal_and_counting(pb, grid=None):
+    """n/nbar, error estimate and q_i of a run and of the counting launch."""
+    h = nu.create(pb, flags=nu.NU_FLAG_KEEP_QI)
+    b = nu.nu_batch_create([h])
+    try:
+        assert grid is None or nu.nu_batch_info(b)["grid"] == grid
+        nu.nu_batch_run(b)
+        runs = [(*nu.nu_profile_result(h, pb.n_out), nu.nu_profile_qi(h, pb.n_traj))]
+        nu.nu_batch_branch_counts(b)
+        runs.append((*nu.nu_profile_result(h, pb.n_out), nu.nu_profile_qi(h, pb.n_traj)))
+        return runs
+    finally:
+        nu.nu_batch_destroy(b)
+        nu.nu_profile_destroy(h)
+
+
 # Tiles of 64 trajectories: up to one an SM (152), and up to 253 with three or more a
 # radius, two pairs of warps share one, with one CTA an SM; otherwise a CTA takes one alone.
 @pytest.mark.parametrize("n_q,n_mu,n_radii,grid", [(8, 16, 76, 152), (8, 16, 77, 154), (8, 16, 126, 252),
@@ -37,16 +53,18 @@ def test_noalloc_wide_tiles_are_bitwise_the_handle_path(block):
 def test_fp64_launches_around_the_split(n_q, n_mu, n_radii, grid):
     pb = PLAIN.replace(precision=W.FP64, n_steps=12, n_q=n_q, n_mu=n_mu,
                        radii=np.geomspace(1.0, 3000.0, n_radii))
-    h = nu.create(pb, flags=nu.NU_FLAG_KEEP_QI)
-    b = nu.nu_batch_create([h])
-    try:
-        assert nu.nu_batch_info(b)["grid"] == grid
-        nu.nu_batch_run(b)
-        runs = [(*nu.nu_profile_result(h, n_radii), nu.nu_profile_qi(h, pb.n_traj))]
-        nu.nu_batch_branch_counts(b)
-        runs.append((*nu.nu_profile_result(h, n_radii), nu.nu_profile_qi(h, pb.n_traj)))
-    finally:
-        nu.nu_batch_destroy(b)
-        nu.nu_profile_destroy(h)
-    for x, y in zip(*runs):
+    for x, y in zip(*_normal_and_counting(pb, grid)):
         assert np.array_equal(x, y)
+
+
+# Two trajectories a lane (the launch fills the chip), and warps that stay out of the NFW
+# part for long: beyond R, grazing the shell, off the float range, without a halo.
+@pytest.mark.parametrize("change", [{"radii": np.geomspace(1500.0, 30000.0, 300)},
+                                    {"radii": np.geomspace(200.0, 1500.0, 300), "n_steps": 203},
+                                    {"radii": np.append(np.geomspace(900.0, 3000.0, 299), 1e25)},
+                                    {"radii": np.geomspace(900.0, 3000.0, 300), "c": 25.0, "z_end": 6.0},
+                                    {"M_h": 0.0}])
+def test_steps_outside_the_nfw_part_are_bitwise_the_counting_loop(change):
+    pb = PLAIN.replace(radii=np.geomspace(1.0, 3000.0, 300), n_steps=120, n_q=40).replace(**change)
+    for x, y in zip(*_normal_and_counting(pb)):
+        assert np.array_equal(x, y, equal_nan=True)
