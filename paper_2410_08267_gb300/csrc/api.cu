@@ -504,7 +504,8 @@ int nuprof::profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_
     // ---- host tables (FP64) ----
     const int nq = p_grid->n_q, nmu = p_grid->n_mu, N = o.n_steps;
     std::vector<double> q, wq, wqc, mu, wmu;
-    const std::shared_ptr<const CoefTable> coef = coef_table(*cosmo, *halo, d, N);
+    const std::shared_ptr<const CoefTable> coef = coef_table(*cosmo, *halo, d, N, o.precision);
+    const float* f32 = o.precision == NU_FP64 ? nullptr : coef->f32(N, d).data();
     log_nodes(nq, p_grid->q_min, p_grid->q_max, q, wq, wqc);
     gauss_legendre(nmu, mu, wmu);
     const double kT0 = kKB * cosmo->T0_K;                 // eV
@@ -619,7 +620,7 @@ int nuprof::profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_
             put<double>(stage, o_mu, mu.data(), nmu);
             put<double>(stage, o_smu, smu.data(), nmu);
         } else {
-            std::memcpy(stage + o_coef, coef->f32.data(), coef->f32.size() * sizeof(float));
+            std::memcpy(stage + o_coef, f32, (size_t)N * C_COUNT * sizeof(float));
             put<float>(stage, o_x0, x0.data(), n_radii);
             put<float>(stage, o_v0, v0.data(), nq);
             put<float>(stage, o_mu, mu.data(), nmu);

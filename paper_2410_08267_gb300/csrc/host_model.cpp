@@ -294,7 +294,7 @@ static std::shared_ptr<const std::vector<StageBackground>> background(const nu_c
 }
 
 std::shared_ptr<const CoefTable> coef_table(const nu_cosmo& cosmo, const nu_halo& halo,
-                                            const Derived& d, int n_steps)
+                                            const Derived& d, int n_steps, int precision)
 {
     constexpr size_t kKept = 8;
     static std::mutex mu;
@@ -311,14 +311,24 @@ std::shared_ptr<const CoefTable> coef_table(const nu_cosmo& cosmo, const nu_halo
     }
     auto tab = std::make_shared<CoefTable>();
     tab->f64.resize((size_t)n_steps * C_COUNT);
-    tab->f32.resize((size_t)n_steps * C_COUNT);
     coef_table_into(cosmo, halo, d, n_steps, tab->f64.data(),
                     background(cosmo, d, n_steps)->data());
-    fp32_table(tab->f64.data(), n_steps, d, tab->f32.data());
+    if (precision != NU_FP64) tab->f32(n_steps, d);
     std::lock_guard<std::mutex> g(mu);
     if (kept.size() == kKept) kept.erase(kept.begin());
     kept.emplace_back(key, tab);
     return tab;
+}
+
+const std::vector<float>& CoefTable::f32(int n_steps, const Derived& d) const
+{
+    std::lock_guard<std::mutex> g(mu);                   // (a once_flag wakes waiters by a system call)
+    if (image32.empty()) {
+        std::vector<float> image(f64.size());
+        fp32_table(f64.data(), n_steps, d, image.data());
+        image32.swap(image);
+    }
+    return image32;
 }
 
 // |P| nodes: log-spaced on [q_min, q_max]; the integral of P^2 f dP is taken

@@ -68,3 +68,18 @@ def test_steps_outside_the_nfw_part_are_bitwise_the_counting_loop(change):
     pb = PLAIN.replace(radii=np.geomspace(1.0, 3000.0, 300), n_steps=120, n_q=40).replace(**change)
     for x, y in zip(*_normal_and_counting(pb)):
         assert np.array_equal(x, y, equal_nan=True)
+
+
+def test_kept_tables_serve_both_precisions():
+    """A halo's kept table, first made for a request of either mode, then read by the
+    other, gives the results of a table made afresh."""
+    mixed = PLAIN.replace(M_h=1.7e12, radii=np.array([4.0, 60.0]), n_q=16, n_mu=8, n_steps=50)
+    both = [mixed, mixed.replace(precision=W.FP64)]
+    fresh = {}
+    for order in (both, both[::-1]):
+        for k in range(9):                          # as many halos as tables are kept, and one
+            nu.profile(mixed.replace(M_h=3e12 + 1e10 * k))
+        for pb in order:
+            got = nu.profile(pb)
+            for a, b in zip(got, fresh.setdefault(int(pb.precision), got)):
+                assert np.array_equal(a, b)
