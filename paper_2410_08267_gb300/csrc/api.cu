@@ -326,9 +326,9 @@ private:
         static std::mutex m;
         return m;
     }
-    static Pool& pool()
-    {
-        static Pool p;
+    static Pool& pool()                                   // never destroyed: a program may give
+    {                                                     // its handles back while it exits
+        static Pool& p = *new Pool;
         return p;
     }
 };
