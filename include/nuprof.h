@@ -65,7 +65,7 @@ extern "C" {
 #define NU_ECUDA      -3   /* a CUDA runtime call failed (no GPU, launch error) */
 #define NU_EBUSY      -4   /* result asked for before any run was enqueued     */
 #define NU_ETIMEDOUT  -5   /* a bounded wait ran out                           */
-#define NU_EDEVICE    -6   /* the device status word reports a non-finite sum  */
+#define NU_EDEVICE    -6   /* a result of the device is not finite             */
 #define NU_ENOTSUP    -7   /* valid but unsupported combination                */
 #define NU_ECANCELED  -8   /* serving: the request was cancelled               */
 #define NU_EAGAIN     -9   /* serving: the request is not finished yet         */

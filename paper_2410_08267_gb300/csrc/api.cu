@@ -583,7 +583,6 @@ int nuprof::profile_create(const nu_cosmo* cosmo, const nu_halo* halo, const nu_
     if (host_results) h->host_out = HostResults::take((size_t)2 * nm * n_radii);
     P.host_out = h->host_out;
     P.qi = keep_qi ? static_cast<void*>(base + o_qi) : nullptr;
-    P.status = reinterpret_cast<int*>(base + o_ctrl) + kCtrlStatus;
     P.q_scale = relic->m_eV / (kC * kT0);                 // Liouville map: q_i = m |v| / (c k_B T0)
     P.invIc = 1.0 / d.Ic;
     P.invR3 = d.R > 0.0 ? 1.0 / (d.R * d.R * d.R) : 0.0;

@@ -94,9 +94,9 @@ void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w);
 void resolve_opts(const nu_opts* in, nu_opts& out);
 long long device_bytes(int precision, int n_steps, int n_radii, int n_q, int n_mu,
                        int tiles_per_seg, bool keep_qi, int n_mass, int n_ftab, long long* h2d_bytes);
-// Control words of a launch: the next tile to claim, the status, the CTAs that have
-// left.  Zero before the first launch; each launch leaves them so.
-enum CtrlWord { kCtrlNext = 0, kCtrlStatus, kCtrlLeft, kCtrlWords = 4 };
+// Control words of a launch: the next tile to claim and the CTAs that have left.  Zero
+// before the first launch; each launch leaves them so.
+enum CtrlWord { kCtrlNext = 0, kCtrlLeft, kCtrlWords = 4 };
 // Number of masses read from one trajectory set (Sec. III mass reuse).
 inline int relic_n_mass(const nu_relic& r) { return r.n_masses > 0 ? r.n_masses : 1; }
 
@@ -118,7 +118,6 @@ struct DevProblem {
     double* err;            // [n_mass][n_radii] relative quadrature-error estimate
     double* host_out;       // out and err once more, in mapped host memory (optional)
     void* qi;               // [n_radii][n_q][n_mu] final q in the state precision (optional)
-    int* status;            // bit 0: non-finite sums so far
     double q_scale;         // q_i = |v| * q_scale (fiducial mass)
     double invIc, invR3, R2;
     double c_nfw;           // concentration: the NFW edge in y = r / (r_s (1+z))

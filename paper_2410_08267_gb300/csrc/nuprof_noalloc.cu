@@ -218,7 +218,6 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
     P.out = reinterpret_cast<double*>(dev + o_out);
     P.err = reinterpret_cast<double*>(dev + o_err);
     P.qi = nullptr;
-    P.status = reinterpret_cast<int*>(dev + o_ctrl) + kCtrlStatus;
     P.q_scale = relic->m_eV / (kC * kT0);
     P.invIc = 1.0 / d.Ic;
     P.invR3 = d.R > 0.0 ? 1.0 / (d.R * d.R * d.R) : 0.0;

@@ -1189,7 +1189,7 @@ __device__ int queue_wait(QueueCtl* q, unsigned g, int* n_probs)
 // into ones of a unit, two or four gives the same bits.
 constexpr int kUnit = 64;
 
-// Sums over the warp of N (2 or 8) values a lane, each by warp_sum's tree: at every
+// Sums over the warp of N values a lane (2 kMassGroup), each by warp_sum's tree: at every
 // level the lanes of one half hand over the values that the other half goes on with,
 // so 8 sums take 9 FP64 additions a lane where one after another they take 40.
 // Lane l returns the sum of value l N / 32.
@@ -1577,7 +1577,6 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
                         P.host_out[(size_t)a * P.n_radii + seg] = ratio;
                         P.host_out[(size_t)(nm + a) * P.n_radii + seg] = err;
                     }
-                    if (!isfinite(ratio)) atomicOr(P.status, 1);
                 }
             }
             if (lane == 0) {
