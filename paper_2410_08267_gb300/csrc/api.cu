@@ -73,18 +73,6 @@ struct RunEvent {
     }
 };
 
-int sm_count()
-{
-    static std::atomic<int> cached{0};
-    int v = cached.load();
-    if (v) return v;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    cached.store(v);
-    return v;
-}
-
 int persistent_grid(const LaunchShape& shape, int n_tiles, int* grid)
 {
     int per_sm = 0;

@@ -229,7 +229,8 @@ int launch_traj(const LaunchShape& shape, int grid, const DevProblem* d_probs,
 int launch_traj_tally(int precision, const LaunchShape& shape, int grid, const DevProblem* d_probs,
                       const int* d_tile_prefix, int n_probs, int n_tiles, unsigned* d_tile_counter,
                       unsigned long long* d_tallies, void* stream);
-int max_ctas_per_sm(const LaunchShape& shape, int* out);
+int max_ctas_per_sm(const LaunchShape& shape, int* out);   // on the current device
+int sm_count();                                            // of the current device; 0: none
 // Smallest tile (block 64 x 1 trajectory): request buffers of tile sums are
 // sized for it, so a batch may run any tile shape over existing requests.
 constexpr int kMinTile = 64;

@@ -1671,24 +1671,36 @@ int launch_force_probe(int precision, const DevProblem* d_prob, int stage, const
 // and with one or two tiles a radius each tile holds slow momenta, and nothing ends early
 // on any halo (200 tiles 1.71 against 1.56 ms), so from two waves on those run whole.
 constexpr int kFp64WarpsPerSm = 4;
-constexpr int kSms = 152;
 constexpr int kPackedTile = 256;
 constexpr int kPackedCtas = 6;                       // on an SM
+constexpr int kDevices = 32;                         // whose properties are kept
+
+int sm_count()
+{
+    static std::atomic<int> kept[kDevices];
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (dev < kDevices && (n = kept[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    if (dev < kDevices) kept[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
 
 LaunchShape plan_shape(int precision, int tile, const LaunchSize& size)
 {
     if (size.n_traj > (1LL << 35)) return whole_tiles(precision, tile);   // few enough to count
+    const long long sms = std::max(1, sm_count());
     LaunchShape s;
     s.tile = tile;
     if (precision == NU_FP64) {
         const bool split = tile % kUnit == 0 &&
-                           (size.tiles64 <= kSms ||
-                            (size.tiles64 * 3 <= kSms * 5 && size.tiles64 >= 3 * size.radii));
+                           (size.tiles64 <= sms ||
+                            (size.tiles64 * 3 <= sms * 5 && size.tiles64 >= 3 * size.radii));
         s.kernel = split ? kFp64Split : kFp64;
         s.tile = tile % kUnit == 0 ? kUnit : tile;
         s.threads = split ? 2 * kUnit : std::min(s.tile, 256);
     } else {
-        const long long w1 = (size.tiles128 + kSms - 1) / kSms, w2 = (size.tiles256 + kSms - 1) / kSms;
+        const long long w1 = (size.tiles128 + sms - 1) / sms, w2 = (size.tiles256 + sms - 1) / sms;
         const bool one = tile % kRingThreads == 0 && w2 <= kPackedCtas &&
                          std::max(440LL, 270 + 125 * w1) < std::max(500LL, 90 + 300 * w2);
         s.kernel = !one ? kPacked : size.most_masses > 1 ? kRingMasses : kRing;
@@ -1778,16 +1790,18 @@ int launch_traj_tally(int precision, const LaunchShape& shape, int grid, const D
 
 int max_ctas_per_sm(const LaunchShape& shape, int* out)
 {
-    // asked for by every run: kept, as the GPUs of a process are taken to be alike
-    static std::atomic<int> kept[kKernelKinds][512 / 32 + 1];
-    std::atomic<int>& known = kept[shape.kernel][shape.threads / 32];
-    if ((*out = known.load(std::memory_order_relaxed)) > 0) return NU_OK;
+    // asked for by every run: kept for each device
+    static std::atomic<int> kept[kDevices][kKernelKinds][512 / 32 + 1];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return NU_ECUDA;
+    std::atomic<int>* known = dev < kDevices ? &kept[dev][shape.kernel][shape.threads / 32] : nullptr;
+    if (known && (*out = known->load(std::memory_order_relaxed)) > 0) return NU_OK;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kernel_of(shape.kernel), shape.threads,
                                                       ring_bytes(shape)) != cudaSuccess)
         return NU_ECUDA;
     if (shape.kernel == kFp64 || shape.kernel == kFp64Split)
         *out = std::min(*out, std::max(1, kFp64WarpsPerSm * 32 / shape.threads));
-    known.store(*out, std::memory_order_relaxed);
+    if (known) known->store(*out, std::memory_order_relaxed);
     return NU_OK;
 }
 
