@@ -1657,19 +1657,20 @@ int launch_force_probe(int precision, const DevProblem* d_prob, int stage, const
 // and 109 / 143 / 146 / 202 / 260 / 353 / 411 us packed).  The cheaper one is taken; a
 // launch that fills the chip runs packed.
 //   FP64: one trajectory a lane, in the smallest CTAs there are sums for, and of
-// those only as many on an SM as give each scheduler a warp: one keeps its FP64
+// those the fewest on an SM that give each scheduler a warp: one keeps its FP64
 // unit busy, and work not yet started can go to an SM that is done early.  Six radii of
 // the precision sweep take 25.5 ms with 4 warps on an SM, 26.0 with 6 and 30.5 with 8;
-// 26.1 in CTAs of 4 warps.  A second pair of warps takes half of the force evaluations
-// where each SM has a tile at most (16 to 144 tiles of the plain workload 3.75-3.79 ms
-// instead of 5.7-6.4).  The split kernel has one CTA on an SM, so further tiles wait for
-// one to end, which costs nothing while fast trajectories leave their tiles early.  At 100
-// steps, split against whole: 160 to 225 tiles of the plain and the sweep grid 1.00-1.08 ms
-// against 1.53-1.69, 248 to 253 1.0-1.8 against 1.6-1.7, 256 to 260 1.1-1.8, 272 to 320
-// 1.7-1.95 against 1.5-1.7.  So it is taken up to 5/3 tiles an SM.  Where nothing leaves
-// (relics of 0.3 eV and more, the heaviest halos) it costs up to 15 % from 185 tiles on;
-// and with one or two tiles a radius each tile holds slow momenta, and nothing ends early
-// on any halo (200 tiles 1.71 against 1.56 ms), so from two waves on those run whole.
+// 26.1 in CTAs of 4 warps; in tiles of 96 26.6 with 6 warps and 31.7 with 3.
+//   A second pair of warps takes half of the force evaluations where each SM has a tile
+// at most (16 to 144 tiles of the plain workload 3.75-3.79 ms instead of 5.7-6.4).  The
+// split kernel has one CTA on an SM, so further tiles wait for one to end, which costs
+// nothing while fast trajectories leave their tiles early.  At 100 steps, split against
+// whole: 160 to 225 tiles of the plain and the sweep grid 1.00-1.08 ms against 1.53-1.69,
+// 248 to 253 1.0-1.8 against 1.6-1.7, 256 to 260 1.1-1.8, 272 to 320 1.7-1.95 against
+// 1.5-1.7.  So it is taken up to 5/3 tiles an SM.  Where nothing leaves (relics of 0.3 eV
+// and more, the heaviest halos) it costs up to 15 % from 185 tiles on; and with one or two
+// tiles a radius each tile holds slow momenta, and nothing ends early on any halo (200
+// tiles 1.71 against 1.56 ms), so from two waves on those run whole.
 constexpr int kFp64WarpsPerSm = 4;
 constexpr int kPackedTile = 256;
 constexpr int kPackedCtas = 6;                       // on an SM
@@ -1800,7 +1801,7 @@ int max_ctas_per_sm(const LaunchShape& shape, int* out)
                                                       ring_bytes(shape)) != cudaSuccess)
         return NU_ECUDA;
     if (shape.kernel == kFp64 || shape.kernel == kFp64Split)
-        *out = std::min(*out, std::max(1, kFp64WarpsPerSm * 32 / shape.threads));
+        *out = std::min(*out, (kFp64WarpsPerSm * 32 + shape.threads - 1) / shape.threads);
     if (known) known->store(*out, std::memory_order_relaxed);
     return NU_OK;
 }

@@ -57,6 +57,19 @@ def test_fp64_launches_around_the_split(n_q, n_mu, n_radii, grid):
         assert np.array_equal(x, y)
 
 
+# FP64 CTAs on an SM: the fewest that give each of its four schedulers a warp
+@pytest.mark.parametrize("block,ctas", [(64, 2), (96, 2), (160, 1), (256, 2), (480, 1)])
+def test_fp64_ctas_of_a_large_launch(block, ctas):
+    pb = PLAIN.replace(precision=W.FP64, n_steps=2, radii=np.geomspace(1.0, 3000.0, 200))
+    h = nu.create(pb, block=block)
+    b = nu.nu_batch_create([h])
+    try:
+        assert nu.nu_batch_info(b)["grid"] == ctas * 152
+    finally:
+        nu.nu_batch_destroy(b)
+        nu.nu_profile_destroy(h)
+
+
 # Two trajectories a lane (the launch fills the chip), and warps that stay out of the NFW
 # part for long: beyond R, grazing the shell, off the float range, without a halo.
 @pytest.mark.parametrize("change", [{"radii": np.geomspace(1500.0, 30000.0, 300)},
