@@ -320,13 +320,14 @@ NU_API int nu_batch_kernel_ms(nu_batch* b, float* ms);
  * NU_EINVAL, NU_ENOMEM, NU_ECUDA. */
 NU_API int nu_batch_branch_counts(nu_batch* b, void* stream, long long* counts);
 
-/* Launch-shape autotuner: times the batch of requests `hs` with each candidate
- * shape (block x tpt: 256x1, 512x1, 256x2, 256x1, 384x1, and for mixed precision
- * 256x3, 128x3, 256x3, some of them with NU_FLAG_GTAB; one warm-up and the median
- * of three runs) and reports the fastest.  The library chooses the kernel and its
- * threads by itself, so shapes of one tile run alike.  With cache_path != NULL, a JSON-lines cache keyed by GPU name,
- * precision, step-count and trajectory-count buckets (powers of two) is read
- * first and appended to after tuning.  Results of different shapes agree to
+/* Launch-shape autotuner: times the batch of requests `hs` with the tile of each
+ * candidate shape (block x tpt: 256x1, 512x1, 256x2, 256x1, 384x1, and for mixed
+ * precision 256x3, 128x3, 256x3, some of them with NU_FLAG_GTAB; one warm-up and the
+ * median of three runs) and reports the fastest.  The library chooses the kernel and
+ * its threads by itself, so shapes of one tile are one launch: they are timed once,
+ * and the first of them stands for its tile.  With cache_path != NULL, a JSON-lines
+ * cache keyed by GPU name, precision, step-count and trajectory-count buckets (powers
+ * of two) is read first and appended to after tuning.  Results of different shapes agree to
  * rounding, not bit for bit (the reduction order changes).  All requests must
  * share a precision.  Errors: NU_EINVAL, NU_ENOMEM, NU_ECUDA. */
 typedef struct nu_tune_result {

@@ -96,3 +96,19 @@ def test_kept_tables_serve_both_precisions():
             got = nu.profile(pb)
             for a, b in zip(got, fresh.setdefault(int(pb.precision), got)):
                 assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("precision,n", [(W.MIXED, 8), (W.FP64, 5)])
+def test_autotune_takes_shapes_of_one_tile_for_one_launch(precision, n):
+    pb = PLAIN.replace(precision=precision, n_steps=20)
+    h = nu.create(pb)
+    try:
+        r = nu.nu_autotune([h])
+    finally:
+        nu.nu_profile_destroy(h)
+    by_tile = {}
+    for block, tpt, flags, ms in r["candidates"]:
+        by_tile.setdefault(block * min(tpt, 2), []).append((ms, block, tpt, flags))
+    assert len(r["candidates"]) == n and set(by_tile) == {256, 384, 512}
+    assert all(len({c[0] for c in same}) == 1 for same in by_tile.values())
+    assert (r["best_ms"], r["block"], r["tpt"], r["flags"]) in [same[0] for same in by_tile.values()]
