@@ -186,14 +186,17 @@ void put(unsigned char* buf, size_t off, const double* v, size_t n)
     for (size_t i = 0; i < n; ++i) p[i] = (T)v[i];
 }
 
-// Page-locked host staging for the uploads of create and the reads of
-// result: one process-wide buffer that grows to the largest request, held
-// under a lock for one copy at a time (copies from page-locked memory run
-// as true DMA, without the driver's intermediate bounce).  If page-locked
-// memory cannot be had, an ordinary heap buffer is used instead.
-class Stage {
+// Page-locked host staging: one process-wide buffer a use that grows to the largest
+// request, held under a lock for one copy at a time (copies from page-locked memory run
+// as true DMA, without the driver's intermediate bounce).  If page-locked memory cannot
+// be had, an ordinary heap buffer is used instead.  Uses: the uploads of create and the
+// reads of result; the reads of the momenta, which may take long and would keep others
+// from creating requests.
+enum StageUse { kStageRequests, kStageMomenta };
+template <StageUse USE>
+class StageOf {
 public:
-    explicit Stage(size_t bytes) : lk_(mu())
+    explicit StageOf(size_t bytes) : lk_(mu())
     {
         Buf& b = buf();
         if (b.cap < bytes) {
@@ -239,6 +242,9 @@ private:
     std::vector<unsigned char> heap_;
     unsigned char* p_ = nullptr;
 };
+using Stage = StageOf<kStageRequests>;
+using MomentaStage = StageOf<kStageMomenta>;
+constexpr long long kMomentaPart = 1LL << 20;        // read at a time
 
 // Page-locked, mapped host memory in which the kernel leaves results besides device
 // memory, so that reading them takes no copy (a copy of 10 values costs the
@@ -350,7 +356,11 @@ int staging_reserve(size_t bytes)
     return Stage::capacity() >= bytes ? NU_OK : NU_ENOMEM;
 }
 
-void host_results_reserve() { HostResults::give(HostResults::take(1)); }
+void host_results_reserve()
+{
+    HostResults::give(HostResults::take(1));
+    MomentaStage st((size_t)kMomentaPart * sizeof(float));
+}
 
 const DevProblem& profile_desc(const nu_profile* h) { return h->hdp; }
 nu_profile* profile_twin(const nu_profile* h) { return h->twin; }
@@ -734,8 +744,8 @@ int nu_profile_qi(nu_profile* h, double* qi, long long n)
         return NU_OK;
     }
     // through the page-locked buffer a part at a time, widened from there
-    const long long part = std::min(total, 1LL << 20);
-    Stage staging((size_t)part * sizeof(float));
+    const long long part = std::min(total, kMomentaPart);
+    MomentaStage staging((size_t)part * sizeof(float));
     const float* tmp = reinterpret_cast<const float*>(staging.data());
     for (long long at = 0; at < total; at += part) {
         const long long m = std::min(part, total - at);

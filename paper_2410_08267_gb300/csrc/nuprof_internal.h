@@ -179,7 +179,7 @@ int profile_read(const nu_profile* h, double* out, double* err, void* stream);
 // the host).
 size_t staging_capacity();
 int staging_reserve(size_t bytes);
-void host_results_reserve();   // page-lock the block of results in host memory
+void host_results_reserve();   // page-lock what results and momenta are read through
 // NU_FLAG_VERIFY: the FP64 twin of a handle (nullptr without the flag), a
 // launch of the twin alone with an event after it, and a query of that event
 // (NU_OK done, NU_EAGAIN running, NU_EBUSY never run, NU_ECUDA).

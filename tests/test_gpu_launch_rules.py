@@ -1,5 +1,8 @@
 """The kernels and tiles that plan_shape and whole_tiles choose give the bits of the
-other paths at the sizes where a rule changes over."""
+other paths at the sizes where a rule changes over, and what calls share in the host's
+memory does not tie them to one another."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -112,3 +115,24 @@ def test_autotune_takes_shapes_of_one_tile_for_one_launch(precision, n):
     assert len(r["candidates"]) == n and set(by_tile) == {256, 384, 512}
     assert all(len({c[0] for c in same}) == 1 for same in by_tile.values())
     assert (r["best_ms"], r["block"], r["tpt"], r["flags"]) in [same[0] for same in by_tile.values()]
+
+
+def test_requests_are_created_while_momenta_are_read():
+    """Reading 6e7 momenta takes a tenth of a second or more; a request is created in
+    some 50 us, in another thread, meanwhile."""
+    pb = PLAIN.replace(radii=np.geomspace(1.0, 300.0, 60), n_q=2000, n_mu=512, n_steps=1)
+    h = nu.create(pb, flags=nu.NU_FLAG_KEEP_QI)
+    try:
+        nu.nu_profile_run(h)
+        nu.nu_profile_result(h, pb.n_out)
+        reader = threading.Thread(target=nu.nu_profile_qi, args=(h, pb.n_traj))
+        nu.nu_profile_destroy(nu.create(PLAIN))
+        reader.start()
+        created = 0
+        while reader.is_alive():
+            nu.nu_profile_destroy(nu.create(PLAIN))
+            created += 1
+        reader.join()
+        assert created > 50
+    finally:
+        nu.nu_profile_destroy(h)
