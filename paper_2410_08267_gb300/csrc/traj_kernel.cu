@@ -1275,7 +1275,10 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
     __shared__ double s_red[16][2 * kMasses];
     __shared__ double s_half[TPT == 1 ? (kMasses > 1 ? 2 : 8) : 1][2 * kMasses][32];
     __shared__ double s_pass[LOOP == kLoopFp64 ? 8 : LOOP == kLoopFp64Split ? 8 : 1][32];
-    extern __shared__ __align__(16) float4 s_ring[];   // kRing16 words a warp (not kLoopGeneral)
+    // kRing16 words a warp (not kLoopGeneral).  From 16 bytes past a multiple of 32 on the
+    // copies into it take longer, seen where little else is done: 614,000 trajectories
+    // without a halo 111 us, 83 at 32 and 64 bytes, 76 at 128.
+    extern __shared__ __align__(128) float4 s_ring[];
     float4* ring = s_ring + warp_id() * kRing16;
 
     const int lane = threadIdx.x & 31;
