@@ -56,8 +56,8 @@ FLOPS_EVAL = (3, 8, 15, 15)
 FLOPS_COMBINE = 61
 FLOPS_FULL = 121
 SMS, FP32_LANES_PER_SM = 152, 128
-# DRAM bytes (read + write) per launch of the trajectory kernel at the tuned
-# this workload (every shape runs the same kernel): mean of two launches of one ncu capture
+# DRAM bytes (read + write) per launch of the trajectory kernel on this workload (every
+# shape runs the same kernel): mean of two launches of one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum), recorded in
 # profiles/traj_kernel_precision_sweep_mixed.md.  Must be reset to None
 # whenever the kernel changes, until it is captured again.
@@ -595,7 +595,6 @@ def bench_ours(args):
                 "flops_per_launch": flops, "flops_per_executed_traj_step": flops / live_steps,
                 "executed_traj_steps": live_steps,
                 "finished_early_frac": 1.0 - live_steps / traj_steps,
-                "lane_steps_run": counts[5], "needed_lane_frac": live_steps / counts[5],
                 "branch_counts": {"beyond_R": counts[0], "shell": counts[1],
                                   "nfw_rational_or_series": counts[2], "nfw_log": counts[3]},
                 "full_eval_equiv_tflops": FLOPS_FULL * traj_steps / (kms / 1e3) / 1e12,

@@ -310,11 +310,12 @@ NU_API int nu_batch_kernel_ms(nu_batch* b, float* ms);
  * y < 1), counts[3] on its logarithm branch, counts[4]
  * trajectory-steps integrated.  A trajectory is finished once its velocity
  * can no longer change (it lies beyond R on a line that does not re-enter
- * before z_end): its remaining steps are not needed work (its warp stops when
- * all of its lanes are finished; the test runs every 4 steps, so up to 3 steps
- * past the finish are counted).  counts[5] is every lane-step that the warps
- * ran, finished trajectories and padding lanes included, so counts[4] /
- * counts[5] is the fraction of lane-steps doing needed work.  The force is
+ * before z_end): its remaining steps are not needed work (the counting launch
+ * tests for it every 4 steps, so up to 3 steps past the finish are counted).
+ * counts[5] is every lane-step that the warps of the counting launch ran,
+ * finished trajectories and padding lanes included; other launches put the
+ * trajectories into other warps, test at other steps and repeat a few steps,
+ * so theirs is another number.  The force is
  * data dependent (App. A has three branches), so these counts turn one run
  * into an exact algorithmic flop count.  counts must hold 6 values.  Errors:
  * NU_EINVAL, NU_ENOMEM, NU_ECUDA. */

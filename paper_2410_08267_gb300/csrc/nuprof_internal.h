@@ -190,7 +190,9 @@ int profile_twin_query(const nu_profile* h);
 // Kernel launch helpers (traj_kernel.cu).  A request's or batch's shape
 // (nu_opts.block x tpt) fixes its tile, whose sums are added in order, and so the
 // rounding of its results; how a launch runs such tiles is chosen by plan_shape.
-enum TrajKernelKind { kPacked, kPackedPasses, kRing, kRingMasses, kFp64, kFp64Split, kCountF32, kCountF64, kKernelKinds };
+enum TrajKernelKind {
+    kPacked, kPackedFew, kPackedPasses, kRing, kRingMasses, kFp64, kFp64Split, kCountF32, kCountF64, kKernelKinds
+};
 struct LaunchShape {
     int kernel;      // TrajKernelKind
     int threads;     // of a CTA

@@ -91,7 +91,7 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
     nu_opts o;
     resolve_opts(opts, o);
     if (o.flags != 0 || o.timeout_ms < 0.0) return NU_EINVAL;
-    if (o.tpt == kTptPacked) return NU_ENOTSUP;   // scalar shapes only
+    if (o.tpt == kTptPacked) return NU_ENOTSUP;   // tpt 2 names the same tiles
     if (relic && relic->n_masses > 0) return NU_ENOTSUP;   // one mass per call
     if (relic && relic->f_kind == NU_F_TABLE) return NU_ENOTSUP;   // closed-form f only
     int rc = validate(cosmo, halo, relic, radii, n_radii, p_grid, &o);
@@ -267,8 +267,8 @@ extern "C" int nu_profile_compute_noalloc(const nu_cosmo* cosmo, const nu_halo* 
     const int grid = n_tiles < per_sm * sms ? n_tiles : per_sm * sms;
 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    // The array keeps the previous call's contents: the control words are part of the zeroed upload and the per-radius
-    // completion counters are cleared explicitly.
+    // The array keeps the previous call's contents: the control words are part of the
+    // zeroed upload and the per-radius completion counters are cleared explicitly.
     if (cudaMemcpyAsync(dev, st, upload_end, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemsetAsync(dev + o_cnt, 0, (size_t)n_radii * sizeof(unsigned), s) != cudaSuccess) {
         cudaGetLastError();

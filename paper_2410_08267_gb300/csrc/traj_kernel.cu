@@ -280,7 +280,7 @@ __device__ __forceinline__ void nfw_series2(double ta, double tb, int J_max, dou
     pb = p[1];
 }
 
-// Steps between two tests of the early exit (a power of two).
+// Steps between two tests of the early exit in the counting launch (a power of two).
 constexpr int kExitEvery = 4;
 
 // Added to r^2 in FP32 so that a trajectory through r = 0 exactly gets a
@@ -693,10 +693,10 @@ __device__ __forceinline__ f2 m_form(f2 r2, f2 S, float Yq0, float Yq1, f2 T, co
 // `rational` where this lane's last evaluation was on another branch.
 //
 // Two trajectories of a lane: the halves of every pair are theirs.
+template <bool OUTSIDE>                                // with kOutside steps
 struct TwoTrajectories {
-    static constexpr bool kOutsideSteps = true;
+    static constexpr bool kOutsideSteps = OUTSIDE;
     f2 x, y, vx, vy;
-    float y_least = 0.0f;                            // of selecting steps' last evaluations
     __device__ __forceinline__ void begin(const float4*) {}
     __device__ __forceinline__ TwoTrajectories(const float* x_, const float* y_, const float* vx_,
                                                const float* vy_)
@@ -718,6 +718,13 @@ struct TwoTrajectories {
         const f2 v2 = fma2(vx, vx, mul2(vy, vy));
         return (!act[0] || escapes(f2lo(r2), f2lo(dot), f2lo(v2), hc.R2, hc.R, irem)) &&
                (!act[1] || escapes(f2hi(r2), f2hi(dot), f2hi(v2), hc.R2, hc.R, irem));
+    }
+    // Whether both trajectories are out of the NFW part, to the rounding: r S >= c.
+    __device__ __forceinline__ bool outside(float S, const HaloX2& hc) const
+    {
+        const f2 r2 = fma2(x, x, mul2(y, y));
+        const float S2 = S * S, c2 = hc.c * hc.c;
+        return !(f2lo(r2) * S2 < c2) && !(f2hi(r2) * S2 < c2);
     }
     template <bool NARROW, StepForm FORM>
     __device__ __forceinline__ bool step(const float4* row, const float4*, const HaloX2& hc, bool& rational)
@@ -752,10 +759,8 @@ struct TwoTrajectories {
             const float a = fminf(fminf(f2lo(y1), f2hi(y1)), fminf(f2lo(y2), f2hi(y2)));
             const float b = fminf(fminf(f2lo(y3), f2hi(y3)), fminf(f2lo(y4), f2hi(y4)));
             if (__any_sync(0xffffffffu, fminf(a, b) < hc.c)) return false;
-            rational = false;
         } else {
             rational = rational && f2lo(y4) < q3.w && f2hi(y4) < q3.w;
-            y_least = fminf(y_least, fminf(f2lo(y4), f2hi(y4)));
         }
 
         const f2 W1 = dup(q2.x), W2 = dup(q2.y);
@@ -905,11 +910,13 @@ __device__ __forceinline__ void over_ring(float4* ring, const float4* tab, int s
 // it is done again in a form that lets each lane select its branch, and so are the
 // following steps: every kSelectEvery of them the warp stops if its lanes are all
 // finished, and goes back to kRational steps if they were all on that branch.  With two
-// trajectories a lane it goes on to kOutside steps, half the work, if they were all out
-// of the NFW part, until one fails: precision sweep 5.61 -> 5.47 ms, uneven batch 25.9 ->
-// 25.5, 614,000 trajectories from beyond R 0.45 -> 0.33 (0.36 in a kernel that skips the
-// force by branches).  One trajectory a lane is faster without (plain profile 97 us
-// against 104).
+// trajectories a lane it takes kOutside steps, half the work, while they are all out of
+// the NFW part: precision sweep 5.61 -> 5.37 ms, uneven batch 25.9 -> 25.2, 614,000
+// trajectories from beyond R 0.45 -> 0.31 (0.36 in a kernel that skips the force by
+// branches).  Where the chain of a step counts, the loop is faster without: one trajectory
+// a lane (plain profile 97 us against 104), and up to three CTAs of two on an SM
+// (kPackedFew: 12,000 to 38,000 trajectories 109 us against 120-125, 76,000 145-149 against
+// 155-164, 114,000 200-207 against 206-215; from four on there is no difference).
 // Evaluating the branches of such a warp by votes and warp-uniform paths took 1900
 // cycles a step on one scheduler, selecting takes 479 (412 one trajectory a lane).
 constexpr int kSelectEvery = 8;
@@ -922,7 +929,6 @@ __device__ __forceinline__ void step_loop(State& s, const float4* tab, int s_beg
     if (__all_sync(0xffffffffu, done)) return;
     bool rational = true;
     bool select = false;             // the warp runs steps that select
-    bool outside = false;            // ... of the kOutside form
     int k_select = 0;
     over_ring<kRow16>(ring, tab, s_begin, s_end, lane, [&](const float4* rows, int count) {
         const float4* const end = rows + count * kRow16;
@@ -939,7 +945,6 @@ __device__ __forceinline__ void step_loop(State& s, const float4* tab, int s_beg
                 select = true;
                 k_select = 0;
                 rational = false;
-                if constexpr (State::kOutsideSteps) s.y_least = 0.0f;
             }
             if ((k_select++ & (kSelectEvery - 1)) == 0) {
                 done |= s.finished(act, hc, rows[C_IREM / 4].w);
@@ -947,16 +952,19 @@ __device__ __forceinline__ void step_loop(State& s, const float4* tab, int s_beg
                 select = !__all_sync(0xffffffffu, rational);
                 rational = true;
                 if constexpr (State::kOutsideSteps) {
-                    outside = __all_sync(0xffffffffu, !(s.y_least < hc.c));
-                    s.y_least = INFINITY;
-                }
-            }
-            if constexpr (State::kOutsideSteps) {
-                if (outside) {
-                    outside = s.template step<NARROW, kOutside>(rows, next(), hc, rational);
-                    if (outside) {
-                        rows += kRow16;
-                        continue;
+                    if (__all_sync(0xffffffffu, s.outside(rows[C_S0 / 4].z, hc))) {
+                        int n = 0;
+                        while (n < kSelectEvery && rows < end &&
+                               s.template step<NARROW, kOutside>(rows, next(), hc, rational)) {
+                            rows += kRow16;
+                            ++n;
+                        }
+                        if (n == kSelectEvery || rows >= end) {
+                            select = true;
+                            rational = false;
+                            k_select = 0;
+                            continue;
+                        }
                     }
                 }
             }
@@ -1224,11 +1232,12 @@ __device__ __forceinline__ double sum_of_four(int n, int have, Load load)
 // consecutive trajectories of one radius and integrate them in passes of
 // blockDim.x * TPT.  The step loop:
 //   kLoopPacked  two trajectories per thread in packed FP32x2, 24 warps per SM (80
-//                registers, 5.61 ms on the precision sweep of four masses; before the
-//                coefficients were read ahead 5.75 ms, 5.95 with 64 registers, which
-//                spill, and 5.74 with 96 and 20 warps, but the uneven batch 27.5
-//                against 27.0 ms);
-//   kLoopPackedPasses  the same for tiles of more trajectories than a CTA holds
+//                registers, 5.37 ms on the precision sweep of four masses; 5.61 without
+//                kOutside steps; before that and the coefficients' being read ahead 5.75
+//                ms, 5.95 with 64 registers, which spill, and 5.74 with 96 and 20 warps,
+//                but the uneven batch 27.5 against 27.0 ms);
+//   kLoopPackedFew  the same without kOutside steps, for few CTAs on an SM (step_loop);
+//   kLoopPackedPasses  kLoopPacked for tiles of more trajectories than a CTA holds
 //                (whole_tiles);
 //   kLoopRing    one trajectory per thread, for small launches (plan_shape);
 //   kLoopRingMasses  the same with an epilogue that takes kMassGroup masses at a time,
@@ -1245,11 +1254,12 @@ __device__ __forceinline__ double sum_of_four(int n, int have, Load load)
 //                warps and 64 trajectories;
 //   kLoopGeneral one trajectory after another with the general force: the counting
 //                variant of either mode.
-enum StepLoop { kLoopGeneral, kLoopPacked, kLoopPackedPasses, kLoopRing, kLoopRingMasses, kLoopFp64,
-                kLoopFp64Split };
+enum StepLoop { kLoopGeneral, kLoopPacked, kLoopPackedFew, kLoopPackedPasses, kLoopRing, kLoopRingMasses,
+                kLoopFp64, kLoopFp64Split };
 constexpr int kRingThreads = 128;
 constexpr int kMassGroup = 4;
-template <StepLoop LOOP> constexpr bool kTwo = LOOP == kLoopPacked || LOOP == kLoopPackedPasses;
+template <StepLoop LOOP> constexpr bool kTwo =
+    LOOP == kLoopPacked || LOOP == kLoopPackedFew || LOOP == kLoopPackedPasses;
 
 __device__ __forceinline__ int warp_id() { return threadIdx.x >> 5; }
 
@@ -1388,7 +1398,8 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
                       done, hc, ring, lane, pair);
             if (warp >> 1) act[0] = false;               // counted once
         } else if constexpr (LOOP != kLoopGeneral) {
-            using State = typename std::conditional<kTwo<LOOP>, TwoTrajectories, OneTrajectory>::type;
+            using State = typename std::conditional<kTwo<LOOP>, TwoTrajectories<LOOP != kLoopPackedFew>,
+                                                    OneTrajectory>::type;
             static_assert(TPT == (kTwo<LOOP> ? 2 : 1), "trajectories of a lane");
             const HaloX2 h2{dup(hc.invIc), dup(-hc.invR3), hc.R2, hc.R, hc.c};
             const float4* tab4 = reinterpret_cast<const float4*>(tab);
@@ -1677,6 +1688,7 @@ int launch_force_probe(int precision, const DevProblem* d_prob, int stage, const
 constexpr int kFp64WarpsPerSm = 4;
 constexpr int kPackedTile = 256;
 constexpr int kPackedCtas = 6;                       // on an SM
+constexpr int kPackedFewCtas = 3;                    // on an SM: the loop without kOutside
 constexpr int kDevices = 32;                         // whose properties are kept
 
 int sm_count()
@@ -1707,7 +1719,8 @@ LaunchShape plan_shape(int precision, int tile, const LaunchSize& size)
         const long long w1 = (size.tiles128 + sms - 1) / sms, w2 = (size.tiles256 + sms - 1) / sms;
         const bool one = tile % kRingThreads == 0 && w2 <= kPackedCtas &&
                          std::max(440LL, 270 + 125 * w1) < std::max(500LL, 90 + 300 * w2);
-        s.kernel = !one ? kPacked : size.most_masses > 1 ? kRingMasses : kRing;
+        s.kernel = !one ? (w2 <= kPackedFewCtas ? kPackedFew : kPacked)
+                        : size.most_masses > 1 ? kRingMasses : kRing;
         for (int t : {one ? kRingThreads : kPackedTile, 128, 64})
             if (tile % t == 0) {
                 s.tile = t;
@@ -1753,6 +1766,7 @@ static TrajKernel kernel_of(int kernel)
     case kRingMasses: return traj_kernel<float, 1, false, kLoopRingMasses>;
     case kFp64: return traj_kernel<double, 1, false, kLoopFp64>;
     case kFp64Split: return traj_kernel<double, 1, false, kLoopFp64Split>;
+    case kPackedFew: return traj_kernel<float, 2, false, kLoopPackedFew>;
     case kPackedPasses: return traj_kernel<float, 2, false, kLoopPackedPasses>;
     case kCountF32: return traj_kernel<float, 2, true, kLoopGeneral>;
     default: return traj_kernel<double, 2, true, kLoopGeneral>;
@@ -1782,7 +1796,8 @@ int launch_traj_tally(int precision, const LaunchShape& shape, int grid, const D
                       const int* d_prefix, int n_probs, int n_tiles, unsigned* d_counter,
                       unsigned long long* d_tallies, void* stream)
 {
-    // the tallies are trajectory facts: every kernel integrates the same values
+    // the branches and needed steps are trajectory facts: every kernel integrates the same
+    // values.  The lane-steps run are this launch's own.
     const int threads = std::min((shape.tile + kUnit - 1) / kUnit * 32, 512);
     kernel_of(precision == NU_FP64 ? kCountF64 : kCountF32)
         <<<grid, threads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
