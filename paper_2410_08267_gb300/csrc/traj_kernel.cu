@@ -230,7 +230,7 @@ __device__ __forceinline__ double series_start(double t, int J, int J_max)
     float s = 0.0f;
 #pragma unroll
     for (int i = kSeriesTail / 4 - 1; i >= 0; --i) {
-        const float4 q = __ldg(c + i);
+                const float4 q = __ldg(c + i);
         s = fmaf(fmaf(fmaf(fmaf(s, tf, q.w), tf, q.z), tf, q.y), tf, q.x);
     }
     double p = widen_f32(s);
@@ -241,16 +241,15 @@ __device__ __forceinline__ double series_start(double t, int J, int J_max)
     return p;
 }
 
-// sums_{k=0}^{50} t^k/(k+2) of N values 0 < t < 1/2, their chains side by side.  J_max:
-// the most steps that a value of the warp needs (or more).
+// sums_{k=0}^{50} t^k/(k+2) of N values 0 < t < 1/2, their chains side by side.  J: the
+// steps that they need (series_steps); J_max: the most of the warp's, or more.
 template <int N>
-__device__ __forceinline__ void nfw_series_n(const double (&t)[N], int J_max, double (&p)[N])
+__device__ __forceinline__ void nfw_series_n(const double (&t)[N], const int (&J)[N], int J_max,
+                                             double (&p)[N])
 {
-    int J[N];
     double start[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-        J[i] = series_steps(t[i]);
         p[i] = start[i] = series_start(t[i], J[i], J_max);
     }
 #define NU_TERMS(K)                                                                      \
@@ -266,16 +265,17 @@ __device__ __forceinline__ void nfw_series_n(const double (&t)[N], int J_max, do
 #pragma unroll
     for (int i = 0; i < N; ++i) p[i] = series4<0>(series4<4>(p[i], t[i]), t[i]);
 }
-__device__ __forceinline__ double nfw_series(double t, int J_max)
+__device__ __forceinline__ double nfw_series(double t, int J, int J_max)
 {
     double p[1];
-    nfw_series_n<1>({t}, J_max, p);
+    nfw_series_n<1>({t}, {J}, J_max, p);
     return p[0];
 }
-__device__ __forceinline__ void nfw_series2(double ta, double tb, int J_max, double& pa, double& pb)
+__device__ __forceinline__ void nfw_series2(double ta, double tb, int Ja, int Jb, int J_max, double& pa,
+                                            double& pb)
 {
     double p[2];
-    nfw_series_n<2>({ta, tb}, J_max, p);
+    nfw_series_n<2>({ta, tb}, {Ja, Jb}, J_max, p);
     pa = p[0];
     pb = p[1];
 }
@@ -414,12 +414,13 @@ __device__ __forceinline__ double accel_m(double x, double y, double S, double Q
         t = quotient(ys, 1.0 + ys);
         series = less_nonneg(t, 0.5);
     }
-    int J_max = series ? series_steps(t) : 0;
+    const int J = series_steps(t);
+    int J_max = series ? J : 0;
     if (WARP) J_max = __reduce_max_sync(0xffffffffu, J_max);
     if (in) {
         if (nfw) {
             ctr.add(ys < 1.0 ? 2 : 3);
-            const double I = series ? (t * t) * nfw_series(t, J_max) : log1p(ys) - t;
+            const double I = series ? (t * t) * nfw_series(t, J, J_max) : log1p(ys) - t;
             sel = I * hc.invIc;
         } else {
             ctr.add(1);
@@ -986,6 +987,12 @@ __device__ __forceinline__ void step_loop(State& s, const float4* tab, int s_beg
 // evaluations of the pair that need the series are gathered into one pass over the
 // warp if they are 32 or fewer, and those that need the logarithm likewise.
 // ---------------------------------------------------------------------------
+// (A value's series length goes with it into a pass: found again there it would lengthen
+// the chain, 25.5 ms instead of 25.15 for six radii of the precision sweep.)
+struct PassBuffer {
+    double v[32];
+    int k[32];
+};
 struct Compact {                                     // a pair's evaluations that need a pass
     unsigned a, b, below;                            // their lanes; the lanes below this one
     __device__ __forceinline__ Compact(bool need_a, bool need_b, int lane)
@@ -997,27 +1004,34 @@ struct Compact {                                     // a pair's evaluations tha
     __device__ __forceinline__ bool one_pass() const { return a && b && count() <= 32; }
     __device__ __forceinline__ int slot_a() const { return __popc(a & below); }
     __device__ __forceinline__ int slot_b() const { return __popc(a) + __popc(b & below); }
-    // f of va where need_a and of vb where need_b, in one pass (one_pass())
+    // f(va, ka) where need_a and f(vb, kb) where need_b, in one pass (one_pass())
     template <class F>
-    __device__ __forceinline__ void pass(bool need_a, bool need_b, double& va, double& vb, double* buf,
-                                         int lane, F f) const
+    __device__ __forceinline__ void pass(bool need_a, bool need_b, double& va, double& vb, int ka, int kb,
+                                         PassBuffer& buf, int lane, F f) const
     {
-        if (need_a) buf[slot_a()] = va;
-        if (need_b) buf[slot_b()] = vb;
+        if (need_a) {
+            buf.v[slot_a()] = va;
+            buf.k[slot_a()] = ka;
+        }
+        if (need_b) {
+            buf.v[slot_b()] = vb;
+            buf.k[slot_b()] = kb;
+        }
         __syncwarp();
-        const double r = f(buf[lane < count() ? lane : 0]);
+        const int from = lane < count() ? lane : 0;
+        const double r = f(buf.v[from], buf.k[from]);
         __syncwarp();
-        buf[lane] = r;
+        buf.v[lane] = r;
         __syncwarp();
-        if (need_a) va = buf[slot_a()];
-        if (need_b) vb = buf[slot_b()];
+        if (need_a) va = buf.v[slot_a()];
+        if (need_b) vb = buf.v[slot_b()];
         __syncwarp();
     }
 };
 
 __device__ __forceinline__ void accel_pair(double xa, double ya, double Sa, double Qa, double xb,
                                            double yb, double Sb, double Qb, const HaloF64& hc,
-                                           double* buf, int lane, double& ma, double& mb)
+                                           PassBuffer& buf, int lane, double& ma, double& mb)
 {
     const unsigned full = 0xffffffffu;
     const double r2a = fma(xa, xa, ya * ya), r2b = fma(xb, xb, yb * yb);
@@ -1036,27 +1050,27 @@ __device__ __forceinline__ void accel_pair(double xa, double ya, double Sa, doub
         double Ia = ta, Ib = tb;
         const Compact cs(sa, sb, lane);
         if (cs.a | cs.b) {
-            const int J_max = __reduce_max_sync(full, max(sa ? series_steps(ta) : 0,
-                                                          sb ? series_steps(tb) : 0));
+            const int Ja = series_steps(ta), Jb = series_steps(tb);
+            const int J_max = __reduce_max_sync(full, max(sa ? Ja : 0, sb ? Jb : 0));
             if (cs.one_pass()) {
-                cs.pass(sa, sb, Ia, Ib, buf, lane,
-                        [&](double t) { return (t * t) * nfw_series(t, J_max); });
+                cs.pass(sa, sb, Ia, Ib, Ja, Jb, buf, lane,
+                        [&](double t, int J) { return (t * t) * nfw_series(t, J, J_max); });
             } else if (cs.a && cs.b) {
                 double pa, pb;
-                nfw_series2(ta, tb, J_max, pa, pb);
+                nfw_series2(ta, tb, Ja, Jb, J_max, pa, pb);
                 Ia = (ta * ta) * pa;
                 Ib = (tb * tb) * pb;
             } else if (cs.a) {
-                Ia = (ta * ta) * nfw_series(ta, J_max);
+                Ia = (ta * ta) * nfw_series(ta, Ja, J_max);
             } else {
-                Ib = (tb * tb) * nfw_series(tb, J_max);
+                Ib = (tb * tb) * nfw_series(tb, Jb, J_max);
             }
         }
         const Compact cl(la, lb, lane);
         if (cl.a | cl.b) {
             double ga = ysa, gb = ysb;
             if (cl.one_pass()) {
-                cl.pass(la, lb, ga, gb, buf, lane, [](double v) { return log1p(v); });
+                cl.pass(la, lb, ga, gb, 0, 0, buf, lane, [](double v, int) { return log1p(v); });
             } else {
                 if (cl.a) ga = log1p(ysa);
                 if (cl.b) gb = log1p(ysb);
@@ -1284,7 +1298,8 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
     constexpr int kMasses = LOOP == kLoopRingMasses ? kMassGroup : 1;   // of an epilogue's pass
     __shared__ double s_red[16][2 * kMasses];
     __shared__ double s_half[TPT == 1 ? (kMasses > 1 ? 2 : 8) : 1][2 * kMasses][32];
-    __shared__ double s_pass[LOOP == kLoopFp64 ? 8 : LOOP == kLoopFp64Split ? 8 : 1][32];
+    __shared__ double s_pair[LOOP == kLoopFp64Split ? 8 : 1][32];
+    __shared__ PassBuffer s_pass[LOOP == kLoopFp64 ? 8 : 1];
     // kRing16 words a warp (not kLoopGeneral).  From 16 bytes past a multiple of 32 on the
     // copies into it take longer, seen where little else is done: 614,000 trajectories
     // without a halo 111 us, 83 at 32 and 64 bytes, 76 at 128.
@@ -1393,7 +1408,7 @@ traj_kernel(const DevProblem* __restrict__ probs, const int* __restrict__ tile_p
                           accel_pair(xa, ya, Sa, Qa, xb, yb, Sb, Qb, hc, s_pass[warp], lane, ma, mb);
                       });
         } else if constexpr (kSplit) {
-            SplitPair pair{hc, s_pass[group * 4], 1 + group, warp >> 1, lane, 0};
+            SplitPair pair{hc, s_pair[group * 4], 1 + group, warp >> 1, lane, 0};
             fp64_loop(x[0], y[0], vx[0], vy[0], reinterpret_cast<const float4*>(tab), s_begin, s_end,
                       done, hc, ring, lane, pair);
             if (warp >> 1) act[0] = false;               // counted once
