@@ -1680,11 +1680,15 @@ int launch_force_probe(int precision, const DevProblem* d_prob, int stage, const
 //   Mixed precision: one trajectory a lane or two (packed), each in CTAs of four
 // warps, one for each scheduler of an SM.  As a CTA is one warp more on every scheduler of
 // its SM, a step of a launch that fits the chip takes the time of the SM with most CTAs:
-// with w of them, about max(440, 270 + 125 w) cycles one trajectory a lane and
-// max(500, 90 + 300 w) packed, fitted to launches of 4k to 307k trajectories (400 steps
-// over 8k / 51k / 76k / 102k / 153k / 204k / 307k: 96 / 132 / 174 / 211 / 255 / 309 / 424 us
-// and 109 / 143 / 146 / 202 / 260 / 353 / 411 us packed).  The cheaper one is taken; a
-// launch that fills the chip runs packed.
+// with w of them (more than four one a lane take turns), about max(440, 280 + 115 w)
+// cycles one trajectory a lane and max(540, 250 + 240 w) packed.  The cheaper one is taken.
+// Measured, one a lane / packed, us for 400 steps of the sweep's halo over
+//    12k    25k    38k    51k    65k    77k    92k   102k   116k   153k   184k   208k   233k
+//  90/109 102/111 104/110 125/143 153/150 160/151 166/204 174/202 197/205 248/258 293/305 321/355 346/357
+// trajectories.  At 97 to 116k packed is taken: one a lane is up to 20 % faster on many
+// halos, and up to 15 % slower on the heaviest.  From 233k on (more packed CTAs than fit
+// the chip) it is taken too: 250k 354/361, 271k 383/369, 307k 422/397, with one a lane 5 to
+// 30 % faster where most trajectories leave, and up to 12 % slower where none does.
 //   FP64: one trajectory a lane, in the smallest CTAs there are sums for, and of
 // those the fewest on an SM that give each scheduler a warp: one keeps its FP64
 // unit busy, and work not yet started can go to an SM that is done early.  Six radii of
@@ -1733,7 +1737,7 @@ LaunchShape plan_shape(int precision, int tile, const LaunchSize& size)
     } else {
         const long long w1 = (size.tiles128 + sms - 1) / sms, w2 = (size.tiles256 + sms - 1) / sms;
         const bool one = tile % kRingThreads == 0 && w2 <= kPackedCtas &&
-                         std::max(440LL, 270 + 125 * w1) < std::max(500LL, 90 + 300 * w2);
+                         std::max(440LL, 280 + 115 * w1) < std::max(540LL, 250 + 240 * w2);
         s.kernel = !one ? (w2 <= kPackedFewCtas ? kPackedFew : kPacked)
                         : size.most_masses > 1 ? kRingMasses : kRing;
         for (int t : {one ? kRingThreads : kPackedTile, 128, 64})

@@ -60,6 +60,17 @@ def test_fp64_launches_around_the_split(n_q, n_mu, n_radii, grid):
         assert np.array_equal(x, y)
 
 
+# Mixed launches of 1024 trajectories a radius: one a lane in tiles of 128 (up to 4 CTAs
+# on an SM) or two in tiles of 256 (6), by the most CTAs that an SM gets
+@pytest.mark.parametrize("n_radii,grid", [(19, 152), (25, 200), (38, 304), (39, 312), (57, 456), (58, 232),
+                                          (76, 304), (77, 608), (95, 608), (96, 384), (115, 608), (228, 608),
+                                          (229, 912)])
+def test_mixed_launches_around_the_rule(n_radii, grid):
+    pb = PLAIN.replace(n_steps=20, n_q=32, n_mu=32, radii=np.geomspace(1.0, 3000.0, n_radii))
+    for x, y in zip(*_normal_and_counting(pb, grid)):
+        assert np.array_equal(x, y)
+
+
 # FP64 CTAs on an SM: the fewest that give each of its four schedulers a warp
 @pytest.mark.parametrize("block,ctas", [(64, 2), (96, 2), (160, 1), (256, 2), (480, 1)])
 def test_fp64_ctas_of_a_large_launch(block, ctas):
