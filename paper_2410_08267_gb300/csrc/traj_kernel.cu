@@ -230,7 +230,7 @@ __device__ __forceinline__ double series_start(double t, int J, int J_max)
     float s = 0.0f;
 #pragma unroll
     for (int i = kSeriesTail / 4 - 1; i >= 0; --i) {
-                const float4 q = __ldg(c + i);
+        const float4 q = __ldg(c + i);
         s = fmaf(fmaf(fmaf(fmaf(s, tf, q.w), tf, q.z), tf, q.y), tf, q.x);
     }
     double p = widen_f32(s);

@@ -71,6 +71,34 @@ def test_mixed_launches_around_the_rule(n_radii, grid):
         assert np.array_equal(x, y)
 
 
+def test_fp64_results_do_not_depend_on_what_shares_the_launch():
+    """A request alone (its pairs of points split over two warps), beside others of other
+    series lengths, and the counting launch's: halos on both sides of y = 1 and beyond."""
+    def q_i(problems, count):
+        hs = [nu.create(pb, flags=nu.NU_FLAG_KEEP_QI) for pb in problems]
+        b = nu.nu_batch_create(hs)
+        try:
+            nu.nu_batch_run(b)
+            if count:
+                nu.nu_batch_branch_counts(b)
+            return [(nu.nu_profile_qi(h, pb.n_traj), *nu.nu_profile_result(h, pb.n_out))
+                    for h, pb in zip(hs, problems)]
+        finally:
+            nu.nu_batch_destroy(b)
+            for h in hs:
+                nu.nu_profile_destroy(h)
+
+    base = PLAIN.replace(precision=W.FP64, n_steps=60, n_q=37, n_mu=9)
+    small = [base.replace(radii=np.array([0.01, 3.0, 90.0]), c=c, M_h=M)
+             for c, M in ((0.9, 1e12), (4.0, 1e15), (10.0, 1e12), (40.0, 1e13))]
+    beside = base.replace(radii=np.geomspace(0.1, 3000.0, 60), c=6.0)
+    alone = [q_i([pb], False)[0] for pb in small]
+    for together in (q_i([beside] + small, False)[1:], q_i(small[::-1], True)[::-1]):
+        for one, other in zip(alone, together):
+            for x, y in zip(one, other):
+                assert np.array_equal(x, y)
+
+
 # FP64 CTAs on an SM: the fewest that give each of its four schedulers a warp
 @pytest.mark.parametrize("block,ctas", [(64, 2), (96, 2), (160, 1), (256, 2), (480, 1)])
 def test_fp64_ctas_of_a_large_launch(block, ctas):
